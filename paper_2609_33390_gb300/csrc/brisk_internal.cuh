@@ -237,9 +237,10 @@ __device__ __forceinline__ void fence_async_smem() {
 // into a CUDA graph keep launch attributes, but not the priority of the stream they were captured
 // from, so without it a replay of the tail's three-priority schedule runs every kernel at the
 // default priority.
+// With cluster > 1 the grid runs as clusters of that many CTAs.
 template <typename... KArgs, typename... Args>
-inline cudaError_t launch_prio(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem,
-                               cudaStream_t stream, Args&&... args) {
+inline cudaError_t launch_cluster(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem,
+                                  cudaStream_t stream, int cluster, Args&&... args) {
   int prio = 0;
   cudaError_t e = cudaStreamGetPriority(stream, &prio);
   if (e != cudaSuccess) return e;
@@ -248,12 +249,37 @@ inline cudaError_t launch_prio(void (*kernel)(KArgs...), dim3 grid, dim3 block, 
   cfg.blockDim = block;
   cfg.dynamicSmemBytes = smem;
   cfg.stream = stream;
-  cudaLaunchAttribute attr[1];
+  cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributePriority;
   attr[0].val.priority = prio;
+  attr[1].id = cudaLaunchAttributeClusterDimension;
+  attr[1].val.clusterDim.x = (unsigned)cluster;
+  attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
   cfg.attrs = attr;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = cluster > 1 ? 2 : 1;
   return cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...);
+}
+template <typename... KArgs, typename... Args>
+inline cudaError_t launch_prio(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem,
+                               cudaStream_t stream, Args&&... args) {
+  return launch_cluster(kernel, grid, block, smem, stream, 1, std::forward<Args>(args)...);
+}
+
+// Every thread of every CTA of the cluster arrives; writes before it are visible after it.
+__device__ __forceinline__ void cluster_sync() {
+  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" :::
+               "memory");
+}
+// 16 bytes at this CTA's shared address p, in the shared memory of CTA `rank` of the cluster.
+__device__ __forceinline__ float4 ld_cluster(const float* p, unsigned rank) {
+  uint32_t addr;
+  float4 v;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(addr) : "r"(su32(p)), "r"(rank));
+  asm volatile("ld.shared::cluster.v4.f32 {%0,%1,%2,%3}, [%4];"
+               : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
+               : "r"(addr)
+               : "memory");
+  return v;
 }
 
 __device__ __forceinline__ void set_status(int32_t* status, int code) {

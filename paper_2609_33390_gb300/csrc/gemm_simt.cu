@@ -1,103 +1,193 @@
-// Plain tiled fp32 dense products and a conversion copy. They serve the one-off
-// folding of the frozen vocabulary rows into the corrector tables
-// (App. C.3: E, E_out and the backbone are frozen at inference) and the fp32
-// configurations; every product accumulates in fp32.
+// Tiled fp32 dense products and a conversion copy. They serve the fp32 configurations (the
+// hidden products of a call and the one-off folds of the frozen vocabulary rows, App. C.3) and
+// the small folds of every configuration; every product accumulates in fp32.
 #include "brisk_internal.cuh"
 
 namespace brisk {
 
 namespace {
 
-constexpr int TM = 64, TN = 64, TK = 16;
+// One CTA computes a 128 x 64 tile of one product on 256 threads, 8 x 4 outputs a thread in
+// packed fp32 pairs, over 16-wide K slices double-buffered in shared memory (the next slice's
+// global loads are in flight while the present one is multiplied). Large products are bound by
+// the FMA pipes. A product with few tiles is bound by the K loop's latency instead (12 sequences
+// x 24 positions x 1000 by 96: 10 tiles, 145 us on 64 x 64 tiles over the whole K), so there a
+// cluster of up to 8 CTAs shares a tile: each takes a part of K, and each adds and stores its
+// share of the tile's rows from all parts, in part order, through distributed shared memory.
+constexpr int TM = 128, TN = 64, TK = 16;
+constexpr int SIMT_THREADS = 256;
+constexpr int SIMT_SPLIT_MAX = 8;
+constexpr int SIMT_FILL = 152;        // CTAs a split aims for: one an SM
+constexpr int SIMT_MIN_SLICES = 2;    // K slices a part has at least
+
+struct SimtProblem {
+  int M, N, K;
+  const void* A;
+  int lda;
+  const void* B;
+  int ldb;
+  int transB;
+  float* C;
+  int ldc;
+  int ntiles;        // tiles along N
+  int split;         // CTAs (one cluster) that share a tile, each a part of K
+  int vecA, vecB;    // rows may be read as 4-element vectors
+  const float* bias; // optional [bias_period, N], row m % bias_period added to row m
+  int bias_period;
+};
+
+// Elements k .. k + 3 of a row (zero past K).
+template <typename T>
+__device__ __forceinline__ float4 row4(const T* row, int k, int K, bool vec) {
+  if (vec && k + 3 < K) {
+    if constexpr (sizeof(T) == 4) {
+      return __ldg(reinterpret_cast<const float4*>(row + k));
+    } else {
+      const uint2 w = __ldg(reinterpret_cast<const uint2*>(row + k));
+      return make_float4(__uint_as_float(w.x << 16), __uint_as_float(w.x & 0xffff0000u),
+                         __uint_as_float(w.y << 16), __uint_as_float(w.y & 0xffff0000u));
+    }
+  }
+  float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+  if (k < K) v.x = to_f32(row[k]);
+  if (k + 1 < K) v.y = to_f32(row[k + 1]);
+  if (k + 2 < K) v.z = to_f32(row[k + 2]);
+  if (k + 3 < K) v.w = to_f32(row[k + 3]);
+  return v;
+}
+
+struct SimtSlices {
+  float a[2][TK][TM + 4];
+  float b[2][TK][TN + 4];
+};
+union SimtSmem {
+  SimtSlices s;
+  float part[TM][TN];   // this CTA's partial tile (split K)
+};
 
 template <typename TA, typename TB>
-__global__ void __launch_bounds__(256)
-gemm_simt_kernel(int M, int N, int K, const TA* __restrict__ A, int lda,
-                 const TB* __restrict__ B, int ldb, int transB, float* __restrict__ C, int ldc,
-                 const float* __restrict__ bias, int bias_period) {
-  __shared__ float As[TK][TM + 4];
-  __shared__ float Bs[TK][TN + 4];
-  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-  const long long m0 = (long long)blockIdx.y * TM, n0 = (long long)blockIdx.x * TN;
-  float acc[4][4];
+__global__ void __launch_bounds__(SIMT_THREADS)
+gemm_simt_kernel(const __grid_constant__ SimtProblem P) {
+  __shared__ __align__(16) SimtSmem sm;
+  const int tid = threadIdx.x;
+  const int split = P.split, tile = blockIdx.x / split, part = blockIdx.x - tile * split;
+  const int M = P.M, N = P.N, K = P.K;
+  const long long m0 = (long long)(tile / P.ntiles) * TM, n0 = (long long)(tile % P.ntiles) * TN;
+  const TA* A = static_cast<const TA*>(P.A);
+  const TB* B = static_cast<const TB*>(P.B);
+  const int slices = (K + TK - 1) / TK, per = (slices + split - 1) / split;
+  const int s0 = min(slices, part * per), s1 = min(slices, s0 + per);
+
+  // a thread loads k 4q .. 4q + 3 of rows r and r + 64 of A and of row r of B, q = tid % 4;
+  // with transB, columns 4c .. 4c + 3 of row kk of B
+  const int q = tid & 3, r = tid >> 2;
+  const int kk = tid >> 4, c = tid & 15;
+  const bool ra = m0 + r < M, rb = m0 + r + 64 < M, rn = n0 + r < N;
+  const TA* arow = A + (m0 + (ra ? r : 0)) * P.lda;
+  const TA* brow_a = A + (m0 + (rb ? r + 64 : 0)) * P.lda;
+  const TB* brow = B + (P.transB ? 0 : (n0 + (rn ? r : 0)) * P.ldb);
+  const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
+  float4 va, vb, vn;
+  auto load = [&](int s) {
+    const int k = s * TK + 4 * q;
+    va = ra ? row4(arow, k, K, P.vecA) : zero;
+    vb = rb ? row4(brow_a, k, K, P.vecA) : zero;
+    if (!P.transB) {
+      vn = rn ? row4(brow, k, K, P.vecB) : zero;
+    } else {
+      const int kt = s * TK + kk;
+      vn = kt < K ? row4(B + (long long)kt * P.ldb + n0, 4 * c, (int)min((long long)TN, N - n0), P.vecB)
+                  : zero;
+    }
+  };
+  auto store = [&](int buf) {
+    SimtSlices& z = sm.s;
+    z.a[buf][4 * q][r] = va.x; z.a[buf][4 * q + 1][r] = va.y;
+    z.a[buf][4 * q + 2][r] = va.z; z.a[buf][4 * q + 3][r] = va.w;
+    z.a[buf][4 * q][r + 64] = vb.x; z.a[buf][4 * q + 1][r + 64] = vb.y;
+    z.a[buf][4 * q + 2][r + 64] = vb.z; z.a[buf][4 * q + 3][r + 64] = vb.w;
+    if (!P.transB) {
+      z.b[buf][4 * q][r] = vn.x; z.b[buf][4 * q + 1][r] = vn.y;
+      z.b[buf][4 * q + 2][r] = vn.z; z.b[buf][4 * q + 3][r] = vn.w;
+    } else {
+      *reinterpret_cast<float4*>(&z.b[buf][kk][4 * c]) = vn;
+    }
+  };
+  // outputs: rows 8 ty .. 8 ty + 7 in pairs, columns 4 tx .. 4 tx + 3
+  const int tx = tid & 15, ty = tid >> 4;
+  float2 acc[4][4];
 #pragma unroll
   for (int i = 0; i < 4; ++i)
 #pragma unroll
-    for (int j = 0; j < 4; ++j) acc[i][j] = 0.f;
-  for (int k0 = 0; k0 < K; k0 += TK) {
-    for (int e = threadIdx.x; e < TM * TK; e += 256) {
-      const int mm = e / TK, kk = e % TK;
-      const long long gm = m0 + mm;
-      const int gk = k0 + kk;
-      As[kk][mm] = (gm < M && gk < K) ? to_f32(A[gm * lda + gk]) : 0.f;
-    }
-    for (int e = threadIdx.x; e < TN * TK; e += 256) {
-      int nn, kk;
-      if (transB) { kk = e / TN; nn = e % TN; } else { nn = e / TK; kk = e % TK; }
-      const long long gn = n0 + nn;
-      const int gk = k0 + kk;
-      float v = 0.f;
-      if (gn < N && gk < K) v = to_f32(transB ? B[(long long)gk * ldb + gn] : B[gn * ldb + gk]);
-      Bs[kk][nn] = v;
-    }
-    __syncthreads();
+    for (int j = 0; j < 4; ++j) acc[i][j] = make_float2(0.f, 0.f);
+  if (s0 < s1) {
+    load(s0);
+    store(0);
+  }
+  __syncthreads();
+  for (int s = s0; s < s1; ++s) {
+    const int buf = (s - s0) & 1;
+    if (s + 1 < s1) load(s + 1);
 #pragma unroll
-    for (int kk = 0; kk < TK; ++kk) {
-      float av[4], bv[4];
-#pragma unroll
-      for (int i = 0; i < 4; ++i) av[i] = As[kk][ty * 4 + i];
-#pragma unroll
-      for (int j = 0; j < 4; ++j) bv[j] = Bs[kk][tx * 4 + j];
+    for (int k = 0; k < TK; ++k) {
+      const float4 x0 = *reinterpret_cast<const float4*>(&sm.s.a[buf][k][8 * ty]);
+      const float4 x1 = *reinterpret_cast<const float4*>(&sm.s.a[buf][k][8 * ty + 4]);
+      const float4 y = *reinterpret_cast<const float4*>(&sm.s.b[buf][k][4 * tx]);
+      const float2 x[4] = {make_float2(x0.x, x0.y), make_float2(x0.z, x0.w),
+                           make_float2(x1.x, x1.y), make_float2(x1.z, x1.w)};
+      const float yv[4] = {y.x, y.y, y.z, y.w};
 #pragma unroll
       for (int i = 0; i < 4; ++i)
 #pragma unroll
-        for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(av[i], bv[j], acc[i][j]);
+        for (int j = 0; j < 4; ++j)
+          acc[i][j] = __ffma2_rn(x[i], make_float2(yv[j], yv[j]), acc[i][j]);
     }
+    if (s + 1 < s1) store(buf ^ 1);
     __syncthreads();
   }
+  auto bias = [&](long long m, long long n) {
+    return P.bias ? P.bias[(m % P.bias_period) * N + n] : 0.f;
+  };
+  if (split == 1) {
 #pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    const long long gm = m0 + ty * 4 + i;
-    if (gm >= M) continue;
+    for (int i = 0; i < 8; ++i) {
+      const long long gm = m0 + 8 * ty + i;
+      if (gm >= M) break;
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const long long gn = n0 + tx * 4 + j;
-      if (gn < N) C[gm * ldc + gn] = acc[i][j] + (bias ? bias[(gm % bias_period) * N + gn] : 0.f);
+      for (int j = 0; j < 4; ++j) {
+        const long long gn = n0 + 4 * tx + j;
+        if (gn < N)
+          P.C[gm * P.ldc + gn] = (i & 1 ? acc[i / 2][j].y : acc[i / 2][j].x) + bias(gm, gn);
+      }
     }
-  }
-}
-
-// Products with few rows (M <= SKINNY_MAX_M, B not transposed): a warp per output column n,
-// lane l accumulating k = l, l + 32, ... for every row, then one warp sum per row. One pass over
-// k with all loads in flight, where the tiled kernel would run a k-loop of K / 16 dependent
-// steps on a single CTA (an 8 x 64 product over k = 512: about 65 us in it, a few us here).
-constexpr int SKINNY_MAX_M = 16;
-constexpr int SKINNY_WARPS = 8;
-
-template <typename TA, typename TB>
-__global__ void __launch_bounds__(SKINNY_WARPS * 32)
-gemm_skinny_kernel(int M, int N, int K, const TA* __restrict__ A, int lda,
-                   const TB* __restrict__ B, int ldb, float* __restrict__ C, int ldc,
-                   const float* __restrict__ bias, int bias_period) {
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const long long n = (long long)blockIdx.x * SKINNY_WARPS + warp;
-  if (n >= N) return;
-  float acc[SKINNY_MAX_M];
-#pragma unroll
-  for (int m = 0; m < SKINNY_MAX_M; ++m) acc[m] = 0.f;
-  const TB* brow = B + n * ldb;
-  for (int k = lane; k < K; k += 32) {
-    const float b = to_f32(brow[k]);
-#pragma unroll
-    for (int m = 0; m < SKINNY_MAX_M; ++m)
-      if (m < M) acc[m] = fmaf(to_f32(A[(long long)m * lda + k]), b, acc[m]);
+    return;
   }
 #pragma unroll
-  for (int m = 0; m < SKINNY_MAX_M; ++m) {
-    if (m >= M) break;
-    const float v = warp_sum(acc[m]);
-    if (lane == 0) C[(long long)m * ldc + n] = v + (bias ? bias[(m % bias_period) * N + n] : 0.f);
+  for (int i = 0; i < 8; ++i) {
+    const float2* v = acc[i / 2];
+    *reinterpret_cast<float4*>(&sm.part[8 * ty + i][4 * tx]) =
+        i & 1 ? make_float4(v[0].y, v[1].y, v[2].y, v[3].y)
+              : make_float4(v[0].x, v[1].x, v[2].x, v[3].x);
   }
+  cluster_sync();
+  // this CTA's share of the tile's valid rows: the parts added in part order
+  const int rows = (int)min((long long)TM, M - m0);
+  const int share = (rows + split - 1) / split;
+  const int r0 = part * share, r1 = min(rows, r0 + share);
+  for (int e = r0 * 16 + tid; e < r1 * 16; e += SIMT_THREADS) {
+    const int row = e >> 4, col = 4 * (e & 15);
+    float4 v = ld_cluster(&sm.part[row][col], 0);
+    for (int o = 1; o < split; ++o) {
+      const float4 w = ld_cluster(&sm.part[row][col], o);
+      v.x += w.x; v.y += w.y; v.z += w.z; v.w += w.w;
+    }
+    const float x[4] = {v.x, v.y, v.z, v.w};
+    float* dst = P.C + (m0 + row) * P.ldc + n0 + col;
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+      if (n0 + col + j < N) dst[j] = x[j] + bias(m0 + row, n0 + col + j);
+  }
+  cluster_sync();   // the other CTAs have read this one's part
 }
 
 template <typename TS, typename TD>
@@ -117,18 +207,19 @@ template <typename TA, typename TB>
 cudaError_t gemm_t(int M, int N, int K, const void* A, int lda, const void* B, int ldb,
                    bool transB, float* C, int ldc, cudaStream_t stream, const float* bias,
                    int bias_period) {
-  if (M <= SKINNY_MAX_M && !transB) {
-    const unsigned grid = (unsigned)((N + SKINNY_WARPS - 1) / SKINNY_WARPS);
-    const cudaError_t e = launch_prio(
-        gemm_skinny_kernel<TA, TB>, dim3(grid), dim3(SKINNY_WARPS * 32), 0, stream, M, N, K,
-        static_cast<const TA*>(A), lda, static_cast<const TB*>(B), ldb, C, ldc, bias,
-        bias_period > 0 ? bias_period : 1);
-    return e != cudaSuccess ? e : cudaGetLastError();
-  }
-  const dim3 grid((N + TN - 1) / TN, (M + TM - 1) / TM);
-  const cudaError_t e = launch_prio(gemm_simt_kernel<TA, TB>, grid, dim3(256), 0, stream,
-      M, N, K, static_cast<const TA*>(A), lda, static_cast<const TB*>(B), ldb, transB ? 1 : 0, C, ldc,
-      bias, bias_period > 0 ? bias_period : 1);
+  const int ntiles = (N + TN - 1) / TN, slices = (K + TK - 1) / TK;
+  const long long tiles = (long long)((M + TM - 1) / TM) * ntiles;
+  int split = 1;
+  while (split < SIMT_SPLIT_MAX && 2 * split * tiles <= SIMT_FILL &&
+         slices >= 2 * split * SIMT_MIN_SLICES)
+    split *= 2;
+  auto vec = [](const void* p, size_t size, int ld) {
+    return reinterpret_cast<uintptr_t>(p) % (4 * size) == 0 && ld % 4 == 0;
+  };
+  const SimtProblem P{M, N, K, A, lda, B, ldb, transB ? 1 : 0, C, ldc, ntiles, split,
+                      vec(A, sizeof(TA), lda), vec(B, sizeof(TB), ldb), bias, bias_period};
+  const cudaError_t e = launch_cluster(gemm_simt_kernel<TA, TB>, dim3((unsigned)(tiles * split)),
+                                       dim3(SIMT_THREADS), 0, stream, split, P);
   return e != cudaSuccess ? e : cudaGetLastError();
 }
 
@@ -155,14 +246,15 @@ cudaError_t gemm_simt(int M, int N, int K, const void* A, int a_dt, int lda, con
   if (M <= 0 || N <= 0) return cudaSuccess;
   if (a_dt == BRISK_DT_BF16 && b_dt == BRISK_DT_BF16)
     return gemm_t<__nv_bfloat16, __nv_bfloat16>(M, N, K, A, lda, B, ldb, transB, C, ldc, stream,
-                                                 bias, bias_period);
+                                                bias, bias_period);
   if (a_dt == BRISK_DT_F32 && b_dt == BRISK_DT_BF16)
-    return gemm_t<float, __nv_bfloat16>(M, N, K, A, lda, B, ldb, transB, C, ldc, stream, bias,
-                                        bias_period);
+    return gemm_t<float, __nv_bfloat16>(M, N, K, A, lda, B, ldb, transB, C, ldc, stream,
+                                                bias, bias_period);
   if (a_dt == BRISK_DT_BF16 && b_dt == BRISK_DT_F32)
-    return gemm_t<__nv_bfloat16, float>(M, N, K, A, lda, B, ldb, transB, C, ldc, stream, bias,
-                                        bias_period);
-  return gemm_t<float, float>(M, N, K, A, lda, B, ldb, transB, C, ldc, stream, bias, bias_period);
+    return gemm_t<__nv_bfloat16, float>(M, N, K, A, lda, B, ldb, transB, C, ldc, stream,
+                                                bias, bias_period);
+  return gemm_t<float, float>(M, N, K, A, lda, B, ldb, transB, C, ldc, stream,
+                                                bias, bias_period);
 }
 
 cudaError_t copy2d(int rows, int cols, const void* src, int s_dt, int lds, void* dst, int d_dt,

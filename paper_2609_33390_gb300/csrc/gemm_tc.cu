@@ -124,6 +124,15 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, float (&v)[32]) {
   for (int j = 0; j < 32; ++j) v[j] = __uint_as_float(r[j]);
 }
 
+// Three bf16 parts of x, hi + mid + lo = x to about 2^-24 relative.
+__device__ __forceinline__ void split3(float x, __nv_bfloat16& hi, __nv_bfloat16& mid,
+                                       __nv_bfloat16& lo) {
+  hi = __float2bfloat16_rn(x);
+  const float r = x - __bfloat162float(hi);
+  mid = __float2bfloat16_rn(r);
+  lo = __float2bfloat16_rn(r - __bfloat162float(mid));
+}
+
 // Shared-memory matrix descriptor of a K-major tile stored as 8-row x 128-byte
 // swizzle atoms (the layout TMA writes with 128-byte swizzling): start address,
 // leading offset 16 B (unused by this layout), 1024 B between 8-row groups,
@@ -147,6 +156,8 @@ __host__ __device__ constexpr uint32_t idesc_bf16(int M, int N) {
 struct TcProblem {
   int M, N, K;
   int mode;         // 0: fp32 C[m*ldc + n]; 1: bf16 parts hi, mid, lo at [m*ldc + {0, N, 2N} + n]
+  void* C;
+  int ldc;
   int mtiles, ntiles;
   const float* bias;   // optional fp32 [bias_period, N], added to row m as bias[m % bias_period]
   int bias_period;
@@ -164,6 +175,7 @@ struct TcArgs {
   int tiles0;       // CTAs of problem 0
   int BN;           // tile columns (multiple of 16, <= 256), shared by both problems
   int tmem_cols;    // power of two >= max(32, BN)
+  int split;        // CTAs (one cluster) that share a tile, each a part of K
   long long wait_limit;   // SM cycles a pipeline or accumulator wait spins before it gives up
   int32_t* status;
 };
@@ -171,6 +183,14 @@ struct TcArgs {
 // Staging of one 32-column output chunk: fp32 (mode 0) or three bf16 parts (mode 1).
 constexpr int TC_OUT_CHUNK_F32 = TC_BM * 32 * 4;
 constexpr int TC_OUT_CHUNK_BF16X3 = 3 * TC_BM * 32 * 2;
+
+// Products with few tiles split K over a cluster: one CTA would walk the whole K alone (4096 in
+// 64 steps for the hidden states of one sequence) while most of the chip is idle.
+constexpr int TC_SPLIT_MAX = 8;
+constexpr int TC_SPLIT_BN = 64;                  // tile columns of a split product
+constexpr int TC_SPLIT_TILES = 76;               // tiles up to which K is split
+constexpr int TC_SPLIT_CTAS = 152;               // CTAs a split aims for: one an SM
+constexpr int TC_PART_LD = TC_SPLIT_BN + 4;      // row stride of a part in shared memory (floats)
 
 // SMALL_CARVEOUT does not change the code: it makes a separate kernel whose shared-memory
 // carveout preference (a per-kernel attribute) is the sweep's.
@@ -192,13 +212,17 @@ gemm_tc_kernel(const __grid_constant__ TcMaps maps, const __grid_constant__ TcAr
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int pi = (a.nprob > 1 && (int)blockIdx.x >= a.tiles0) ? 1 : 0;
+  const int t = (int)blockIdx.x / a.split, krank = (int)blockIdx.x - t * a.split;
+  const int pi = (a.nprob > 1 && t >= a.tiles0) ? 1 : 0;
   const TcProblem& P = a.p[pi];
   const CUtensorMap* tmA = &maps.a[pi];
   const CUtensorMap* tmB = &maps.b[pi];
-  const int tile = (int)blockIdx.x - (pi ? a.tiles0 : 0);
+  const int tile = t - (pi ? a.tiles0 : 0);
   const int m0 = (tile % P.mtiles) * TC_BM, n0 = (tile / P.mtiles) * a.BN;
-  const int nk = (P.K + TC_BK - 1) / TC_BK;
+  // this CTA's K steps [kfirst, kfirst + nk) (with split > 1 every part has at least one)
+  const int nk_all = (P.K + TC_BK - 1) / TC_BK;
+  const int kfirst = (int)((long long)nk_all * krank / a.split);
+  const int nk = (int)((long long)nk_all * (krank + 1) / a.split) - kfirst;
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < TC_STAGES; ++s) {
@@ -227,8 +251,8 @@ gemm_tc_kernel(const __grid_constant__ TcMaps maps, const __grid_constant__ TcAr
         break;
       }
       mbar_expect_tx(&full[s], a_bytes + b_bytes);
-      tma_load_2d(sA + s * a_bytes, tmA, &full[s], kb * TC_BK, m0);
-      tma_load_2d(sB + s * b_bytes, tmB, &full[s], kb * TC_BK, n0);
+      tma_load_2d(sA + s * a_bytes, tmA, &full[s], (kfirst + kb) * TC_BK, m0);
+      tma_load_2d(sB + s * b_bytes, tmB, &full[s], (kfirst + kb) * TC_BK, n0);
       issued = kb + 1;
     }
   } else if (warp == 1 && lane == 0) {
@@ -278,11 +302,62 @@ gemm_tc_kernel(const __grid_constant__ TcMaps maps, const __grid_constant__ TcAr
   const bool ok = !*abort_flag;
   if (!ok && threadIdx.x == 0) set_status(a.status, BRISK_ERR_TIMEOUT);
 
+  // Epilogue of a split product: the parts of a tile meet in distributed shared memory, where
+  // each CTA adds its share of the valid rows from all parts, in part order, and stores it.
+  if (a.split > 1) {
+    float* part = reinterpret_cast<float*>(base);    // the ring is free by then
+    if (ok) {
+      float* mine = part + (size_t)threadIdx.x * TC_PART_LD;
+      for (int c = 0; c < a.BN; c += 32) {
+        float v[32];
+        tmem_ld32(tmem + (static_cast<uint32_t>(warp * 32) << 16) + c, v);
+#pragma unroll
+        for (int q = 0; q < 8; ++q)
+          *reinterpret_cast<float4*>(mine + c + 4 * q) =
+              make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
+      }
+    }
+    cluster_sync();
+    if (ok) {
+      const int rows = min(TC_BM, P.M - m0), share = (rows + a.split - 1) / a.split;
+      const int r0 = krank * share, r1 = min(rows, r0 + share);
+      const int per_row = a.BN / 4;
+      for (int e = r0 * per_row + (int)threadIdx.x; e < r1 * per_row; e += TC_THREADS) {
+        const int row = e / per_row, col = 4 * (e - row * per_row);
+        if (n0 + col >= P.N) continue;               // N is a multiple of 16
+        const float* src = part + (size_t)row * TC_PART_LD + col;
+        float4 v = ld_cluster(src, 0);
+        for (int o = 1; o < a.split; ++o) {
+          const float4 w = ld_cluster(src, o);
+          v.x += w.x; v.y += w.y; v.z += w.z; v.w += w.w;
+        }
+        if (P.bias) {
+          const float* w = P.bias + (size_t)((m0 + row) % P.bias_period) * P.N + n0 + col;
+          v.x += w[0]; v.y += w[1]; v.z += w[2]; v.w += w[3];
+        }
+        const size_t at = (size_t)(m0 + row) * P.ldc + n0 + col;
+        if (P.mode == 0) {
+          *reinterpret_cast<float4*>(static_cast<float*>(P.C) + at) = v;
+        } else {
+          const float x[4] = {v.x, v.y, v.z, v.w};
+          __align__(8) __nv_bfloat16 q[3][4];
+#pragma unroll
+          for (int j = 0; j < 4; ++j) split3(x[j], q[0][j], q[1][j], q[2][j]);
+#pragma unroll
+          for (int h = 0; h < 3; ++h)
+            *reinterpret_cast<uint2*>(static_cast<__nv_bfloat16*>(P.C) + at + (size_t)h * P.N) =
+                *reinterpret_cast<const uint2*>(q[h]);
+        }
+      }
+    }
+    cluster_sync();   // the other CTAs have read this one's part
+  }
+
   // Epilogue. Warp w holds tile rows [32w, 32w + 32) in its TMEM lanes, one row a thread. A
   // finished 32-column chunk is staged in shared memory and written by TMA tensor stores
   // (which clip rows and columns outside the product); chunk c uses stage buffer c % nbuf, so
   // up to nbuf stores are in flight while the next chunks are staged.
-  if (ok) {
+  if (ok && a.split == 1) {
     const uint32_t trow = tmem + (static_cast<uint32_t>(warp * 32) << 16);
     const int rt = warp * 32 + lane;                 // row within the tile
     const int row = m0 + rt;
@@ -313,14 +388,10 @@ gemm_tc_kernel(const __grid_constant__ TcMaps maps, const __grid_constant__ TcAr
 #pragma unroll
         for (int q = 0; q < 8; ++q) st[q] = make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
       } else {
-        // three bf16 parts, hi + mid + lo = x to about 2^-24 relative
         __align__(16) __nv_bfloat16 hi[32], mid[32], lo[32];
 #pragma unroll
         for (int j = 0; j < 32; ++j) {
-          hi[j] = __float2bfloat16_rn(v[j]);
-          const float r1 = v[j] - __bfloat162float(hi[j]);
-          mid[j] = __float2bfloat16_rn(r1);
-          lo[j] = __float2bfloat16_rn(r1 - __bfloat162float(mid[j]));
+          split3(v[j], hi[j], mid[j], lo[j]);
         }
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
@@ -424,7 +495,25 @@ cudaError_t gemm_tc_grouped(const TcSpec* spec, int nprob, int32_t* status, cuda
   if (small_carveout && stages != 2) return cudaErrorInvalidValue;
   int nmax = 0;
   for (int i = 0; i < nprob; ++i) nmax = spec[i].N > nmax ? spec[i].N : nmax;
-  if (spec[0].max_bn >= 16 && nmax > spec[0].max_bn) nmax = spec[0].max_bn;
+  // Few tiles: split K. The rule looks at the products alone, so a product is summed in the same
+  // order whichever schedule it runs in.
+  int tiles = 0, nk = 0;
+  for (int i = 0; i < nprob; ++i) {
+    tiles += ((spec[i].M + TC_BM - 1) / TC_BM) * ((spec[i].N + TC_SPLIT_BN - 1) / TC_SPLIT_BN);
+    const int k = (spec[i].K + TC_BK - 1) / TC_BK;
+    nk = i == 0 || k < nk ? k : nk;
+  }
+  int split = 1;
+  while (tiles <= TC_SPLIT_TILES && split < TC_SPLIT_MAX && 2 * split * tiles <= TC_SPLIT_CTAS + 8 &&
+         nk >= 4 * split)
+    split *= 2;
+  int max_bn = spec[0].max_bn;
+  if (split > 1) {
+    max_bn = TC_SPLIT_BN;
+    stages = 4;
+    small_carveout = false;
+  }
+  if (max_bn >= 16 && nmax > max_bn) nmax = max_bn;
   const int BN = tc_bn(nmax);
   int cols = 32;
   while (cols < BN) cols *= 2;
@@ -433,6 +522,7 @@ cudaError_t gemm_tc_grouped(const TcSpec* spec, int nprob, int32_t* status, cuda
   a.nprob = nprob;
   a.BN = BN;
   a.tmem_cols = cols;
+  a.split = split;
   a.wait_limit = wait_limit_cycles();
   a.status = status;
   int total = 0;
@@ -452,7 +542,7 @@ cudaError_t gemm_tc_grouped(const TcSpec* spec, int nprob, int32_t* status, cuda
     }
     if (i >= nprob) continue;
     TcProblem& P = a.p[i];
-    P.M = q.M; P.N = q.N; P.K = q.K; P.mode = q.mode;
+    P.M = q.M; P.N = q.N; P.K = q.K; P.mode = q.mode; P.C = q.C; P.ldc = q.ldc;
     P.bias = q.bias;
     P.bias_period = q.bias_period > 0 ? q.bias_period : 1;
     P.mtiles = (q.M + TC_BM - 1) / TC_BM;
@@ -469,7 +559,7 @@ cudaError_t gemm_tc_grouped(const TcSpec* spec, int nprob, int32_t* status, cuda
                                        static_cast<int>(smem));
   if (e == cudaSuccess) e = prefer_carveout(kernel, small_carveout ? CARVEOUT_SMALL_KB : CARVEOUT_GEMM_KB);
   if (e != cudaSuccess) return e;
-  e = launch_prio(kernel, dim3(total), dim3(TC_THREADS), smem, stream, maps, a);
+  e = launch_cluster(kernel, dim3(total * split), dim3(TC_THREADS), smem, stream, split, maps, a);
   if (e != cudaSuccess) return e;
   return cudaGetLastError();
 }
