@@ -35,12 +35,13 @@ enum TailSchedule { SCHEDULE_OVERLAP = 0, SCHEDULE_SEPARATE = 1, SCHEDULE_FUSED 
 // (direct calls / graph replays): one sequence (16 MB) 124.9 / 106.4 us separate, 117.7 / 102.5
 // us fused; 16 sequences (259 MB, stochastic) 188.9 / 175.2 us separate, 243.6 / 210.6 fused.
 constexpr size_t FUSE_MAX_BYTES = size_t(64) << 20;
+constexpr size_t OVERLAP_ROWS = 2432;      // proposal rows from which the sweeps overlap
+constexpr size_t OVERLAP_VECTORS = 2048;   // 16-byte vectors a row below which they do
 
 struct WsLayout {
   size_t status, counters, part_val, part_id, part_m, part_s, argmax_p, lse_p;
   size_t cand_ids, cand_logprob, lse_q, sel, refined, Hm, G, G0, distill, base_rank, total;
-  int nchunk_q, nchunk_p, KP;   // chunks per proposal row (row layout) and verifier row
-  int mode_p;                   // layout of the verifier rows' sweep (SweepMode)
+  int nsplit, KP;               // segments per row of either tensor
   int schedule;                 // TailSchedule of brisk_decode_tail
 };
 
@@ -48,24 +49,18 @@ WsLayout ws_layout(const brisk_dims* d) {
   WsLayout w{};
   const size_t BL = (size_t)d->B * d->L;
   const size_t S = 2 * (size_t)d->r;
-  w.nchunk_q = sweep_chunks((int)BL, d->V, d->logits_dtype, SWEEP_ROWS);
-  // Schedule of the fused tail and the verifier rows' layout (every entry point sweeps the
-  // verifier rows the same way, so that the fused and separate calls give the same bits):
-  //  OVERLAP  one task per proposal row: verifier rows in the split layout, beside the corrector;
-  //  FUSED    chunked proposal rows and both logit tensors within FUSE_MAX_BYTES: verifier rows
-  //           in the row layout with the proposal rows' chunks, both tensors in one launch;
-  //  SEPARATE chunked proposal rows, larger tensors: verifier rows in the split layout, beside
-  //           the corrector (the verifier sweep then takes long enough that overlapping it with
-  //           the corrector beats one launch before it).
-  const size_t sweep_bytes = 2 * BL * (size_t)d->V * esize(d->logits_dtype);
-  if (w.nchunk_q == 1) w.schedule = SCHEDULE_OVERLAP;
-  else w.schedule = sweep_bytes <= FUSE_MAX_BYTES ? SCHEDULE_FUSED : SCHEDULE_SEPARATE;
-  w.mode_p = w.schedule == SCHEDULE_FUSED ? SWEEP_ROWS : SWEEP_SPLIT;
-  w.nchunk_p = w.schedule == SCHEDULE_FUSED
-                   ? w.nchunk_q
-                   : sweep_chunks((int)BL, d->V, d->logits_dtype, SWEEP_SPLIT);
+  w.nsplit = sweep_splits((int)BL, d->V, d->logits_dtype, d->K);
+  // Schedule of the fused tail (every entry point sweeps a row the same way, so fused and separate
+  // calls give the same bits):
+  //  OVERLAP  many rows, or rows of few vectors: the verifier rows' sweep from the start, on the
+  //           lowest priority;
+  //  FUSED    few rows and both logit tensors within FUSE_MAX_BYTES: both in one sweep launch;
+  //  SEPARATE otherwise: the verifier rows' sweep after the proposal rows', beside the corrector.
+  const size_t row_bytes = (size_t)d->V * esize(d->logits_dtype);
+  if (BL >= OVERLAP_ROWS || row_bytes / 16 < OVERLAP_VECTORS) w.schedule = SCHEDULE_OVERLAP;
+  else w.schedule = 2 * BL * row_bytes <= FUSE_MAX_BYTES ? SCHEDULE_FUSED : SCHEDULE_SEPARATE;
   w.KP = kp_for(d->K);
-  const size_t np = BL * (size_t)(w.nchunk_q + w.nchunk_p);
+  const size_t np = 2 * BL * (size_t)w.nsplit;
   size_t o = 0;
   auto take = [&](size_t bytes) { const size_t r = o; o = up(o + bytes); return r; };
   w.status = take(ALIGN);
@@ -161,7 +156,7 @@ brisk_status clear_ws(const WsLayout& w, const brisk_dims* d, void* ws, cudaStre
 SweepSeg make_seg(const WsLayout& w, void* ws, int seg, const void* logits, int rows, int kout,
                   int32_t* out_ids, float* out_logprob, float* out_lse) {
   SweepSeg s{};
-  const size_t off = seg ? (size_t)rows * w.nchunk_q : 0;   // segment 1 follows segment 0
+  const size_t off = seg ? (size_t)rows * w.nsplit : 0;   // segment 1 follows segment 0
   s.logits = logits;
   s.rows = rows;
   s.kout = kout;
@@ -439,8 +434,7 @@ brisk_status brisk_topk_candidates(const brisk_dims* d, const void* logits_q, in
   a.seg[0] = make_seg(w, ws, 0, logits_q, d->B * d->L, d->K, cand_ids, cand_logprob, lse_q);
   a.nseg = 1;
   a.V = d->V;
-  a.mode = SWEEP_ROWS;
-  a.nchunk = w.nchunk_q;
+  a.nsplit = w.nsplit;
   a.KP = w.KP;
   a.dtype = d->logits_dtype;
   a.status = at<int32_t>(ws, w.status);
@@ -505,8 +499,7 @@ brisk_status brisk_verify_block(const brisk_dims* d, const void* logits_p, const
                        at<float>(ws, w.lse_p));
   sw.nseg = 1;
   sw.V = d->V;
-  sw.mode = w.mode_p;
-  sw.nchunk = w.nchunk_p;
+  sw.nsplit = w.nsplit;
   sw.KP = w.KP;
   sw.dtype = d->logits_dtype;
   sw.status = at<int32_t>(ws, w.status);
@@ -602,16 +595,13 @@ brisk_status brisk::decode_tail_locked(const brisk_dims* d, const brisk_params* 
   sq.seg[0] = make_seg(w, ws, 0, io->logits_q, BL, d->K, cand_ids, cand_lp, lse_q);
   sq.nseg = 1;
   sq.V = d->V;
-  sq.mode = SWEEP_ROWS;
-  sq.nchunk = w.nchunk_q;
+  sq.nsplit = w.nsplit;
   sq.KP = w.KP;
   sq.dtype = d->logits_dtype;
   sq.status = at<int32_t>(ws, w.status);
   SweepLaunch sp = sq;
   sp.seg[0] = make_seg(w, ws, 1, io->logits_p, BL, 1, at<int32_t>(ws, w.argmax_p), nullptr,
                        at<float>(ws, w.lse_p));
-  sp.mode = w.mode_p;
-  sp.nchunk = w.nchunk_p;
   ScanArgs a = scan_args(d, p, tables, w, ws);
   a.select_mode = select_mode;
   a.verify_mode = verify_mode;
@@ -776,8 +766,7 @@ brisk_status brisk_replay_diagnostics(const brisk_dims* d, const brisk_params* p
   sq.seg[0] = make_seg(w, ws, 0, logits_q, BL, d->K, cand_ids, cand_lp, at<float>(ws, w.lse_q));
   sq.nseg = 1;
   sq.V = d->V;
-  sq.mode = SWEEP_ROWS;
-  sq.nchunk = w.nchunk_q;
+  sq.nsplit = w.nsplit;
   sq.KP = w.KP;
   sq.dtype = d->logits_dtype;
   sq.status = at<int32_t>(ws, w.status);
@@ -785,8 +774,6 @@ brisk_status brisk_replay_diagnostics(const brisk_dims* d, const brisk_params* p
   SweepLaunch sp = sq;
   sp.seg[0] = make_seg(w, ws, 1, logits_p, BL, 1, at<int32_t>(ws, w.argmax_p), nullptr,
                        at<float>(ws, w.lse_p));
-  sp.mode = w.mode_p;
-  sp.nchunk = w.nchunk_p;
   BRISK_CUDA(launch_sweep(sp, st));
   // the head along the factual base prefix
   s = hidden_products(d, p, tables, hidden, h_ctx, w, ws, st, false);

@@ -296,33 +296,30 @@ struct SweepSeg {
   int32_t* out_ids;       // [rows, kout]
   float* out_logprob;     // [rows, kout] or nullptr
   float* out_lse;         // [rows]
-  float* part_val;        // [rows, nchunk, KP]
-  int32_t* part_id;       // [rows, nchunk, KP]
-  float* part_m;          // [rows, nchunk]
-  float* part_s;          // [rows, nchunk]
+  float* part_val;        // [rows, nsplit, KP]
+  int32_t* part_id;       // [rows, nsplit, KP]
+  float* part_m;          // [rows, nsplit]
+  float* part_s;          // [rows, nsplit]
   int32_t* counters;      // [rows]
 };
-
-// Work layouts of the sweep: each warp its own (row, chunk), or each CTA one (row, split).
-enum SweepMode { SWEEP_ROWS = 0, SWEEP_SPLIT = 1 };
 
 struct SweepLaunch {
   SweepSeg seg[2];
   int nseg;
   int V;
-  int mode;               // SweepMode
-  int nchunk;             // chunks per row (a multiple of 4 for SWEEP_SPLIT)
+  int nsplit;             // segments (CTAs) per row
   int KP;
   int dtype;              // brisk_dtype of the logits
   int32_t* status;
 };
 
-int sweep_chunks(int rows_per_tensor, int V, int dtype, int mode);
+int sweep_splits(int rows_per_tensor, int V, int dtype, int K);
 int kp_for(int K);
 cudaError_t launch_sweep(const SweepLaunch& a, cudaStream_t stream);
 
 // ---------------------------------------------------------------- dense products (SIMT, fp32 accumulate)
-// C[m, n] = sum_k A(m, k) B(n, k), A(m,k) = A[m*lda + k], B(n,k) = transB ? B[k*ldb + n] : B[n*ldb + k].
+// C[m, n] = sum_k A(m, k) B(n, k) (+ bias[m % bias_period][n]), A(m,k) = A[m*lda + k],
+// B(n,k) = transB ? B[k*ldb + n] : B[n*ldb + k].
 cudaError_t gemm_simt(int M, int N, int K, const void* A, int a_dt, int lda, const void* B,
                       int b_dt, int ldb, bool transB, float* C, int ldc, cudaStream_t stream,
                       const float* bias = nullptr, int bias_period = 1);

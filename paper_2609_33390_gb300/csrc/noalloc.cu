@@ -6,7 +6,7 @@
 // manager has already reserved all of HBM and forbids ad-hoc cudaMalloc, or
 // a host that must not allocate on its decode path at all. For them this
 // entry point runs the same sweep kernel with its scratch (per-row arrival
-// counters and per-chunk partial results) in a fixed array that lives in the
+// counters and per-segment partial results) in a fixed array that lives in the
 // library itself, so nothing is allocated at call time.
 #include <mutex>
 
@@ -58,11 +58,11 @@ extern "C" brisk_status brisk_topk_candidates_noalloc(const brisk_dims* d, const
   if (!logits_q || !cand_ids || !cand_logprob || !lse_q ||
       reinterpret_cast<uintptr_t>(logits_q) % es != 0)
     return BRISK_ERR_INVALID_ARG;
-  // scratch layout: status word, arrival counters, per-chunk partial results
+  // scratch layout: status word, arrival counters, per-segment partial results
   const int rows = d->B * d->L;
-  const int nchunk = sweep_chunks(rows, d->V, d->logits_dtype, SWEEP_ROWS);
+  const int nsplit = sweep_splits(rows, d->V, d->logits_dtype, d->K);
   const int KP = kp_for(d->K);
-  const size_t np = (size_t)rows * nchunk;
+  const size_t np = (size_t)rows * nsplit;
   const size_t o_cnt = 256;
   const size_t o_val = o_cnt + up256(sizeof(int32_t) * rows);
   const size_t o_id = o_val + up256(sizeof(float) * np * KP);
@@ -92,8 +92,7 @@ extern "C" brisk_status brisk_topk_candidates_noalloc(const brisk_dims* d, const
   s.part_s = reinterpret_cast<float*>(scratch + o_s);
   a.nseg = 1;
   a.V = d->V;
-  a.mode = SWEEP_ROWS;
-  a.nchunk = nchunk;
+  a.nsplit = nsplit;
   a.KP = KP;
   a.dtype = d->logits_dtype;
   a.status = reinterpret_cast<int32_t*>(scratch);
