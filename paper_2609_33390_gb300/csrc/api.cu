@@ -203,7 +203,7 @@ brisk_status hidden_products(const brisk_dims* d, const brisk_params* p, const v
     BRISK_CUDA(gemm_tc_grouped(first, 2, status, st, wide ? 2 : 4, share));
     const TcSpec second[2] = {
         {BL, 2 * S, r3, Hs, r3, at<__nv_bfloat16>(tables, t.W2s), r3, 0, at<float>(ws, w.G), 2 * S,
-         nullptr, 0, share ? 64 : 0},
+         at<float>(tables, t.posG), d->L, share ? 64 : 0},
         {d->B, S, r3, Hs + (size_t)BL * r3, r3, at<__nv_bfloat16>(tables, t.W0s), r3, 0,
          at<float>(ws, w.G0), S, nullptr, 0, share ? 64 : 0}};
     BRISK_CUDA(gemm_tc_grouped(second, 2, status, st, 2, share));
@@ -214,7 +214,7 @@ brisk_status hidden_products(const brisk_dims* d, const brisk_params* p, const v
   BRISK_CUDA(gemm_simt(d->B, r, d->d, h_ctx, hd, d->d, p->P_h, hd, d->d, false,
                        Hm + (size_t)BL * r, r, st));
   BRISK_CUDA(gemm_simt(BL, 2 * S, r, Hm, BRISK_DT_F32, r, at<float>(tables, t.W2), BRISK_DT_F32, r,
-                       false, at<float>(ws, w.G), 2 * S, st));
+                       false, at<float>(ws, w.G), 2 * S, st, at<float>(tables, t.posG), d->L));
   BRISK_CUDA(gemm_simt(d->B, S, r, Hm + (size_t)BL * r, BRISK_DT_F32, r, at<float>(tables, t.W0h),
                        BRISK_DT_F32, r, false, at<float>(ws, w.G0), S, st));
   return BRISK_OK;
@@ -271,7 +271,6 @@ ScanArgs scan_args(const brisk_dims* d, const brisk_params* p, const void* table
   if (tables) {
     const TbLayout t = tb_layout(d);
     a.Tzh = at<float>(tables, t.Tzh);
-    a.posG = at<float>(tables, t.posG);
     a.U = at<float>(tables, t.U);
     a.T0 = at<float>(tables, t.T0);
     a.Fz = at<float>(tables, t.Fz);
@@ -614,6 +613,7 @@ brisk_status brisk::decode_tail_locked(const brisk_dims* d, const brisk_params* 
   a.u_sel = io->u_sel;
   a.sel_tokens = sel;
   a.refined = refined;
+  a.beside_sweep = w.schedule == SCHEDULE_OVERLAP;
 
   if (w.schedule == SCHEDULE_FUSED) {
     // both tensors' rows in one launch (the same layout and chunks as the separate calls)

@@ -367,8 +367,7 @@ struct ScanArgs {
   const float* cand_logprob;
   const int32_t* x0;
   const float* u_sel;
-  const float* G;        // [B*L, 2S] hidden shares of the GRU pre-activations (z | h)
-  const float* posG;     // [L, 2S]   position shares of the GRU pre-activations (z | h)
+  const float* G;        // [B*L, 2S] hidden and position shares of the GRU pre-activations (z | h)
   const float* G0;       // [B, S]    hidden-state part of Init
   const float* Tzh;      // [V, 2S]   token part of the GRU pre-activations (z | h)
   const float* U;        // [V, S]    residual rows: d = <s, U[c]>
@@ -382,6 +381,10 @@ struct ScanArgs {
   // record its rank
   int base_prefix;
   int32_t* base_rank;    // [B, L] (base_prefix only)
+  int beside_sweep;      // the corrector runs beside the verifier-row sweep
+  // set by the launch (see corrector_kernel)
+  int groups, ring_depth, tok_ranks, ask_rows, ask_tokens;
+  long long wait_limit;
   // select outputs (or verify inputs when do_select == 0)
   int32_t* sel_tokens;   // [B, L]
   float* refined;        // [B, L, K]

@@ -67,99 +67,32 @@ __host__ __device__ inline size_t smem_layout(int L, int K, int S, int V, char* 
 
 __device__ __forceinline__ float4 ld4(const float* p) { return *reinterpret_cast<const float4*>(p); }
 
-// A lane's chunk of CW consecutive state elements (CW = 1, 2 or 4), loaded as one vector;
-// CG: cached in L2 only (rows read once per step must not displace the L1 lines that hold a
-// concurrent streaming kernel's loads in flight).
-template <int CW>
-struct Chunk {
-  float v[CW];
-};
-template <int CW>
-__device__ __forceinline__ Chunk<CW> chunk_of(const float4& t) {
-  if constexpr (CW == 4) return {{t.x, t.y, t.z, t.w}};
-  else return {{t.x, t.y}};
-}
-template <int CW, bool CG>
-__device__ __forceinline__ Chunk<CW> ldc(const float* p) {
-  if constexpr (CW == 4) {
-    return chunk_of<4>(CG ? __ldcg(reinterpret_cast<const float4*>(p))
-                          : *reinterpret_cast<const float4*>(p));
-  } else if constexpr (CW == 2) {
-    const float2 t = CG ? __ldcg(reinterpret_cast<const float2*>(p))
-                        : *reinterpret_cast<const float2*>(p);
-    return {{t.x, t.y}};
-  } else {
-    return {{CG ? __ldcg(p) : *p}};
-  }
-}
-template <int CW>
-__device__ __forceinline__ Chunk<CW> addc(const Chunk<CW>& x, const Chunk<CW>& y) {
-  Chunk<CW> r;
-#pragma unroll
-  for (int e = 0; e < CW; ++e) r.v[e] = x.v[e] + y.v[e];
-  return r;
-}
-// acc + sum_e x_e y_e, the last element first (the order of the four-element form)
-template <int CW>
-__device__ __forceinline__ float dotc(const Chunk<CW>& x, const Chunk<CW>& y, float acc) {
-#pragma unroll
-  for (int e = CW - 1; e >= 0; --e) acc = fmaf(x.v[e], y.v[e], acc);
-  return acc;
-}
-// Logistic function with the hardware exponential (relative error ~1e-6).
-__device__ __forceinline__ float sigmoid_fast(float x) { return __fdividef(1.f, 1.f + __expf(-x)); }
-
-// Warp reduce-scatter of NP values per lane: afterwards lane l holds the warp-wide sum of value
-// ((l >> 1) & 15) for NP = 16 and of value l for NP = 32.
-template <int NP>
-__device__ __forceinline__ float reduce_scatter(float (&v)[NP]) {
-  const int lane = threadIdx.x & 31;
-#pragma unroll
-  for (int m = 16, n = NP; n > 1; m >>= 1, n >>= 1) {
-    const bool upper = (lane & m) != 0;
-#pragma unroll
-    for (int j = 0; j < n / 2; ++j) {
-      const float send = upper ? v[j] : v[j + n / 2];
-      const float keep = upper ? v[j + n / 2] : v[j];
-      v[j] = keep + __shfl_xor_sync(FULL_MASK, send, m);
-    }
-  }
-  float r = v[0];
-  if (NP == 16) r += __shfl_xor_sync(FULL_MASK, r, 1);
-  return r;
-}
-
 __device__ __forceinline__ float load_logit(const void* base, int dt, size_t idx) {
   if (dt == BRISK_DT_BF16) return __bfloat162float(reinterpret_cast<const __nv_bfloat16*>(base)[idx]);
   return reinterpret_cast<const float*>(base)[idx];
 }
 
-// Order-preserving map of a float (not NaN) to an unsigned key; -0 and +0 map alike.
-__device__ __forceinline__ unsigned ordered_key(float f) {
-  const unsigned u = __float_as_uint(f + 0.f);
-  return (u & 0x80000000u) ? ~u : (u | 0x80000000u);
-}
-__device__ __forceinline__ float key_value(unsigned k) {
-  return __uint_as_float((k & 0x80000000u) ? (k & 0x7fffffffu) : ~k);
+// Largest of one float per lane, none of them NaN (one warp reduction).
+__device__ __forceinline__ float redux_max(float x) {
+  float r;
+  asm volatile("redux.sync.max.f32 %0, %1, 0xffffffff;" : "=f"(r) : "f"(x));
+  return r;
 }
 
 // Select with lane k holding refined score k (lanes >= K hold -inf); the same in every lane.
 // Greedy: argmax, the lowest rank on ties. Sample: the first rank whose cumulative softmax mass
-// exceeds u * total (warp prefix sums), else the last rank with mass. The maxima are single
-// warp reductions of the scores' order-preserving keys (five shuffle rounds before: single
-// 102 -> 100 us, large_vocab 246 -> 241 us for the products and the corrector).
+// exceeds u * total (warp prefix sums), else the last rank with mass.
 __device__ __forceinline__ int select_warp(float ref, int K, int mode, float u) {
   const int lane = threadIdx.x & 31;
   if (mode == BRISK_SELECT_GREEDY) {
     // a NaN score ranks as -inf, so every lane agrees on one rank in [0, K) whatever the
-    // scores hold: the lowest rank holding the warp's largest key (one warp reduction)
+    // scores hold: the lowest rank holding the warp's largest score
     const float bv = (lane < K && !isnan(ref)) ? ref : -INFINITY;
-    const unsigned key = ordered_key(bv);
-    const unsigned mk = __reduce_max_sync(FULL_MASK, key);
-    const unsigned hit = __ballot_sync(FULL_MASK, lane < K && key == mk);
+    const float mx = redux_max(bv);   // (by the whole warp)
+    const unsigned hit = __ballot_sync(FULL_MASK, lane < K && bv == mx);
     return hit ? __ffs(hit) - 1 : 0;
   }
-  const float mx = key_value(__reduce_max_sync(FULL_MASK, ordered_key(isnan(ref) ? -INFINITY : ref)));
+  const float mx = redux_max(isnan(ref) ? -INFINITY : ref);
   const float w = lane < K ? expf(ref - mx) : 0.f;
   float cum = w;
 #pragma unroll
@@ -446,41 +379,56 @@ verify_kernel(const __grid_constant__ ScanArgs a) {
 }
 
 // ---------------------------------------------------------------- corrector
-constexpr int CORR_WARPS = 4;   // warps per sequence: one per SM sub-partition
+constexpr int CORR_SPAN = 128;   // state elements a computing warp owns, 4 a lane
+constexpr int CORR_PART = 8;     // slots for the dots' parts: S <= 1024, so at most 8 warps
+constexpr int CORR_DEPTH = 4;    // positions the ring holds at most
+constexpr int CORR_AHEAD = 4;    // positions whose table rows are asked into L2 ahead of use
+constexpr int CORR_OTHERS = 64;  // threads of a sequence that do not compute
+constexpr int CORR_GROUPS = 2;   // sequences a CTA takes at most
 
 struct CorrSmem {
-  float* F;      // [2][S][5]  Fz then Fh
-  float* wg;     // [S]
-  int* cid;      // [L][K]
-  float* clp;    // [L][K]
-  float* top;    // [L][3]  l_i(c_0), l_i(c_1), l_i(c_3)
-  float* lprev;  // [L][K]  l_i(c_{i-1,k}); row 0 holds l_0(x0) in slot 0
-  float* red;    // [2][NW][32] per-warp reduced residual dots (NW > 1)
-  float* gpart;  // [2][NW]
-  Smem v;        // selections, ranks and refined scores kept for verification in the same CTA
+  uint64_t* full;  // [CORR_DEPTH] mbarriers: a stage's rows have landed
+  int* cid;        // [L][K], with K copies of x0 before it
+  float* clp;      // [L][K]
+  float4* feat;    // [L][K]  features 2, 3, 4 given that rank k of the position before was fed on,
+                   //         and the gate's share of all five features
+  float2* gap;     // [L]     features 0 and 1
+  float* usel;     // [L]
+  float* red;      // [2][32][CORR_PART] the residual dots' parts, zero past the computing warps
+  float* gpart;    // [2][CORR_PART]     the gate's parts
+  float* ring;     // [depth][stage]: the token rows and residual rows of a position
+  Smem v;          // selections, ranks and refined scores kept for verification in the same CTA
 };
 
-__host__ __device__ inline size_t corr_layout(int L, int K, int S, int NW, int V, bool verify,
-                                              char* base, CorrSmem* sm) {
+// Floats of one ring stage: the token rows of the first R candidates of the position before (2S
+// each) and, with rows, the residual rows of the K candidates (S each).
+__host__ __device__ inline int corr_stage(int K, int S, int R, bool rows) {
+  return 2 * S * R + (rows ? K * S : 0);
+}
+
+// Shared memory of one sequence.
+__host__ __device__ inline size_t corr_layout(int L, int K, int S, int V, int depth, int stage,
+                                              bool verify, char* base, CorrSmem* sm) {
   size_t off = 0;
   auto take = [&](size_t bytes) {
     const size_t o = off;
     off = align16(off + bytes);
     return base ? base + o : nullptr;
   };
-  char* pF = take(sizeof(float) * 10 * S);
-  char* pw = take(sizeof(float) * S);
-  char* pc = take(sizeof(int) * L * K);
+  char* pb = take(sizeof(uint64_t) * CORR_DEPTH);
+  char* pc = take(sizeof(int) * (L + 1) * K);
   char* pl = take(sizeof(float) * L * K);
-  char* pt = take(sizeof(float) * L * 3);
-  char* pp = take(sizeof(float) * L * K);
-  char* pr = take(sizeof(float) * 2 * NW * 32);
-  char* pg = take(sizeof(float) * 2 * NW);
+  char* pf = take(sizeof(float4) * L * K);
+  char* pg = take(sizeof(float2) * L);
+  char* pu = take(sizeof(float) * L);
+  char* pr = take(sizeof(float) * 2 * 32 * CORR_PART);
+  char* pp = take(sizeof(float) * 2 * CORR_PART);
+  char* pt = take(sizeof(float) * depth * stage);
   const size_t voff = off;
   if (sm) {
-    sm->F = (float*)pF; sm->wg = (float*)pw;
-    sm->cid = (int*)pc; sm->clp = (float*)pl; sm->top = (float*)pt; sm->lprev = (float*)pp;
-    sm->red = (float*)pr; sm->gpart = (float*)pg;
+    sm->full = (uint64_t*)pb;
+    sm->cid = (int*)pc + K; sm->clp = (float*)pl; sm->feat = (float4*)pf; sm->gap = (float2*)pg;
+    sm->usel = (float*)pu; sm->red = (float*)pr; sm->gpart = (float*)pp; sm->ring = (float*)pt;
   }
   // with verification in the same CTA its tables follow (the candidate table is the corrector's)
   if (!verify) return off;
@@ -515,390 +463,329 @@ __device__ __forceinline__ float reduce_scatter_n(float (&v)[NP]) {
   return r;
 }
 
-// Gathers n logits, entry e at index_of(e) into *dst_of(e), eight loads in flight per lane.
-template <int NT, typename IndexOf, typename DstOf>
-__device__ __forceinline__ void gather_logits(const void* logits, int dt, int n, IndexOf index_of,
-                                              DstOf dst_of) {
-  const int tid = threadIdx.x;
-  for (int base = 0; base < n; base += 8 * NT) {
-    float v[8];
-#pragma unroll
-    for (int j = 0; j < 8; ++j) {
-      const int e = base + j * NT + tid;
-      v[j] = e < n ? load_logit(logits, dt, index_of(e)) : 0.f;
-    }
-#pragma unroll
-    for (int j = 0; j < 8; ++j) {
-      const int e = base + j * NT + tid;
-      if (e < n) *dst_of(e) = v[j];
-    }
-  }
+// Asynchronous bulk copy of `bytes` (a multiple of 16) into shared memory, counted on `bar`.
+__device__ __forceinline__ void bulk_load(float* dst, const float* src, unsigned bytes,
+                                          uint64_t* bar) {
+  asm volatile(
+      "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
+          su32(dst)),
+      "l"(src), "r"(bytes), "r"(su32(bar))
+      : "memory");
 }
+// Asks for `bytes` (a multiple of 16) at p in L2.
+__device__ __forceinline__ void prefetch_l2(const float* p, unsigned bytes) {
+  asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p), "r"(bytes));
+}
+// Barrier `id` of the block for `threads` of its threads.
+__device__ __forceinline__ void group_sync(int id, int threads) {
+  asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(threads) : "memory");
+}
+// Bounded wait for the phase of the given parity (more than `limit` SM cycles: false).
+__device__ __forceinline__ bool mbar_wait_limit(uint64_t* bar, uint32_t parity, long long limit) {
+  if (mbar_test(bar, parity)) return true;
+  const long long t0 = clock64();
+  while (!mbar_test(bar, parity))
+    if (clock64() - t0 > limit) return false;
+  return true;
+}
+// Packed fp32 pairs of four elements: w x + y, and the sum of x y.
+__device__ __forceinline__ float4 fma4(const float4& w, const float2& x, const float4& y) {
+  const float2 lo = __ffma2_rn(make_float2(w.x, w.y), x, make_float2(y.x, y.y));
+  const float2 hi = __ffma2_rn(make_float2(w.z, w.w), x, make_float2(y.z, y.w));
+  return make_float4(lo.x, lo.y, hi.x, hi.y);
+}
+__device__ __forceinline__ float4 fma4(const float4& w, float x, const float4& y) {
+  return fma4(w, make_float2(x, x), y);
+}
+__device__ __forceinline__ float4 add4(const float4& x, const float4& y) {
+  const float2 lo = __fadd2_rn(make_float2(x.x, x.y), make_float2(y.x, y.y));
+  const float2 hi = __fadd2_rn(make_float2(x.z, x.w), make_float2(y.z, y.w));
+  return make_float4(lo.x, lo.y, hi.x, hi.y);
+}
+__device__ __forceinline__ float dot4(const float4& x, const float4& y) {
+  const float2 p = __ffma2_rn(make_float2(x.z, x.w), make_float2(y.z, y.w),
+                              __fmul2_rn(make_float2(x.x, x.y), make_float2(y.x, y.y)));
+  return p.x + p.y;
+}
+// Logistic function on the hardware exponential and reciprocal (relative error ~1e-7).
+__device__ __forceinline__ float rcp_hw(float x) {
+  float y;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
+}
+__device__ __forceinline__ float sigmoid_hw(float x) { return rcp_hw(1.f + ex2(-LOG2E * x)); }
 
-// The sequential corrector (Sec. 3.3 Eqs. 4-5; App. C.3 Eq. 9; Algorithm 1(b) loop), one CTA of
-// NW warps per sequence. Lane l of warp w owns the CW-element state chunks (CW = 1, 2 or 4)
-// c = l + 32 (w + NW m), m < CMC. The residual dots and the gate are reduced with warp
-// shuffles, then across the warps through shared memory (one block barrier a position), and
-// Select runs in every warp with lane k holding candidate k. Spreading a sequence over the
-// SM's four sub-partitions shortens the dependent chain of a position and keeps each
-// sub-partition's share small, so the verifier-row sweep beside it keeps its issue slots.
-// Every load of the step is issued unconditionally (chunk and candidate indices clamped into
-// range, the surplus contributions multiplied by zero state or never read) so the compiler can
-// keep them all in flight. Table rows are read through L2 (cache-global loads) a whole position
-// ahead into registers; an L2 line prefetch two positions ahead on top of that was slower
-// (single 105.7 -> 102.5 us for the products and the corrector without it, large_vocab
-// 269 -> 253 us). Shared memory holds the per-sequence tables (candidates, their log-probs, the
-// features' logits) and, for 4-element chunks, the feature shares and gate weights.
-// VERIFY: the CTA also verifies its sequence after the scan (the fused small-batch schedule); a
-// separate instantiation, since the verification code raises the scan's register count (122 ->
-// 143 a thread for four warps of 2-element chunks and K = 8), which would leave less room for
-// the verifier-row sweep beside the corrector in the overlapping schedule.
-template <int NW, int NP, int CMC, int CW, bool VERIFY>
-__global__ void __launch_bounds__(NW * 32)
+// The sequential corrector (Sec. 3.3 Eqs. 4-5; App. C.3 Eq. 9; Algorithm 1(b) loop). What bounds
+// it is the number of instructions on the dependent chain of a position, and beside it the ones
+// that every warp repeats; so few warps compute and the rest of the work is done by others or
+// beforehand. A sequence has ceil(S / 128) computing warps that own four state elements a lane.
+// A position is:
+//  - the minimal-GRU step on the lane's elements, its residual-dot and gate partials (packed
+//    fp32 pairs), a warp reduce-scatter, the warps' parts to shared memory, one barrier;
+//  - gate, refined scores and Select, in every warp alike: lane k adds the parts of candidate k.
+// A copying warp fetches the token rows of the first R candidates (one of which is usually fed
+// forward) and, with ROWS, the residual rows into a ring of `depth` positions by bulk copies, a
+// row a lane; a rank past R reads its token row through L2, and without ROWS the computing warps
+// load the residual rows themselves. One more warp asks rows into L2 some positions ahead (where
+// the ring is shallow) and stores the outputs. The features of every (position, rank fed
+// forward) pair are tabulated first; the shares of a position that do not depend on the
+// selection are summed before the barrier of the position before. A CTA takes one sequence, or
+// several side by side (a.groups), each with its own warps, barrier and shared memory.
+template <int NP, bool ROWS, bool SAMPLE, bool VERIFY>
+__global__ void __launch_bounds__(384)
 corrector_kernel(const __grid_constant__ ScanArgs a) {
   extern __shared__ __align__(16) char smem_raw[];
+  const int L = a.L, K = a.K, S = a.S, V = a.V, R = a.tok_ranks, D = a.ring_depth;
+  const int stage = corr_stage(K, S, R, ROWS);
+  const int NT = blockDim.x / a.groups, grp = threadIdx.x / NT;   // threads of a sequence
+  const int b = blockIdx.x * a.groups + grp;
+  if (b >= a.B) return;
+  const int tid = threadIdx.x - grp * NT, warp = tid >> 5, lane = tid & 31;
+  const int NC = NT - CORR_OTHERS;                                 // computing threads
+  auto sync = [&] { group_sync(1 + grp, NT); };
   CorrSmem sm;
-  corr_layout(a.L, a.K, a.S, NW, a.V, VERIFY, smem_raw, &sm);
-  constexpr int NT = NW * 32;
-  constexpr int LSTEP = 32 / NP;           // lane stride between reduced dots
-  const int b = blockIdx.x;
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int L = a.L, K = a.K, S = a.S, V = a.V;
+  const size_t own = corr_layout(L, K, S, V, D, stage, VERIFY, nullptr, nullptr);
+  corr_layout(L, K, S, V, D, stage, VERIFY, smem_raw + grp * own, &sm);
   const size_t bL = (size_t)b * L;
-  const int nch = S / CW;
+  constexpr int MODE = SAMPLE ? BRISK_SELECT_SAMPLE : BRISK_SELECT_GREEDY;
 
-  // Prologue in two dependent rounds of loads. First everything that depends neither on the
-  // candidates nor on x0, issued at once with the candidate table itself; then, after one
-  // barrier, what depends on them (the token shares of x0, the first position's residual rows
-  // and the features' logit gathers, in one batch).
-  // lane chunks, clamped into range; a chunk past the state keeps s = 0 throughout
-  int cc[CMC];
-  bool ok[CMC];
-#pragma unroll
-  for (int m = 0; m < CMC; ++m) {
-    const int c = lane + 32 * (warp + NW * m);
-    ok[m] = c < nch;
-    cc[m] = ok[m] ? c : nch - 1;
-  }
-  using C = Chunk<CW>;
+  // Prologue: the candidate table, then what depends on it.
   int x0 = a.x0[b];
-  // the Init share of h_c and the first position's hidden and position shares
-  C g0c[CMC], gz4[CMC], gh4[CMC], pz0[CMC], ph0[CMC];
-#pragma unroll
-  for (int m = 0; m < CMC; ++m) {
-    const int c = cc[m];
-    g0c[m] = ldc<CW, true>(a.G0 + (size_t)b * S + CW * c);
-    gz4[m] = ldc<CW, true>(a.G + bL * 2 * S + CW * c);
-    gh4[m] = ldc<CW, true>(a.G + bL * 2 * S + S + CW * c);
-    pz0[m] = ldc<CW, false>(a.posG + CW * c);
-    ph0[m] = ldc<CW, false>(a.posG + S + CW * c);
+  if (x0 < 0 || x0 >= V) {
+    if (tid == 0) set_status(a.status, BRISK_ERR_INVALID_ARG);
+    x0 = 0;
   }
-  float wgf[5];
-#pragma unroll
-  for (int f = 0; f < 5; ++f) wgf[f] = a.wg[S + f];
-  // chunks of up to two elements: this lane's feature shares (5 CW floats of F[S, 5] for z and
-  // for h) and gate weights, read every step, held in registers for the whole scan (4-element
-  // chunks read them from shared memory: in registers they would spill)
-  constexpr bool FREG = CW <= 2;
-  constexpr int FR = FREG ? CMC : 1;
-  float fzr[FR][5 * CW], fhr[FR][5 * CW];
-  C wgr[FR];
-  if constexpr (FREG) {
-#pragma unroll
-    for (int m = 0; m < CMC; ++m) {
-#pragma unroll
-      for (int q = 0; q < 5; ++q) {
-        const C vz = ldc<CW, false>(a.Fz + 5 * CW * cc[m] + CW * q);
-        const C vh = ldc<CW, false>(a.Fh + 5 * CW * cc[m] + CW * q);
-#pragma unroll
-        for (int e = 0; e < CW; ++e) {
-          fzr[m][CW * q + e] = vz.v[e];
-          fhr[m][CW * q + e] = vh.v[e];
-        }
-      }
-      wgr[m] = ldc<CW, false>(a.wg + CW * cc[m]);
-    }
-  }
-  const float sig_alpha = sigmoidf_(a.alpha);
-  // the candidate table
   for (int e = tid; e < L * K; e += NT) {
     int c = a.cand_ids[bL * K + e];
     if (c < 0 || c >= V) { set_status(a.status, BRISK_ERR_NUMERIC); c = 0; }
     sm.cid[e] = c;
     sm.clp[e] = a.cand_logprob[bL * K + e];
   }
-  if (x0 < 0 || x0 >= V) {
-    if (tid == 0) set_status(a.status, BRISK_ERR_INVALID_ARG);
-    x0 = 0;
+  if (tid < K) sm.cid[tid - K] = x0;
+  for (int i = tid; i < L; i += NT) sm.usel[i] = SAMPLE ? a.u_sel[bL + i] : 0.f;
+  for (int e = tid; e < 2 * 32 * CORR_PART; e += NT) sm.red[e] = 0.f;
+  if (tid < 2 * CORR_PART) sm.gpart[tid] = 0.f;
+  if (tid == 0) {
+    for (int d = 0; d < CORR_DEPTH; ++d) mbar_init(&sm.full[d], 1);
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    fence_async_smem();
   }
-  if constexpr (!FREG) {
-    // the feature shares and the gate weights into shared memory, all loads first
-    constexpr int FV = 2 * 5 * 1024 / 4 / NT + 1;   // float4 of Fz and Fh a thread, S <= 1024
-    float4 fv[FV];
-    const int nf = 5 * S / 4;
-#pragma unroll
-    for (int j = 0; j < FV; ++j) {
-      const int e = tid + j * NT;
-      fv[j] = e < nf ? ld4(a.Fz + 4 * e) : (e < 2 * nf ? ld4(a.Fh + 4 * (e - nf)) : float4{});
-    }
-    const float4 wv = tid < S / 4 ? ld4(a.wg + 4 * tid) : float4{};
-#pragma unroll
-    for (int j = 0; j < FV; ++j) {
-      const int e = tid + j * NT;
-      if (e < 2 * nf) reinterpret_cast<float4*>(sm.F)[e] = fv[j];
-    }
-    for (int e = tid; e < S / 4; e += NT)
-      reinterpret_cast<float4*>(sm.wg)[e] = e == tid ? wv : ld4(a.wg + 4 * e);
-  }
-  __syncthreads();
+  sync();
 
-  // second round: the token shares of x0, the first position's residual rows (below) and the
-  // features' logit gathers, all independent of the selections
-  C t0c[CMC], tz4[CMC], th4[CMC];
+  // the features of every position for every rank that may be fed forward (position 0: x0)
+  auto features = [&] {
+    const void* lq = a.logits_q;
+    float w[5];
 #pragma unroll
-  for (int m = 0; m < CMC; ++m) {
-    const int c = cc[m];
-    t0c[m] = ldc<CW, true>(a.T0 + (size_t)x0 * S + CW * c);
-    tz4[m] = ldc<CW, true>(a.Tzh + (size_t)x0 * 2 * S + CW * c);   // token share of x_{-1} = x0
-    th4[m] = ldc<CW, true>(a.Tzh + (size_t)x0 * 2 * S + S + CW * c);
-  }
-  const void* lq = a.logits_q;
-  const int ldt = a.logits_dt;
-  gather_logits<NT>(
-      lq, ldt, L * 3 + L * K,
-      [&](int e) {
-        if (e < L * 3) {
-          const int i = e / 3, w = e % 3;
-          return (bL + i) * V + sm.cid[i * K + (w == 0 ? 0 : (w == 1 ? 1 : 3))];
-        }
-        e -= L * 3;
-        const int i = e / K, k = e % K;
-        return i == 0 ? bL * V + x0 : (bL + i) * V + sm.cid[(i - 1) * K + k];
-      },
-      [&](int e) { return e < L * 3 ? sm.top + e : sm.lprev + (e - L * 3); });
-  C s4[CMC];
-#pragma unroll
-  for (int m = 0; m < CMC; ++m) {
-#pragma unroll
-    for (int e = 0; e < CW; ++e)                              // s_{-1} = u_0 = Init(h_c, E(x0))
-      s4[m].v[e] = ok[m] ? tanhf(g0c[m].v[e] + t0c[m].v[e]) : 0.f;
-    gz4[m] = addc(gz4[m], pz0[m]);
-    gh4[m] = addc(gh4[m], ph0[m]);
-  }
-  __syncthreads();
-
-  // Software pipeline across positions: the next position's residual rows (rank K-1 repeated
-  // past K) and hidden and position shares are loaded into registers one step ahead (issued at
-  // the top of the step: issued after the step's dots they were still in flight when the next
-  // step began, single 118 -> 110 us for the products and the corrector), and so is the
-  // token-share row of this position's rank-0 candidate, the usual next previous token.
-  // (Only while the rows fit in registers: NP * CMC <= 16 vectors a lane; wider variants load
-  // them in the step.)
-  constexpr bool PIPE = NP * CMC <= 16;
-  constexpr int PK = PIPE ? NP : 1;
-  C ub[PK][CMC];
-  if constexpr (PIPE) {
-#pragma unroll
-    for (int k = 0; k < NP; ++k) {
-      const float* Uk = a.U + (size_t)sm.cid[k < K ? k : K - 1] * S;
-#pragma unroll
-      for (int m = 0; m < CMC; ++m) ub[k][m] = ldc<CW, true>(Uk + CW * cc[m]);
+    for (int f = 0; f < 5; ++f) w[f] = a.wg[S + f];
+    for (int e = tid; e < L * K; e += NT) {
+      const int i = e / K, k = e - i * K;
+      const int* ci = sm.cid + i * K;
+      const int x = sm.cid[e - K];
+      const size_t row = (bL + i) * V;
+      const float l0 = load_logit(lq, a.logits_dt, row + ci[0]);
+      const float l1 = load_logit(lq, a.logits_dt, row + ci[1]);
+      const float l3 = load_logit(lq, a.logits_dt, row + ci[3]);
+      const float lx = load_logit(lq, a.logits_dt, row + x);
+      const float phi0 = l0 - l1, phi1 = l0 - l3, phi4 = l0 - lx;
+      const float phi2 = x == ci[0] ? 1.f : 0.f;
+      const float phi3 = x == ci[0] || x == ci[1] || x == ci[2] || x == ci[3] ? 1.f : 0.f;
+      if (k == 0) sm.gap[i] = make_float2(phi0, phi1);
+      float g = a.b_g;
+      g = fmaf(w[0], phi0, g); g = fmaf(w[1], phi1, g); g = fmaf(w[2], phi2, g);
+      g = fmaf(w[3], phi3, g); g = fmaf(w[4], phi4, g);
+      sm.feat[e] = make_float4(phi2, phi3, phi4, g);
     }
-  }
-  C tsz[CMC], tsh[CMC];                      // token share of the speculated previous token
-  int ts_id = -1;
+  };
 
-  int prev = x0, prank = 0;
-  float u_cur = (a.select_mode == BRISK_SELECT_SAMPLE) ? a.u_sel[bL] : 0.f;
-  for (int i = 0; i < L; ++i) {
-    const int buf = i & 1;
-    const int* ci = sm.cid + i * K;
-    // into registers, for step i + 1: its hidden and position shares, residual rows and the
-    // rank-0 token-share row
-    C un[PK][CMC], tnz[CMC], tnh[CMC], gnz[CMC], gnh[CMC], pnz[CMC], pnh[CMC];
-    if (i + 1 < L) {
-      const float* Gn = a.G + (bL + i + 1) * 2 * S;
-      const float* Pn = a.posG + (size_t)(i + 1) * 2 * S;
+  const float sig_alpha = sigmoidf_(a.alpha);
+  // gate, refined scores and Select of position i: every lane gets the selection, lane k the
+  // refined score of candidate k; `share` is the gate's share of the features
+  auto decide = [&](int i, float share, float& ref) -> int {
+    const float* red = sm.red + ((i & 1) * 32 + lane) * CORR_PART;
+    const float* gp = sm.gpart + (i & 1) * CORR_PART;
+    const float lp = lane < K ? sm.clp[i * K + lane] : -INFINITY;
+    const float4 d0 = ld4(red), q0 = ld4(gp);
+    float dk = (d0.x + d0.y) + (d0.z + d0.w);
+    float gs = (q0.x + q0.y) + (q0.z + q0.w);
+    if (NC > 128) {
+      const float4 d1 = ld4(red + 4), q1 = ld4(gp + 4);
+      dk += (d1.x + d1.y) + (d1.z + d1.w);
+      gs += (q1.x + q1.y) + (q1.z + q1.w);
+    }
+    ref = fmaf(sig_alpha * sigmoid_hw(share + gs), dk, lp);   // (lanes past K: dk = 0)
+    return select_warp(ref, K, MODE, SAMPLE ? sm.usel[i] : 0.f);
+  };
+  // the token fed forward: the head's selection, or in a same-state replay the base selection
+  // (the Select rule on the base scores log q, same draw)
+  auto base_pick = [&](int i) {
+    return select_warp(lane < K ? sm.clp[i * K + lane] : -INFINITY, K, MODE,
+                       SAMPLE ? sm.usel[i] : 0.f);
+  };
+
+  if (tid < NC) {
+    const bool owns = 4 * tid < S;           // state elements 4 tid .. 4 tid + 3
+    const int e4 = owns ? 4 * tid : 0;       // (others keep a zero state)
+    const float4 g0 = __ldcg(reinterpret_cast<const float4*>(a.G0 + (size_t)b * S + e4));
+    const float4 t0 = __ldcg(reinterpret_cast<const float4*>(a.T0 + (size_t)x0 * S + e4));
+    const float* gp = a.G + bL * 2 * S + e4;
+    float4 zb = __ldcg(reinterpret_cast<const float4*>(gp));
+    float4 hb = __ldcg(reinterpret_cast<const float4*>(gp + S));
+    float4 fz[5], fh[5];                     // feature shares of the four elements, by feature
+    {
+      float z[20], h[20];
 #pragma unroll
-      for (int m = 0; m < CMC; ++m) {
-        gnz[m] = ldc<CW, true>(Gn + CW * cc[m]);
-        gnh[m] = ldc<CW, true>(Gn + S + CW * cc[m]);
-        pnz[m] = ldc<CW, false>(Pn + CW * cc[m]);
-        pnh[m] = ldc<CW, false>(Pn + S + CW * cc[m]);
+      for (int q = 0; q < 5; ++q) {
+        *reinterpret_cast<float4*>(z + 4 * q) = ld4(a.Fz + 5 * e4 + 4 * q);
+        *reinterpret_cast<float4*>(h + 4 * q) = ld4(a.Fh + 5 * e4 + 4 * q);
       }
-      if constexpr (PIPE) {
 #pragma unroll
-        for (int k = 0; k < NP; ++k) {
-          const float* Uk = a.U + (size_t)ci[K + (k < K ? k : K - 1)] * S;
-#pragma unroll
-          for (int m = 0; m < CMC; ++m) un[k][m] = ldc<CW, true>(Uk + CW * cc[m]);
-        }
-      }
-      const float* Tn = a.Tzh + (size_t)ci[0] * 2 * S;
-#pragma unroll
-      for (int m = 0; m < CMC; ++m) {
-        tnz[m] = ldc<CW, true>(Tn + CW * cc[m]);
-        tnh[m] = ldc<CW, true>(Tn + S + CW * cc[m]);
+      for (int f = 0; f < 5; ++f) {
+        fz[f] = make_float4(z[f], z[5 + f], z[10 + f], z[15 + f]);
+        fh[f] = make_float4(h[f], h[5 + f], h[10 + f], h[15 + f]);
       }
     }
-    // confidence features of position i (App. C.3)
-    const float l0 = sm.top[i * 3 + 0];
-    float phi[5];
-    phi[0] = l0 - sm.top[i * 3 + 1];
-    phi[1] = l0 - sm.top[i * 3 + 2];
-    phi[2] = (prev == ci[0]) ? 1.f : 0.f;
-    phi[3] = (prev == ci[0] || prev == ci[1] || prev == ci[2] || prev == ci[3]) ? 1.f : 0.f;
-    phi[4] = l0 - sm.lprev[i * K + (i == 0 ? 0 : prank)];
-    // token share of the previous token (x0's came with the prologue; the speculated one is
-    // already in registers)
-    if (i > 0) {
-      if (prev == ts_id) {
-#pragma unroll
-        for (int m = 0; m < CMC; ++m) {
-          tz4[m] = tsz[m];
-          th4[m] = tsh[m];
-        }
+    const float4 wg = ld4(a.wg + e4);
+    features();
+    float4 s = make_float4(0.f, 0.f, 0.f, 0.f);   // s_{-1} = u_0 = Init(h_c, E(x0))
+    if (owns) s = make_float4(tanhf(g0.x + t0.x), tanhf(g0.y + t0.y), tanhf(g0.z + t0.z),
+                              tanhf(g0.w + t0.w));
+    sync();
+    {
+      const float2 gap = sm.gap[0];
+      zb = fma4(fz[0], gap.x, fma4(fz[1], gap.y, zb));
+      hb = fma4(fh[0], gap.x, fma4(fh[1], gap.y, hb));
+    }
+    bool alive = mbar_wait_limit(&sm.full[0], 0, a.wait_limit);
+    const float* st = sm.ring + e4;          // this lane's place in the present stage
+    int prank = 0, slot = 0, parity = 0;
+    for (int i = 0; i < L; ++i) {
+      const bool more = i + 1 < L;
+      const float4 ft = sm.feat[i * K + prank];
+      float4 tz, th;
+      if (prank < R) {
+        const float* t = st + 2 * S * prank;
+        tz = ld4(t);
+        th = ld4(t + S);
       } else {
-        const float* Tp = a.Tzh + (size_t)prev * 2 * S;
+        const float* t = a.Tzh + (size_t)sm.cid[(i - 1) * K + prank] * 2 * S + e4;
+        tz = __ldcg(reinterpret_cast<const float4*>(t));
+        th = __ldcg(reinterpret_cast<const float4*>(t + S));
+      }
+      float4 nz, nh;                          // the next position's hidden shares, on their way
+      if (more) {
+        gp += 2 * S;
+        nz = __ldcg(reinterpret_cast<const float4*>(gp));
+        nh = __ldcg(reinterpret_cast<const float4*>(gp + S));
+      }
+      // minimal-GRU step: s + z (h - s)
+      zb = fma4(fz[2], ft.x, fma4(fz[3], ft.y, fma4(fz[4], ft.z, zb)));
+      hb = fma4(fh[2], ft.x, fma4(fh[3], ft.y, fma4(fh[4], ft.z, hb)));
+      const float4 z = add4(zb, tz);
+      float4 h = add4(hb, th);
+      h = fma4(s, -1.f, h);
+      if (owns) {
+        const float2 lo = __ffma2_rn(make_float2(sigmoid_hw(z.x), sigmoid_hw(z.y)),
+                                     make_float2(h.x, h.y), make_float2(s.x, s.y));
+        const float2 hi = __ffma2_rn(make_float2(sigmoid_hw(z.z), sigmoid_hw(z.w)),
+                                     make_float2(h.z, h.w), make_float2(s.z, s.w));
+        s = make_float4(lo.x, lo.y, hi.x, hi.y);
+      }
+      // residual-dot and gate partials
+      float part[NP];
+      const float* ur = st + 2 * S * R;
 #pragma unroll
-        for (int m = 0; m < CMC; ++m) {
-          tz4[m] = ldc<CW, true>(Tp + CW * cc[m]);
-          th4[m] = ldc<CW, true>(Tp + S + CW * cc[m]);
+      for (int k = 0; k < NP; ++k) {
+        const int kk = k < K ? k : K - 1;
+        float4 u;
+        if constexpr (ROWS) u = ld4(ur + kk * S);
+        else u = __ldcg(reinterpret_cast<const float4*>(a.U + (size_t)sm.cid[i * K + kk] * S + e4));
+        part[k] = dot4(u, s);
+      }
+      const float g = warp_sum(dot4(wg, s));
+      const float r = reduce_scatter_n<NP>(part);
+      constexpr int LSTEP = 32 / NP;
+      if ((lane & (LSTEP - 1)) == 0)
+        sm.red[((i & 1) * 32 + lane / LSTEP) * CORR_PART + warp] = r;
+      if (lane == 0) sm.gpart[(i & 1) * CORR_PART + warp] = g;
+      if (more) {
+        const float2 gap = sm.gap[i + 1];
+        zb = fma4(fz[0], gap.x, fma4(fz[1], gap.y, nz));
+        hb = fma4(fh[0], gap.x, fma4(fh[1], gap.y, nh));
+        // the next position's rows: a wait that gave up is not repeated
+        st += stage;
+        if (++slot == D) {
+          slot = 0;
+          parity ^= 1;
+          st = sm.ring + e4;
         }
+        if (alive) alive = mbar_wait_limit(&sm.full[slot], parity, a.wait_limit);
       }
+      sync();
+      float ref;
+      const int pick = decide(i, ft.w, ref);
+      prank = a.base_prefix ? base_pick(i) : pick;
     }
-    // minimal-GRU step on this lane's chunks and its gate partial
-    float gacc = 0.f;
-#pragma unroll
-    for (int m = 0; m < CMC; ++m) {
-      const int c = cc[m];
-      C zp = addc(gz4[m], tz4[m]), hp = addc(gh4[m], th4[m]);
-      // feature shares of this chunk's elements: 5 CW contiguous floats of F[S, 5]
-      float fz[5 * CW], fh[5 * CW];
-      if constexpr (FREG) {
-#pragma unroll
-        for (int j = 0; j < 5 * CW; ++j) {
-          fz[j] = fzr[m][j];
-          fh[j] = fhr[m][j];
-        }
-      } else {
-#pragma unroll
-        for (int q = 0; q < 5; ++q) {
-          const C vz = ldc<CW, false>(sm.F + 5 * CW * c + CW * q);
-          const C vh = ldc<CW, false>(sm.F + 5 * S + 5 * CW * c + CW * q);
-#pragma unroll
-          for (int e = 0; e < CW; ++e) {
-            fz[CW * q + e] = vz.v[e];
-            fh[CW * q + e] = vh.v[e];
-          }
-        }
+    if (!alive) set_status(a.status, BRISK_ERR_TIMEOUT);
+  } else if (tid < NC + 32) {
+    // rows of position p into a stage, a row a lane: token rows, residual rows
+    const int rows = R + (ROWS ? K : 0);
+    auto fetch = [&](int p, int slot) {
+      if (p >= L) return;
+      float* base = sm.ring + slot * stage;
+      const int* id = sm.cid + p * K;
+      if (lane == 0) mbar_expect_tx(&sm.full[slot], (unsigned)stage * 4);
+      __syncwarp();
+      for (int j = lane; j < rows; j += 32) {
+        if (j < R) bulk_load(base + 2 * S * j, a.Tzh + (size_t)id[j - K] * 2 * S, 8 * S, &sm.full[slot]);
+        else bulk_load(base + 2 * S * R + (j - R) * S, a.U + (size_t)id[j - R] * S, 4 * S, &sm.full[slot]);
       }
-#pragma unroll
-      for (int e = 0; e < CW; ++e)
-#pragma unroll
-        for (int f = 0; f < 5; ++f) {
-          zp.v[e] = fmaf(fz[5 * e + f], phi[f], zp.v[e]);
-          hp.v[e] = fmaf(fh[5 * e + f], phi[f], hp.v[e]);
-        }
-#pragma unroll
-      for (int e = 0; e < CW; ++e) {
-        const float z = sigmoid_fast(zp.v[e]);
-        s4[m].v[e] = ok[m] ? (1.f - z) * s4[m].v[e] + z * hp.v[e] : 0.f;
-      }
-      if constexpr (FREG) gacc = dotc(wgr[m], s4[m], gacc);
-      else gacc = dotc(ldc<CW, false>(sm.wg + CW * c), s4[m], gacc);
+    };
+    for (int p = 0; p < D - 1; ++p) fetch(p, p);
+    features();
+    sync();
+    int slot = D - 1;                     // of position i + D - 1
+    for (int i = 0; i < L; ++i) {
+      fetch(i + D - 1, slot);             // (its stage was last read before the sync just passed)
+      slot = slot + 1 == D ? 0 : slot + 1;
+      sync();
     }
-    // residual-dot partials with the rows of this position's candidates
-    float part[NP];
-#pragma unroll
-    for (int k = 0; k < NP; ++k) {
-      const float* Uk = a.U + (size_t)ci[k < K ? k : K - 1] * S;
-      float acc = 0.f;
-#pragma unroll
-      for (int m = 0; m < CMC; ++m) {
-        C u;
-        if constexpr (PIPE) u = ub[k][m];
-        else u = ldc<CW, true>(Uk + CW * cc[m]);
-        acc = dotc(u, s4[m], acc);
-      }
-      part[k] = acc;
-    }
-    // hidden and position shares of the next position: plain loads first used in the next step
-    if (i + 1 < L) {
-#pragma unroll
-      for (int m = 0; m < CMC; ++m) {
-        gz4[m] = addc(gnz[m], pnz[m]);
-        gh4[m] = addc(gnh[m], pnh[m]);
-      }
-    }
-    // residual dots by a warp reduce-scatter; across warps through shared memory, where lane k
-    // sums the warps' partials of dot k (one shuffle fewer on the step's chain than summing in
-    // the reduce-scatter's lanes and moving dot k to lane k afterwards)
-    const float r = reduce_scatter_n<NP>(part);
-    gacc = warp_sum(gacc);
-    float dk;
-    if constexpr (NW > 1) {
-      float* red = sm.red + buf * NW * 32;
-      if ((lane & (LSTEP - 1)) == 0) red[warp * 32 + lane / LSTEP] = r;
-      if (lane == 0) sm.gpart[buf * NW + warp] = gacc;
-      __syncthreads();
-      const int vidx = lane & (NP - 1);
-      dk = red[vidx];
-      gacc = sm.gpart[buf * NW];
-      for (int w = 1; w < NW; ++w) {
-        dk += red[w * 32 + vidx];
-        gacc += sm.gpart[buf * NW + w];
-      }
-    } else {
-      dk = __shfl_sync(FULL_MASK, r, (lane * LSTEP) & 31);
-    }
-    // gate, refined scores (lane k: candidate k) and Select, identically in every warp
-    float gate = a.b_g + gacc;
-#pragma unroll
-    for (int f = 0; f < 5; ++f) gate = fmaf(wgf[f], phi[f], gate);
-    const float gamma = sig_alpha * sigmoid_fast(gate);
-    const float ref = lane < K ? sm.clp[i * K + lane] + gamma * dk : -INFINITY;
-    const float u_cur_draw = u_cur;
-    const int pick = select_warp(ref, K, a.select_mode, u_cur);
-    if (warp == 0) {
+    // a computing warp that gave up waiting leaves copies in flight: they end before the CTA does
+    if (lane == 0)
+      for (int p = L - D < 0 ? 0 : L - D; p < L; ++p) mbar_drain(&sm.full[p % D], (p / D) & 1);
+  } else {
+    auto ask = [&](int p) {
+      if (!a.ask_rows || p >= L || lane >= K) return;
+      prefetch_l2(a.U + (size_t)sm.cid[p * K + lane] * S, S * 4);
+      if (a.ask_tokens && p + 1 < L) prefetch_l2(a.Tzh + (size_t)sm.cid[p * K + lane] * 2 * S, S * 8);
+    };
+    for (int p = 0; p < CORR_AHEAD; ++p) ask(p);
+    features();
+    sync();
+    int prank = 0;
+    bool bad = false;
+    for (int i = 0; i < L; ++i) {
+      ask(i + CORR_AHEAD);
+      sync();
+      float ref;
+      const int pick = decide(i, sm.feat[i * K + prank].w, ref);
       if (lane < K) a.refined[(bL + i) * K + lane] = ref;
-      if (__any_sync(FULL_MASK, lane < K && isnan(ref)) && lane == 0)
-        set_status(a.status, BRISK_ERR_NUMERIC);
-    }
-    if (a.select_mode == BRISK_SELECT_SAMPLE && i + 1 < L) u_cur = a.u_sel[bL + i + 1];
-    if (tid == 0) {
-      a.sel_tokens[bL + i] = ci[pick];
+      bad |= isnan(ref);
+      if (lane == 0) a.sel_tokens[bL + i] = sm.cid[i * K + pick];
       if constexpr (VERIFY) {
-        sm.v.sel[i] = ci[pick];
-        sm.v.rank[i] = pick;
+        if (lane < K) sm.v.ref[i * K + lane] = ref;
+        if (lane == 0) {
+          sm.v.sel[i] = sm.cid[i * K + pick];
+          sm.v.rank[i] = pick;
+        }
+      }
+      prank = pick;
+      if (a.base_prefix) {
+        prank = base_pick(i);
+        if (lane == 0) a.base_rank[bL + i] = prank;
       }
     }
-    if constexpr (VERIFY)
-      if (warp == 0 && lane < K) sm.v.ref[i * K + lane] = ref;
-    // the token fed forward: the head's selection, or in a same-state replay the base
-    // selection (the Select rule on the base scores log q, same draw)
-    int fwd = pick;
-    if (a.base_prefix) {
-      fwd = select_warp(lane < K ? sm.clp[i * K + lane] : -INFINITY, K, a.select_mode, u_cur_draw);
-      if (tid == 0) a.base_rank[bL + i] = fwd;
-    }
-    prank = fwd;
-    prev = ci[fwd];
-    // advance the pipeline
-    if (i + 1 < L) {
-      if constexpr (PIPE) {
-#pragma unroll
-        for (int k = 0; k < NP; ++k)
-#pragma unroll
-          for (int m = 0; m < CMC; ++m) ub[k][m] = un[k][m];
-      }
-#pragma unroll
-      for (int m = 0; m < CMC; ++m) {
-        tsz[m] = tnz[m];
-        tsh[m] = tnh[m];
-      }
-      ts_id = ci[0];
-    }
+    if (bad) set_status(a.status, BRISK_ERR_NUMERIC);
   }
   // verification of this sequence in the same CTA (the verifier rows' statistics are complete:
   // their sweep ran before this kernel)
@@ -914,45 +801,70 @@ size_t scan_smem_bytes(int L, int K, int S, int V) {
   return smem_layout(L, K, S, V, nullptr, nullptr);
 }
 
-template <int NW, int NP, int CMC, int CW, bool VERIFY>
+namespace {
+
+constexpr size_t CORR_SMEM = 220 * 1024;   // shared memory a CTA may take
+
+template <int NP, bool ROWS, bool SAMPLE, bool VERIFY>
 cudaError_t launch_corrector_k(const ScanArgs& a, cudaStream_t stream) {
-  const size_t smem = corr_layout(a.L, a.K, a.S, NW, a.V, VERIFY, nullptr, nullptr);
-  auto kernel = corrector_kernel<NW, NP, CMC, CW, VERIFY>;
+  const size_t smem = a.groups * corr_layout(a.L, a.K, a.S, a.V, a.ring_depth,
+                                             corr_stage(a.K, a.S, a.tok_ranks, ROWS), VERIFY,
+                                             nullptr, nullptr);
+  auto kernel = corrector_kernel<NP, ROWS, SAMPLE, VERIFY>;
   cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e == cudaSuccess) e = prefer_carveout(kernel, CARVEOUT_SMALL_KB);
   if (e != cudaSuccess) return e;
-  e = launch_prio(kernel, dim3(a.B), dim3(NW * 32), smem, stream, a);
+  const int threads = 32 * ((a.S + CORR_SPAN - 1) / CORR_SPAN) + CORR_OTHERS;
+  e = launch_prio(kernel, dim3((a.B + a.groups - 1) / a.groups), dim3(a.groups * threads), smem,
+                  stream, a);
   if (e != cudaSuccess) return e;
   return cudaGetLastError();
 }
 
-template <int NW, int CW, int NP>
-cudaError_t launch_corrector(const ScanArgs& a, cudaStream_t stream) {
-  if (a.do_verify) return launch_corrector_k<NW, NP, 1, CW, true>(a, stream);
-  return launch_corrector_k<NW, NP, 1, CW, false>(a, stream);
+template <int NP, bool ROWS>
+cudaError_t launch_corrector_m(const ScanArgs& a, cudaStream_t stream) {
+  if (a.select_mode == BRISK_SELECT_SAMPLE)
+    return a.do_verify ? launch_corrector_k<NP, ROWS, true, true>(a, stream)
+                       : launch_corrector_k<NP, ROWS, true, false>(a, stream);
+  return a.do_verify ? launch_corrector_k<NP, ROWS, false, true>(a, stream)
+                     : launch_corrector_k<NP, ROWS, false, false>(a, stream);
 }
 
-template <int NW, int CW>
-cudaError_t launch_corrector_for_k(const ScanArgs& a, cudaStream_t stream) {
-  if (a.K <= 8) return launch_corrector<NW, CW, 8>(a, stream);
-  return a.K <= 16 ? launch_corrector<NW, CW, 16>(a, stream) : launch_corrector<NW, CW, 32>(a, stream);
+cudaError_t launch_corrector(const ScanArgs& args, cudaStream_t stream) {
+  ScanArgs a = args;
+  a.wait_limit = wait_limit_cycles();
+  // Beside the verifier-row sweep, sequences of up to 512 state elements share CTAs: a corrector
+  // CTA keeps the sweep's off its SM, so fewer and fuller ones leave it more SMs.
+  a.groups = a.beside_sweep && a.S <= 512 && !a.do_verify ? CORR_GROUPS : 1;
+  // the ring's depth, the token rows a stage holds, and whether it holds the residual rows: the
+  // first of these that fits
+  struct Shape { int depth, ranks; bool rows; };
+  const Shape shapes[] = {{4, 4, true}, {3, 4, true}, {3, 2, true}, {3, 1, true}, {2, 2, true},
+                          {2, 1, true}, {4, 4, false}, {3, 2, false}, {2, 1, false}};
+  bool rows = false;
+  for (const Shape& s : shapes) {
+    a.ring_depth = s.depth;
+    a.tok_ranks = s.ranks;
+    rows = s.rows;
+    if (a.groups * corr_layout(a.L, a.K, a.S, a.V, s.depth, corr_stage(a.K, a.S, s.ranks, s.rows),
+                               a.do_verify != 0, nullptr, nullptr) <= CORR_SMEM)
+      break;
+  }
+  a.ask_rows = a.ring_depth < 4;
+  a.ask_tokens = !a.beside_sweep;
+  if (a.K <= 8)
+    return rows ? launch_corrector_m<8, true>(a, stream) : launch_corrector_m<8, false>(a, stream);
+  if (a.K <= 16)
+    return rows ? launch_corrector_m<16, true>(a, stream) : launch_corrector_m<16, false>(a, stream);
+  return rows ? launch_corrector_m<32, true>(a, stream) : launch_corrector_m<32, false>(a, stream);
 }
+
+}  // namespace
 
 // The corrector (do_select; with do_verify also the verification in the same CTA) or the
 // verification alone (do_verify) for every sequence.
 cudaError_t launch_scan(const ScanArgs& a, cudaStream_t stream) {
-  if (a.do_select) {
-    // One chunk a lane. A state of up to 256 takes four warps, one per SM sub-partition, of
-    // 1- or 2-element chunks (every lane busy); 257..512 eight warps of 2-element chunks and a
-    // wider one (up to 1024) eight warps of 4-element chunks: two warps of the sequence on each
-    // sub-partition to issue from. (At S = 512 eight warps of 2-element chunks beat four of
-    // 4-element chunks, single 144 -> 135 us a tail, and sixteen of single elements, 138 us:
-    // the cross-warp sums grow with the warps.)
-    if (a.S > 4 * 32 * CORR_WARPS) return launch_corrector_for_k<2 * CORR_WARPS, 4>(a, stream);
-    if (a.S > 2 * 32 * CORR_WARPS) return launch_corrector_for_k<2 * CORR_WARPS, 2>(a, stream);
-    if (a.S > 32 * CORR_WARPS) return launch_corrector_for_k<CORR_WARPS, 2>(a, stream);
-    return launch_corrector_for_k<CORR_WARPS, 1>(a, stream);
-  }
+  if (a.do_select) return launch_corrector(a, stream);
   const size_t smem = scan_smem_bytes(a.L, a.K, a.S, a.V);
   cudaError_t e = cudaFuncSetAttribute(verify_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        (int)smem);
