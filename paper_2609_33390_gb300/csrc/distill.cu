@@ -12,7 +12,7 @@
 namespace brisk {
 namespace {
 
-constexpr int DISTILL_WARPS = 4;
+constexpr int DISTILL_WARPS = 16;   // two positions a warp for blocks of 32
 
 __device__ __forceinline__ float load_logit_d(const void* base, int dt, size_t idx) {
   if (dt == BRISK_DT_BF16) return __bfloat162float(reinterpret_cast<const __nv_bfloat16*>(base)[idx]);
@@ -93,10 +93,19 @@ distill_kernel(const __grid_constant__ DistillArgs a) {
   __syncthreads();
   if (!last) return;
   __threadfence();
+  // the last CTA: every partial is visible; all threads fetch them, one adds them in sequence
+  // order (one thread fetching them as it adds waits for L2 every few of them)
+  __shared__ float fetched[DISTILL_WARPS * 32];
+  float total = 0.f;
+  for (int s0 = 0; s0 < a.B; s0 += DISTILL_WARPS * 32) {
+    const int s = s0 + (int)threadIdx.x;
+    fetched[threadIdx.x] = s < a.B ? __ldcg(a.partial + s) : 0.f;
+    __syncthreads();
+    if (threadIdx.x == 0)
+      for (int j = 0; j < min(a.B - s0, DISTILL_WARPS * 32); ++j) total += fetched[j];
+    __syncthreads();
+  }
   if (threadIdx.x == 0) {
-    // the last CTA: every partial is visible; add them in sequence order
-    float total = 0.f;
-    for (int s = 0; s < a.B; ++s) total += __ldcg(a.partial + s);
     a.loss[0] = total * inv_n;
     *a.arrivals = 0;
   }
