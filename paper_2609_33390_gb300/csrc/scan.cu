@@ -41,6 +41,7 @@ struct Smem {
 __host__ __device__ inline size_t align16(size_t x) { return (x + 15) & ~size_t(15); }
 
 constexpr int RES_BLOCK = 256;  // residual-sampling block: 32 lanes x 8 ids
+constexpr int RES_FLIGHT = 4;   // blocks whose logits a warp loads at once
 
 __host__ __device__ inline size_t smem_layout(int L, int K, int S, int V, char* base, Smem* sm) {
   size_t off = 0;
@@ -117,16 +118,10 @@ __device__ __forceinline__ float proposal_mass(const float* ref, int K, int mode
   return expf(ref[r] - mx) / tot;
 }
 
-// Residual R(v) = max(0, p(v) - pi(v)) of the 8 ids [v0, v0+8) owned by this lane, with
-// p(v) = 2^(l(v) log2 e - lse log2 e) on the hardware exponential (v0 is a multiple of 8, so a
+// The logits of the 8 ids [v0, v0 + 8) owned by this lane (v0 is a multiple of 8, so a
 // 16-byte-aligned row gives aligned 16-byte vector loads; ragged ends and unaligned rows take
-// element loads). Lanes k < K hold candidate k: (cand_id, cand_mass).
-__device__ __forceinline__ void residual8(const void* rowp, int dt, int V, float lse, int v0,
-                                         int blk0, int cand_id, float cand_mass, int K,
-                                         float (&R)[8]) {
-  const int lane = threadIdx.x & 31;
-  const float nlb = -lse * LOG2E;
-  float l[8];
+// element loads). -inf past V.
+__device__ __forceinline__ void logits8(const void* rowp, int dt, int V, int v0, float (&l)[8]) {
   const bool vec = v0 + 8 <= V && (reinterpret_cast<uintptr_t>(rowp) & 15u) == 0;
   if (vec && dt == BRISK_DT_BF16) {
     unpack(__ldg(reinterpret_cast<const uint4*>(reinterpret_cast<const __nv_bfloat16*>(rowp) + v0)),
@@ -145,6 +140,15 @@ __device__ __forceinline__ void residual8(const void* rowp, int dt, int V, float
 #pragma unroll
     for (int e = 0; e < 8; ++e) l[e] = v0 + e < V ? load_logit(rowp, dt, (size_t)(v0 + e)) : -INFINITY;
   }
+}
+
+// Residual R(v) = max(0, p(v) - pi(v)) of the 8 ids [v0, v0 + 8) with logits l, with
+// p(v) = 2^(l(v) log2 e - lse log2 e) on the hardware exponential. Lanes k < K hold candidate k:
+// (cand_id, cand_mass).
+__device__ __forceinline__ void residual8(const float (&l)[8], float lse, int v0, int blk0,
+                                         int cand_id, float cand_mass, int K, float (&R)[8]) {
+  const int lane = threadIdx.x & 31;
+  const float nlb = -lse * LOG2E;
 #pragma unroll
   for (int e = 0; e < 8; ++e) R[e] = ex2(fmaf(l[e], LOG2E, nlb));
   const bool mine = lane < K && cand_id >= blk0 && cand_id < blk0 + RES_BLOCK;
@@ -178,16 +182,27 @@ __device__ int residual_sample(const Smem& sm, const void* rowp, int dt, int V, 
     if (select_mode == BRISK_SELECT_GREEDY) cand_mass = (lane == sel_rank) ? 1.f : 0.f;
     else cand_mass = proposal_mass(ref, K, select_mode, lane);
   }
-  // pass 1: block sums (blocks interleaved over warps)
-  for (int blk = warp; blk < nblk; blk += (int)(blockDim.x >> 5)) {
-    const int blk0 = blk * RES_BLOCK;
-    float R[8];
-    residual8(rowp, dt, V, lse, blk0 + lane * 8, blk0, cand_id, cand_mass, K, R);
-    float t = 0.f;
+  // pass 1: block sums, blocks interleaved over warps, the logits of RES_FLIGHT blocks on their
+  // way at once (one at a time, the walk of a 126464-entry row waited 31 times for memory:
+  // a call waits for memory most of the time)
+  const int nw = (int)(blockDim.x >> 5);
+  for (int base = warp; base < nblk; base += RES_FLIGHT * nw) {
+    float l[RES_FLIGHT][8];
 #pragma unroll
-    for (int e = 0; e < 8; ++e) t += R[e];
-    t = warp_sum(t);
-    if (lane == 0) sm.bsum[blk] = t;
+    for (int u = 0; u < RES_FLIGHT; ++u)   // (a block past the row reads as -inf)
+      logits8(rowp, dt, V, (base + u * nw) * RES_BLOCK + lane * 8, l[u]);
+#pragma unroll
+    for (int u = 0; u < RES_FLIGHT; ++u) {
+      const int blk = base + u * nw, blk0 = blk * RES_BLOCK;
+      if (blk >= nblk) break;
+      float R[8];
+      residual8(l[u], lse, blk0 + lane * 8, blk0, cand_id, cand_mass, K, R);
+      float t = 0.f;
+#pragma unroll
+      for (int e = 0; e < 8; ++e) t += R[e];
+      t = warp_sum(t);
+      if (lane == 0) sm.bsum[blk] = t;
+    }
   }
   __syncthreads();
   // warp 0: total mass and the block holding the target
@@ -244,8 +259,9 @@ __device__ int residual_sample(const Smem& sm, const void* rowp, int dt, int V, 
   // warp 0 walks the block: lane prefix sums, then the lane's 8 ids in order
   if (warp == 0) {
     const int blk0 = blk * RES_BLOCK;
-    float R[8];
-    residual8(rowp, dt, V, lse, blk0 + lane * 8, blk0, cand_id, cand_mass, K, R);
+    float l[8], R[8];
+    logits8(rowp, dt, V, blk0 + lane * 8, l);
+    residual8(l, lse, blk0 + lane * 8, blk0, cand_id, cand_mass, K, R);
     float mine = 0.f;
 #pragma unroll
     for (int e = 0; e < 8; ++e) mine += R[e];
