@@ -196,17 +196,18 @@ brisk_status hidden_products(const brisk_dims* d, const brisk_params* p, const v
     __nv_bfloat16* Hs = at<__nv_bfloat16>(ws, w.Hm);   // [BL + B, 3r]: hi | mid | lo
     const int r3 = 3 * r;
     const bool share = wide && S <= 512;   // tiles that fit the sweep's carveout
+    const int carveout = share ? CARVEOUT_SMALL_KB : CARVEOUT_GEMM_KB;
     const int bn = wide && !share ? 256 : 64;
     const TcSpec first[2] = {
         {BL, r, d->d, hidden, d->d, p->P_h, d->d, 1, Hs, r3, nullptr, 0, bn},
         {d->B, r, d->d, h_ctx, d->d, p->P_h, d->d, 1, Hs + (size_t)BL * r3, r3, nullptr, 0, bn}};
-    BRISK_CUDA(gemm_tc_grouped(first, 2, status, st, wide ? 2 : 4, share));
+    BRISK_CUDA(gemm_tc_grouped(first, 2, status, st, wide ? 2 : 4, carveout));
     const TcSpec second[2] = {
         {BL, 2 * S, r3, Hs, r3, at<__nv_bfloat16>(tables, t.W2s), r3, 0, at<float>(ws, w.G), 2 * S,
          at<float>(tables, t.posG), d->L, share ? 64 : 0},
         {d->B, S, r3, Hs + (size_t)BL * r3, r3, at<__nv_bfloat16>(tables, t.W0s), r3, 0,
          at<float>(ws, w.G0), S, nullptr, 0, share ? 64 : 0}};
-    BRISK_CUDA(gemm_tc_grouped(second, 2, status, st, 2, share));
+    BRISK_CUDA(gemm_tc_grouped(second, 2, status, st, 2, carveout));
     return BRISK_OK;
   }
   float* Hm = at<float>(ws, w.Hm);
@@ -356,6 +357,18 @@ brisk_status brisk_corrector_prepare(const brisk_dims* d, const brisk_params* p,
   float* Tin = at<float>(tables, t.Tin);
   float* Tout = at<float>(tables, t.Tout);
   float* Tzh = at<float>(tables, t.Tzh);
+  // everything that depends on the corrector's weights alone
+  PackArgs pk{};
+  pk.L = L; pk.r = r; pk.dt = hd;
+  pk.Wz = p->Wz; pk.Wh = p->Wh; pk.W0 = p->W0; pk.W_s = p->W_s; pk.w_g = p->w_g;
+  pk.pos = p->pos; pk.P_phi = p->P_phi;
+  pk.W2 = at<float>(tables, t.W2); pk.W0h = at<float>(tables, t.W0h);
+  pk.wg = at<float>(tables, t.wg); pk.posG = at<float>(tables, t.posG);
+  pk.Fz = at<float>(tables, t.Fz); pk.Fh = at<float>(tables, t.Fh);
+  pk.W2s = at<__nv_bfloat16>(tables, t.W2s); pk.W0s = at<__nv_bfloat16>(tables, t.W0s);
+  pk.Wt2s = at<__nv_bfloat16>(tables, t.Wt2s); pk.W0ts = at<__nv_bfloat16>(tables, t.W0ts);
+  pk.Ws3 = at<__nv_bfloat16>(tables, t.Ws3);
+  BRISK_CUDA(pack_weights(pk, st));
   if (hd == BRISK_DT_BF16 && gemm_tc_supported(p->E_in, d->d, p->P_e, d->d, d->d) &&
       gemm_tc_supported(p->E_out, d->d, p->W_c, d->d, d->d)) {
     // On the tensor cores. P_e E_in(v) (then W_c E_out(v)) is written as three bf16 parts
@@ -363,23 +376,20 @@ brisk_status brisk_corrector_prepare(const brisk_dims* d, const brisk_params* p,
     // products multiply the parts by the weight blocks written three times along k, which keeps
     // fp32-level accuracy on bf16 tensor cores. No status word: a bounded wait that gives up
     // here (about 2 s at the default limit) leaves the tables undefined.
-    const int BF = BRISK_DT_BF16, r3 = 3 * r;
+    const int r3 = 3 * r;
     __nv_bfloat16* Wt2s = at<__nv_bfloat16>(tables, t.Wt2s);
     __nv_bfloat16* W0ts = at<__nv_bfloat16>(tables, t.W0ts);
     __nv_bfloat16* Ws3 = at<__nv_bfloat16>(tables, t.Ws3);
-    for (int part = 0; part < 3; ++part) {
-      BRISK_CUDA(copy2d(S, r, wp(p->Wz, r), hd, ldw, Wt2s + part * r, BF, r3, st));
-      BRISK_CUDA(copy2d(S, r, wp(p->Wh, r), hd, ldw, Wt2s + (size_t)S * r3 + part * r, BF, r3, st));
-      BRISK_CUDA(copy2d(S, r, wp(p->W0, r), hd, 2 * r, W0ts + part * r, BF, r3, st));
-      BRISK_CUDA(copy2d(S, r, p->W_s, hd, S, Ws3 + part * r, BF, r3, st, true));   // W_s^T
-    }
     __nv_bfloat16* X3 = at<__nv_bfloat16>(tables, t.Tin);   // [V, 3r] in the Tin and Tout space
-    BRISK_CUDA(gemm_tc(V, r, d->d, p->E_in, d->d, p->P_e, d->d, 1, X3, r3, nullptr, st));
+    const TcSpec ein{V, r, d->d, p->E_in, d->d, p->P_e, d->d, 1, X3, r3, nullptr, 0, 0};
     const TcSpec tok[2] = {{V, 2 * S, r3, X3, r3, Wt2s, r3, 0, Tzh, 2 * S, nullptr, 0, 0},
                            {V, S, r3, X3, r3, W0ts, r3, 0, at<float>(tables, t.T0), S, nullptr, 0, 0}};
-    BRISK_CUDA(gemm_tc_grouped(tok, 2, nullptr, st, 4));
-    BRISK_CUDA(gemm_tc(V, r, d->d, p->E_out, d->d, p->W_c, d->d, 1, X3, r3, nullptr, st));
-    BRISK_CUDA(gemm_tc(V, S, r3, X3, r3, Ws3, r3, 0, at<float>(tables, t.U), S, nullptr, st));
+    const TcSpec eout{V, r, d->d, p->E_out, d->d, p->W_c, d->d, 1, X3, r3, nullptr, 0, 0};
+    const TcSpec res{V, S, r3, X3, r3, Ws3, r3, 0, at<float>(tables, t.U), S, nullptr, 0, 0};
+    BRISK_CUDA(gemm_tc_grouped(&ein, 1, nullptr, st, 2, CARVEOUT_FULL_KB));
+    BRISK_CUDA(gemm_tc_grouped(tok, 2, nullptr, st, 2, CARVEOUT_FULL_KB));
+    BRISK_CUDA(gemm_tc_grouped(&eout, 1, nullptr, st, 2, CARVEOUT_FULL_KB));
+    BRISK_CUDA(gemm_tc_grouped(&res, 1, nullptr, st, 2, CARVEOUT_FULL_KB));
   } else {
     // P_e E_in(v) and W_c E_out(v) for every v
     BRISK_CUDA(gemm_simt(V, r, d->d, p->E_in, hd, d->d, p->P_e, hd, d->d, false, Tin, r, st));
@@ -391,31 +401,6 @@ brisk_status brisk_corrector_prepare(const brisk_dims* d, const brisk_params* p,
                          at<float>(tables, t.T0), S, st));
     // residual rows U(v) = W_s^T (W_c E_out(v)): B(n=j, k=t) = W_s[t, j]
     BRISK_CUDA(gemm_simt(V, S, r, Tout, F32, r, p->W_s, hd, S, true, at<float>(tables, t.U), S, st));
-  }
-  // position shares
-  BRISK_CUDA(gemm_simt(L, S, 16, p->pos, hd, 16, wp(p->Wz, 2 * r), hd, ldw, false,
-                       at<float>(tables, t.posG), 2 * S, st));
-  BRISK_CUDA(gemm_simt(L, S, 16, p->pos, hd, 16, wp(p->Wh, 2 * r), hd, ldw, false,
-                       at<float>(tables, t.posG) + S, 2 * S, st));
-  // feature shares: F(j, f) = sum_t W[j, 2r+16+t] P_phi[t, f]
-  BRISK_CUDA(gemm_simt(S, 5, 16, wp(p->Wz, 2 * r + 16), hd, ldw, p->P_phi, hd, 5, true,
-                       at<float>(tables, t.Fz), 5, st));
-  BRISK_CUDA(gemm_simt(S, 5, 16, wp(p->Wh, 2 * r + 16), hd, ldw, p->P_phi, hd, 5, true,
-                       at<float>(tables, t.Fh), 5, st));
-  // fp32 copies of the gate weights and of the hidden-state blocks
-  BRISK_CUDA(copy2d(1, S + 5, p->w_g, hd, S + 5, at<float>(tables, t.wg), F32, S + 5, st));
-  BRISK_CUDA(copy2d(S, r, p->Wz, hd, ldw, at<float>(tables, t.W2), F32, r, st));
-  BRISK_CUDA(copy2d(S, r, p->Wh, hd, ldw, at<float>(tables, t.W2) + (size_t)S * r, F32, r, st));
-  BRISK_CUDA(copy2d(S, r, p->W0, hd, 2 * r, at<float>(tables, t.W0h), F32, r, st));
-  if (hd == BRISK_DT_BF16) {
-    const int BF = BRISK_DT_BF16;
-    __nv_bfloat16* W2s = at<__nv_bfloat16>(tables, t.W2s);
-    __nv_bfloat16* W0s = at<__nv_bfloat16>(tables, t.W0s);
-    for (int part = 0; part < 3; ++part) {
-      BRISK_CUDA(copy2d(S, r, p->Wz, hd, ldw, W2s + part * r, BF, 3 * r, st));
-      BRISK_CUDA(copy2d(S, r, p->Wh, hd, ldw, W2s + (size_t)S * 3 * r + part * r, BF, 3 * r, st));
-      BRISK_CUDA(copy2d(S, r, p->W0, hd, 2 * r, W0s + part * r, BF, 3 * r, st));
-    }
   }
   return BRISK_OK;
 }

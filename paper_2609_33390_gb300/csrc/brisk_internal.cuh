@@ -151,7 +151,8 @@ __device__ __forceinline__ void warp_lse_combine(float& m, float& s) {
 // the corrector) must leave room in its split for the other's CTAs. Everything not carved out
 // is L1, which holds the sweep's loads in flight: the sweep is fastest with a small split.
 constexpr int CARVEOUT_SMALL_KB = 64;    // sweep (2 KB a CTA), corrector, verification
-constexpr int CARVEOUT_GEMM_KB = 132;    // a dense-product CTA (up to 97 KB) beside six sweep CTAs
+constexpr int CARVEOUT_GEMM_KB = 132;    // a dense-product CTA (up to 97 KB) beside sweep CTAs
+constexpr int CARVEOUT_FULL_KB = 228;    // all of it: two dense-product CTAs
 
 // Sets the carveout preference of `func` on the current device once (kernels of the same
 // signature are distinct entries: the registry is keyed by the function's address).
@@ -326,8 +327,6 @@ cudaError_t gemm_simt(int M, int N, int K, const void* A, int a_dt, int lda, con
 // Tensor-core product on sm_103a: C = A B^T with A [M, K] and B [N, K] bf16 (row strides lda, ldb),
 // fp32 accumulation; mode 0 stores fp32 C[m*ldc + n], mode 1 stores three bf16 parts whose sum
 // is c to about 2^-24 relative (hi at [m*ldc + n], mid at [m*ldc + N + n], lo at [m*ldc + 2N + n]).
-cudaError_t gemm_tc(int M, int N, int K, const void* A, int lda, const void* B, int ldb, int mode,
-                    void* C, int ldc, int32_t* status, cudaStream_t stream);
 // Up to two independent products of the same kind in one launch.
 struct TcSpec {
   int M, N, K;
@@ -344,17 +343,23 @@ struct TcSpec {
   // and a smaller pipeline stage. Read from the first product of a grouped launch.
   int max_bn;
 };
-// `stages` (2 or 4) sets the shared-memory pipeline depth: 2 leaves room on each SM for other
-// kernels running concurrently.
-// small_carveout: the kernel (a separate instantiation) prefers the small shared-memory
-// carveout of the sweep, so that its CTAs can share SMs with sweep CTAs; the tiles must then fit
-// it (64-wide, two stages: 49 KB).
+// `stages` (2 or 4) sets the shared-memory pipeline depth. carveout_kb is the shared-memory
+// carveout to prefer: CARVEOUT_GEMM_KB; with two stages also CARVEOUT_SMALL_KB, the sweep's, so
+// that CTAs can share SMs with sweep CTAs (the tiles must then fit it: 64-wide, 49 KB), or
+// CARVEOUT_FULL_KB, so that two CTAs of 256-wide tiles (97 KB) share an SM and one multiplies
+// while the other stores.
 cudaError_t gemm_tc_grouped(const TcSpec* spec, int nprob, int32_t* status, cudaStream_t stream,
-                            int stages, bool small_carveout = false);
+                            int stages, int carveout_kb = CARVEOUT_GEMM_KB);
 bool gemm_tc_supported(const void* A, int lda, const void* B, int ldb, int K);
-// dst[i*ldd + j] = (dst type) src[i*lds + j], i < rows, j < cols (src[j*lds + i] with transpose).
-cudaError_t copy2d(int rows, int cols, const void* src, int s_dt, int lds, void* dst, int d_dt,
-                   int ldd, cudaStream_t stream, bool transpose = false);
+// The folds that read the corrector's weights alone, in one launch: see brisk_corrector_prepare.
+struct PackArgs {
+  int L, r, dt;                  // dt: brisk_dtype of the weights
+  const void *Wz, *Wh, *W0, *W_s, *w_g, *pos, *P_phi;
+  float *W2, *W0h, *wg, *posG, *Fz, *Fh;
+  // bf16 blocks written three times along k (bf16 weights only)
+  __nv_bfloat16 *W2s, *W0s, *Wt2s, *W0ts, *Ws3;
+};
+cudaError_t pack_weights(const PackArgs& a, cudaStream_t stream);
 
 // ---------------------------------------------------------------- corrector scan and verify
 struct ScanArgs {

@@ -1,6 +1,6 @@
-// Tiled fp32 dense products and a conversion copy. They serve the fp32 configurations (the
+// Tiled fp32 dense products and the folds of the corrector's own weights. They serve the fp32 configurations (the
 // hidden products of a call and the one-off folds of the frozen vocabulary rows, App. C.3) and
-// the small folds of every configuration; every product accumulates in fp32.
+// the token folds' fallback; every product accumulates in fp32.
 #include "brisk_internal.cuh"
 
 namespace brisk {
@@ -190,17 +190,63 @@ gemm_simt_kernel(const __grid_constant__ SimtProblem P) {
   cluster_sync();   // the other CTAs have read this one's part
 }
 
-template <typename TS, typename TD>
-__global__ void copy2d_kernel(int rows, int cols, const TS* __restrict__ src, int lds,
-                              TD* __restrict__ dst, int ldd, int transpose) {
-  const long long n = (long long)rows * cols;
-  for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < n;
-       e += (long long)gridDim.x * blockDim.x) {
-    const long long i = e / cols, j = e % cols;
-    const float v = to_f32(transpose ? src[j * lds + i] : src[i * lds + j]);
-    if constexpr (sizeof(TD) == 4) dst[i * ldd + j] = v;
-    else dst[i * ldd + j] = __float2bfloat16_rn(v);
+// One thread an item: the weight blocks' element (j, t) in every form the products read, then the
+// position shares, the feature shares and the gate weights (each a sum of 16 products in order).
+// Bound by launches when done block by block: 29 launches took about 100 us.
+template <typename T>
+__global__ void __launch_bounds__(256) pack_kernel(const __grid_constant__ PackArgs a) {
+  const int r = a.r, S = 2 * r, ldw = 2 * r + 32;
+  const T *Wz = static_cast<const T*>(a.Wz), *Wh = static_cast<const T*>(a.Wh),
+          *W0 = static_cast<const T*>(a.W0), *Ws = static_cast<const T*>(a.W_s),
+          *pos = static_cast<const T*>(a.pos), *Pp = static_cast<const T*>(a.P_phi);
+  long long e = blockIdx.x * 256ll + threadIdx.x;
+  if (e < (long long)S * r) {
+    const int j = (int)(e / r), t = (int)(e % r);
+    const T z = Wz[(size_t)j * ldw + t], h = Wh[(size_t)j * ldw + t], i = W0[(size_t)j * S + t];
+    const size_t at = (size_t)j * r + t, lower = (size_t)S * r + at;
+    a.W2[at] = to_f32(z);
+    a.W2[lower] = to_f32(h);
+    a.W0h[at] = to_f32(i);
+    if constexpr (sizeof(T) == 2) {
+      const T tz = Wz[(size_t)j * ldw + r + t], th = Wh[(size_t)j * ldw + r + t],
+              ti = W0[(size_t)j * S + r + t], ws = Ws[(size_t)t * S + j];
+#pragma unroll
+      for (int part = 0; part < 3; ++part) {
+        const size_t up = (size_t)j * 3 * r + part * r + t, lo = (size_t)S * 3 * r + up;
+        a.W2s[up] = z;
+        a.W2s[lo] = h;
+        a.W0s[up] = i;
+        a.Wt2s[up] = tz;
+        a.Wt2s[lo] = th;
+        a.W0ts[up] = ti;
+        a.Ws3[up] = ws;
+      }
+    }
+    return;
   }
+  e -= (long long)S * r;
+  auto dot16 = [](auto x, auto y) {
+    float acc = 0.f;
+    for (int t = 0; t < 16; ++t) acc = fmaf(x(t), y(t), acc);
+    return acc;
+  };
+  if (e < (long long)a.L * 2 * S) {        // posG(i, j) = W_{z,h}[j, 2r : 2r + 16] . pos_i
+    const int i = (int)(e / (2 * S)), j = (int)(e % (2 * S));
+    const T* w = (j < S ? Wz + (size_t)j * ldw : Wh + (size_t)(j - S) * ldw) + 2 * r;
+    a.posG[e] = dot16([&](int t) { return to_f32(pos[i * 16 + t]); },
+                      [&](int t) { return to_f32(w[t]); });
+    return;
+  }
+  e -= (long long)a.L * 2 * S;
+  if (e < 10ll * S) {                       // F(j, f) = sum_t W[j, 2r + 16 + t] P_phi[t, f]
+    const int half = (int)(e / (5 * S)), q = (int)(e % (5 * S)), j = q / 5, f = q % 5;
+    const T* w = (half ? Wh : Wz) + (size_t)j * ldw + 2 * r + 16;
+    (half ? a.Fh : a.Fz)[q] = dot16([&](int t) { return to_f32(w[t]); },
+                                    [&](int t) { return to_f32(Pp[t * 5 + f]); });
+    return;
+  }
+  e -= 10ll * S;
+  if (e < S + 5) a.wg[e] = to_f32(static_cast<const T*>(a.w_g)[e]);
 }
 
 template <typename TA, typename TB>
@@ -223,21 +269,6 @@ cudaError_t gemm_t(int M, int N, int K, const void* A, int lda, const void* B, i
   return e != cudaSuccess ? e : cudaGetLastError();
 }
 
-template <typename TS>
-cudaError_t copy_t(int rows, int cols, const void* src, int lds, void* dst, int d_dt, int ldd,
-                   bool transpose, cudaStream_t stream) {
-  const long long n = (long long)rows * cols;
-  const unsigned grid = (unsigned)((n + 255) / 256 > 4096 ? 4096 : (n + 255) / 256);
-  if (d_dt == BRISK_DT_F32)
-    copy2d_kernel<TS, float><<<grid, 256, 0, stream>>>(rows, cols, static_cast<const TS*>(src), lds,
-                                                       static_cast<float*>(dst), ldd, transpose);
-  else
-    copy2d_kernel<TS, __nv_bfloat16><<<grid, 256, 0, stream>>>(
-        rows, cols, static_cast<const TS*>(src), lds, static_cast<__nv_bfloat16*>(dst), ldd,
-        transpose);
-  return cudaGetLastError();
-}
-
 }  // namespace
 
 cudaError_t gemm_simt(int M, int N, int K, const void* A, int a_dt, int lda, const void* B,
@@ -257,12 +288,12 @@ cudaError_t gemm_simt(int M, int N, int K, const void* A, int a_dt, int lda, con
                                                 bias, bias_period);
 }
 
-cudaError_t copy2d(int rows, int cols, const void* src, int s_dt, int lds, void* dst, int d_dt,
-                   int ldd, cudaStream_t stream, bool transpose) {
-  if (rows <= 0 || cols <= 0) return cudaSuccess;
-  if (s_dt == BRISK_DT_BF16)
-    return copy_t<__nv_bfloat16>(rows, cols, src, lds, dst, d_dt, ldd, transpose, stream);
-  return copy_t<float>(rows, cols, src, lds, dst, d_dt, ldd, transpose, stream);
+cudaError_t pack_weights(const PackArgs& a, cudaStream_t stream) {
+  const long long S = 2ll * a.r, items = S * a.r + a.L * 2 * S + 10 * S + S + 5;
+  const unsigned grid = (unsigned)((items + 255) / 256);
+  if (a.dt == BRISK_DT_BF16) pack_kernel<__nv_bfloat16><<<grid, 256, 0, stream>>>(a);
+  else pack_kernel<float><<<grid, 256, 0, stream>>>(a);
+  return cudaGetLastError();
 }
 
 }  // namespace brisk

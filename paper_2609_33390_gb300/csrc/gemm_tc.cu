@@ -192,9 +192,9 @@ constexpr int TC_SPLIT_TILES = 76;               // tiles up to which K is split
 constexpr int TC_SPLIT_CTAS = 152;               // CTAs a split aims for: one an SM
 constexpr int TC_PART_LD = TC_SPLIT_BN + 4;      // row stride of a part in shared memory (floats)
 
-// SMALL_CARVEOUT does not change the code: it makes a separate kernel whose shared-memory
-// carveout preference (a per-kernel attribute) is the sweep's.
-template <int TC_STAGES, bool SMALL_CARVEOUT = false>
+// CARVEOUT_KB does not change the code: it makes a separate kernel with a shared-memory carveout
+// preference (a per-kernel attribute) of its own.
+template <int TC_STAGES, int CARVEOUT_KB>
 __global__ void __launch_bounds__(TC_THREADS, 1)
 gemm_tc_kernel(const __grid_constant__ TcMaps maps, const __grid_constant__ TcArgs a) {
   extern __shared__ __align__(1024) uint8_t smem_raw[];
@@ -218,7 +218,8 @@ gemm_tc_kernel(const __grid_constant__ TcMaps maps, const __grid_constant__ TcAr
   const CUtensorMap* tmA = &maps.a[pi];
   const CUtensorMap* tmB = &maps.b[pi];
   const int tile = t - (pi ? a.tiles0 : 0);
-  const int m0 = (tile % P.mtiles) * TC_BM, n0 = (tile / P.mtiles) * a.BN;
+  // column tiles first: the tiles that share rows of A run together and read them from L2
+  const int m0 = (tile / P.ntiles) * TC_BM, n0 = (tile % P.ntiles) * a.BN;
   // this CTA's K steps [kfirst, kfirst + nk) (with split > 1 every part has at least one)
   const int nk_all = (P.K + TC_BK - 1) / TC_BK;
   const int kfirst = (int)((long long)nk_all * krank / a.split);
@@ -490,9 +491,9 @@ bool gemm_tc_supported(const void* A, int lda, const void* B, int ldb, int K) {
 // One or two products C = A B^T, A [M, K] (row stride lda) and B [N, K] (row stride ldb) bf16,
 // fp32 accumulation, in one launch.
 cudaError_t gemm_tc_grouped(const TcSpec* spec, int nprob, int32_t* status, cudaStream_t stream,
-                            int stages, bool small_carveout) {
+                            int stages, int carveout_kb) {
   if (nprob < 1 || nprob > 2 || (stages != 2 && stages != 4)) return cudaErrorInvalidValue;
-  if (small_carveout && stages != 2) return cudaErrorInvalidValue;
+  if (carveout_kb != CARVEOUT_GEMM_KB && stages != 2) return cudaErrorInvalidValue;
   int nmax = 0;
   for (int i = 0; i < nprob; ++i) nmax = spec[i].N > nmax ? spec[i].N : nmax;
   // Few tiles: split K. The rule looks at the products alone, so a product is summed in the same
@@ -511,7 +512,7 @@ cudaError_t gemm_tc_grouped(const TcSpec* spec, int nprob, int32_t* status, cuda
   if (split > 1) {
     max_bn = TC_SPLIT_BN;
     stages = 4;
-    small_carveout = false;
+    carveout_kb = CARVEOUT_GEMM_KB;
   }
   if (max_bn >= 16 && nmax > max_bn) nmax = max_bn;
   const int BN = tc_bn(nmax);
@@ -552,23 +553,19 @@ cudaError_t gemm_tc_grouped(const TcSpec* spec, int nprob, int32_t* status, cuda
   }
   if (total == 0) return cudaSuccess;
   const size_t smem = gemm_tc_smem(BN, stages);
-  if (small_carveout && smem > (size_t)(CARVEOUT_SMALL_KB - 1) * 1024) return cudaErrorInvalidValue;
-  auto kernel = small_carveout ? gemm_tc_kernel<2, true>
-                               : (stages == 2 ? gemm_tc_kernel<2> : gemm_tc_kernel<4>);
+  if (smem > (size_t)(carveout_kb - 1) * 1024 && carveout_kb == CARVEOUT_SMALL_KB)
+    return cudaErrorInvalidValue;
+  auto kernel = carveout_kb == CARVEOUT_SMALL_KB  ? gemm_tc_kernel<2, CARVEOUT_SMALL_KB>
+                : carveout_kb == CARVEOUT_FULL_KB ? gemm_tc_kernel<2, CARVEOUT_FULL_KB>
+                : stages == 2                     ? gemm_tc_kernel<2, CARVEOUT_GEMM_KB>
+                                                  : gemm_tc_kernel<4, CARVEOUT_GEMM_KB>;
   cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        static_cast<int>(smem));
-  if (e == cudaSuccess) e = prefer_carveout(kernel, small_carveout ? CARVEOUT_SMALL_KB : CARVEOUT_GEMM_KB);
+  if (e == cudaSuccess) e = prefer_carveout(kernel, carveout_kb);
   if (e != cudaSuccess) return e;
   e = launch_cluster(kernel, dim3(total * split), dim3(TC_THREADS), smem, stream, split, maps, a);
   if (e != cudaSuccess) return e;
   return cudaGetLastError();
-}
-
-cudaError_t gemm_tc(int M, int N, int K, const void* A, int lda, const void* B, int ldb, int mode,
-                    void* C, int ldc, int32_t* status, cudaStream_t stream) {
-  if (M <= 0 || N <= 0) return cudaSuccess;
-  const TcSpec s{M, N, K, A, lda, B, ldb, mode, C, ldc, nullptr, 0, 0};
-  return gemm_tc_grouped(&s, 1, status, stream, 4);
 }
 
 }  // namespace brisk
