@@ -36,6 +36,7 @@ enum TailSchedule { SCHEDULE_OVERLAP = 0, SCHEDULE_SEPARATE = 1, SCHEDULE_FUSED 
 // us fused; 16 sequences (259 MB, stochastic) 188.9 / 175.2 us separate, 243.6 / 210.6 fused.
 constexpr size_t FUSE_MAX_BYTES = size_t(64) << 20;
 constexpr size_t OVERLAP_ROWS = 2432;      // proposal rows from which the sweeps overlap
+constexpr int BESIDE_STATE = 512;          // state width up to which the products share SMs with them
 constexpr size_t OVERLAP_VECTORS = 2048;   // 16-byte vectors a row below which they do
 
 struct WsLayout {
@@ -175,19 +176,9 @@ SweepSeg make_seg(const WsLayout& w, void* ws, int seg, const void* logits, int 
 // G = Hm[:BL] [W_z[:, :r] ; W_h[:, :r]]^T and G0 = Hm[BL:] W0[:, :r]^T. With bf16 weights the
 // products run on the tensor cores: the first one writes Hm as three bf16 parts, which the
 // second one multiplies by the weight blocks written three times along k (fp32-level accuracy).
-// The first product (k = d long) has few 128-row tiles for small batches: there it uses 64-wide
-// column tiles and a 4-deep pipeline (four times the CTAs, each streaming a quarter of the
-// weights). With `wide` (large batches, the products running beside the proposal sweep) it uses
-// 256-wide tiles and a 2-deep pipeline: a quarter of the CTAs, so the sweep waits for fewer SMs,
-// and the hidden states are read once; or, where the second product is small (S <= 512), both
-// products in 64-wide tiles and a 2-deep pipeline that fit the sweep's shared-memory carveout,
-// so that their CTAs share SMs with sweep CTAs instead of holding SMs of their own (decode_stream
-// 395 -> 392 us a step; large_vocab's four times larger second product: 561 -> 601 us, not
-// used there). Tile width does not change any product's summation order, so all give the same
-// bits.
 brisk_status hidden_products(const brisk_dims* d, const brisk_params* p, const void* tables,
                              const void* hidden, const void* h_ctx, const WsLayout& w, void* ws,
-                             cudaStream_t st, bool wide) {
+                             cudaStream_t st, bool beside = false) {
   const TbLayout t = tb_layout(d);
   const int BL = d->B * d->L, r = d->r, S = 2 * d->r, hd = d->hidden_dtype;
   int32_t* status = at<int32_t>(ws, w.status);
@@ -195,19 +186,16 @@ brisk_status hidden_products(const brisk_dims* d, const brisk_params* p, const v
       aligned(h_ctx, 16)) {
     __nv_bfloat16* Hs = at<__nv_bfloat16>(ws, w.Hm);   // [BL + B, 3r]: hi | mid | lo
     const int r3 = 3 * r;
-    const bool share = wide && S <= 512;   // tiles that fit the sweep's carveout
-    const int carveout = share ? CARVEOUT_SMALL_KB : CARVEOUT_GEMM_KB;
-    const int bn = wide && !share ? 256 : 64;
     const TcSpec first[2] = {
-        {BL, r, d->d, hidden, d->d, p->P_h, d->d, 1, Hs, r3, nullptr, 0, bn},
-        {d->B, r, d->d, h_ctx, d->d, p->P_h, d->d, 1, Hs + (size_t)BL * r3, r3, nullptr, 0, bn}};
-    BRISK_CUDA(gemm_tc_grouped(first, 2, status, st, wide ? 2 : 4, carveout));
+        {BL, r, d->d, hidden, d->d, p->P_h, d->d, 1, Hs, r3, nullptr, 0},
+        {d->B, r, d->d, h_ctx, d->d, p->P_h, d->d, 1, Hs + (size_t)BL * r3, r3, nullptr, 0}};
+    BRISK_CUDA(gemm_tc_grouped(first, 2, status, st, beside));
     const TcSpec second[2] = {
         {BL, 2 * S, r3, Hs, r3, at<__nv_bfloat16>(tables, t.W2s), r3, 0, at<float>(ws, w.G), 2 * S,
-         at<float>(tables, t.posG), d->L, share ? 64 : 0},
+         at<float>(tables, t.posG), d->L},
         {d->B, S, r3, Hs + (size_t)BL * r3, r3, at<__nv_bfloat16>(tables, t.W0s), r3, 0,
-         at<float>(ws, w.G0), S, nullptr, 0, share ? 64 : 0}};
-    BRISK_CUDA(gemm_tc_grouped(second, 2, status, st, 2, carveout));
+         at<float>(ws, w.G0), S, nullptr, 0}};
+    BRISK_CUDA(gemm_tc_grouped(second, 2, status, st, beside));
     return BRISK_OK;
   }
   float* Hm = at<float>(ws, w.Hm);
@@ -381,15 +369,15 @@ brisk_status brisk_corrector_prepare(const brisk_dims* d, const brisk_params* p,
     __nv_bfloat16* W0ts = at<__nv_bfloat16>(tables, t.W0ts);
     __nv_bfloat16* Ws3 = at<__nv_bfloat16>(tables, t.Ws3);
     __nv_bfloat16* X3 = at<__nv_bfloat16>(tables, t.Tin);   // [V, 3r] in the Tin and Tout space
-    const TcSpec ein{V, r, d->d, p->E_in, d->d, p->P_e, d->d, 1, X3, r3, nullptr, 0, 0};
-    const TcSpec tok[2] = {{V, 2 * S, r3, X3, r3, Wt2s, r3, 0, Tzh, 2 * S, nullptr, 0, 0},
-                           {V, S, r3, X3, r3, W0ts, r3, 0, at<float>(tables, t.T0), S, nullptr, 0, 0}};
-    const TcSpec eout{V, r, d->d, p->E_out, d->d, p->W_c, d->d, 1, X3, r3, nullptr, 0, 0};
-    const TcSpec res{V, S, r3, X3, r3, Ws3, r3, 0, at<float>(tables, t.U), S, nullptr, 0, 0};
-    BRISK_CUDA(gemm_tc_grouped(&ein, 1, nullptr, st, 2, CARVEOUT_FULL_KB));
-    BRISK_CUDA(gemm_tc_grouped(tok, 2, nullptr, st, 2, CARVEOUT_FULL_KB));
-    BRISK_CUDA(gemm_tc_grouped(&eout, 1, nullptr, st, 2, CARVEOUT_FULL_KB));
-    BRISK_CUDA(gemm_tc_grouped(&res, 1, nullptr, st, 2, CARVEOUT_FULL_KB));
+    const TcSpec ein{V, r, d->d, p->E_in, d->d, p->P_e, d->d, 1, X3, r3, nullptr, 0};
+    const TcSpec tok[2] = {{V, 2 * S, r3, X3, r3, Wt2s, r3, 0, Tzh, 2 * S, nullptr, 0},
+                           {V, S, r3, X3, r3, W0ts, r3, 0, at<float>(tables, t.T0), S, nullptr, 0}};
+    const TcSpec eout{V, r, d->d, p->E_out, d->d, p->W_c, d->d, 1, X3, r3, nullptr, 0};
+    const TcSpec res{V, S, r3, X3, r3, Ws3, r3, 0, at<float>(tables, t.U), S, nullptr, 0};
+    BRISK_CUDA(gemm_tc_grouped(&ein, 1, nullptr, st));
+    BRISK_CUDA(gemm_tc_grouped(tok, 2, nullptr, st));
+    BRISK_CUDA(gemm_tc_grouped(&eout, 1, nullptr, st));
+    BRISK_CUDA(gemm_tc_grouped(&res, 1, nullptr, st));
   } else {
     // P_e E_in(v) and W_c E_out(v) for every v
     BRISK_CUDA(gemm_simt(V, r, d->d, p->E_in, hd, d->d, p->P_e, hd, d->d, false, Tin, r, st));
@@ -443,7 +431,7 @@ brisk_status brisk_corrector_select(const brisk_dims* d, const brisk_params* p, 
   const WsLayout w = ws_layout(d);
   brisk_status s = clear_ws(w, d, ws, st);
   if (s != BRISK_OK) return s;
-  s = hidden_products(d, p, tables, hidden, h_ctx, w, ws, st, false);
+  s = hidden_products(d, p, tables, hidden, h_ctx, w, ws, st);
   if (s != BRISK_OK) return s;
   ScanArgs a = scan_args(d, p, tables, w, ws);
   a.select_mode = select_mode;
@@ -571,7 +559,8 @@ brisk_status brisk::decode_tail_locked(const brisk_dims* d, const brisk_params* 
   BRISK_CUDA(cudaStreamWaitEvent(ss->hi, ss->ev[0], 0));
   if (overlap) BRISK_CUDA(cudaStreamWaitEvent(m, ss->ev[0], 0));
   if (w.schedule != SCHEDULE_FUSED) BRISK_CUDA(cudaStreamWaitEvent(ss->lo, ss->ev[0], 0));
-  s = hidden_products(d, p, tables, io->hidden, io->h_ctx, w, ws, ss->hi, overlap);
+  s = hidden_products(d, p, tables, io->hidden, io->h_ctx, w, ws, ss->hi,
+                      overlap && 2 * d->r <= BESIDE_STATE);
   if (s != BRISK_OK) return s;
   BRISK_CUDA(cudaEventRecord(ss->ev[1], ss->hi));
 
@@ -755,7 +744,7 @@ brisk_status brisk_replay_diagnostics(const brisk_dims* d, const brisk_params* p
   if (!ss) return BRISK_ERR_CUDA;
   BRISK_CUDA(cudaEventRecord(ss->ev[0], st));
   BRISK_CUDA(cudaStreamWaitEvent(ss->hi, ss->ev[0], 0));
-  s = hidden_products(d, p, tables, hidden, h_ctx, w, ws, ss->hi, w.schedule == SCHEDULE_OVERLAP);
+  s = hidden_products(d, p, tables, hidden, h_ctx, w, ws, ss->hi);
   if (s != BRISK_OK) return s;
   BRISK_CUDA(cudaEventRecord(ss->ev[1], ss->hi));
   SweepLaunch sq{};

@@ -150,10 +150,8 @@ __device__ __forceinline__ void warp_lse_combine(float& m, float& s) {
 // runs beside another one (the sweep beside the dense products, the verifier-row sweep beside
 // the corrector) must leave room in its split for the other's CTAs. Everything not carved out
 // is L1, which holds the sweep's loads in flight: the sweep is fastest with a small split.
-constexpr int CARVEOUT_SMALL_KB = 64;    // sweep (2 KB a CTA), corrector, verification
-constexpr int CARVEOUT_GEMM_KB = 132;    // a dense-product CTA (up to 97 KB) beside sweep CTAs
-constexpr int CARVEOUT_FULL_KB = 228;    // all of it: two dense-product CTAs
-
+constexpr int CARVEOUT_SMALL_KB = 64;    // sweep (9 KB a CTA), corrector, verification
+constexpr int CARVEOUT_FULL_KB = 228;    // dense products, except beside the sweeps
 // Sets the carveout preference of `func` on the current device once (kernels of the same
 // signature are distinct entries: the registry is keyed by the function's address).
 inline cudaError_t prefer_carveout_fn(const void* func, int kb) {
@@ -339,17 +337,11 @@ struct TcSpec {
   int ldc;
   const float* bias;   // optional fp32 [bias_period, N] added to row m as bias[m % bias_period] (mode 0)
   int bias_period;
-  // Widest output tile (columns) to use, 0 for the default 256; narrower tiles give more CTAs
-  // and a smaller pipeline stage. Read from the first product of a grouped launch.
-  int max_bn;
 };
-// `stages` (2 or 4) sets the shared-memory pipeline depth. carveout_kb is the shared-memory
-// carveout to prefer: CARVEOUT_GEMM_KB; with two stages also CARVEOUT_SMALL_KB, the sweep's, so
-// that CTAs can share SMs with sweep CTAs (the tiles must then fit it: 64-wide, 49 KB), or
-// CARVEOUT_FULL_KB, so that two CTAs of 256-wide tiles (97 KB) share an SM and one multiplies
-// while the other stores.
+// beside: the products run beside the sweeps and should share SMs with them (the results are the
+// same bit for bit).
 cudaError_t gemm_tc_grouped(const TcSpec* spec, int nprob, int32_t* status, cudaStream_t stream,
-                            int stages, int carveout_kb = CARVEOUT_GEMM_KB);
+                            bool beside = false);
 bool gemm_tc_supported(const void* A, int lda, const void* B, int ldb, int K);
 // The folds that read the corrector's weights alone, in one launch: see brisk_corrector_prepare.
 struct PackArgs {

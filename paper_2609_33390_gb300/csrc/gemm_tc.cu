@@ -187,14 +187,14 @@ constexpr int TC_OUT_CHUNK_BF16X3 = 3 * TC_BM * 32 * 2;
 // Products with few tiles split K over a cluster: one CTA would walk the whole K alone (4096 in
 // 64 steps for the hidden states of one sequence) while most of the chip is idle.
 constexpr int TC_SPLIT_MAX = 8;
-constexpr int TC_SPLIT_BN = 64;                  // tile columns of a split product
-constexpr int TC_SPLIT_TILES = 76;               // tiles up to which K is split
-constexpr int TC_SPLIT_CTAS = 152;               // CTAs a split aims for: one an SM
-constexpr int TC_PART_LD = TC_SPLIT_BN + 4;      // row stride of a part in shared memory (floats)
+constexpr int TC_SPLIT_STEPS = 3;   // K steps a part has at least
+constexpr int TC_SPLIT_TILES = 24;   // 128 x 256 tiles up to which K is split
+constexpr int TC_SMS = 152;
+constexpr int TC_PART_PAD = 4;      // floats between the rows of a part in shared memory
 
-// CARVEOUT_KB does not change the code: it makes a separate kernel with a shared-memory carveout
-// preference (a per-kernel attribute) of its own.
-template <int TC_STAGES, int CARVEOUT_KB>
+// SMALL_CARVEOUT does not change the code: it makes a separate kernel whose shared-memory
+// carveout preference (a per-kernel attribute) is the sweep's.
+template <int TC_STAGES, bool SMALL_CARVEOUT = false>
 __global__ void __launch_bounds__(TC_THREADS, 1)
 gemm_tc_kernel(const __grid_constant__ TcMaps maps, const __grid_constant__ TcArgs a) {
   extern __shared__ __align__(1024) uint8_t smem_raw[];
@@ -308,7 +308,7 @@ gemm_tc_kernel(const __grid_constant__ TcMaps maps, const __grid_constant__ TcAr
   if (a.split > 1) {
     float* part = reinterpret_cast<float*>(base);    // the ring is free by then
     if (ok) {
-      float* mine = part + (size_t)threadIdx.x * TC_PART_LD;
+      float* mine = part + (size_t)threadIdx.x * (a.BN + TC_PART_PAD);
       for (int c = 0; c < a.BN; c += 32) {
         float v[32];
         tmem_ld32(tmem + (static_cast<uint32_t>(warp * 32) << 16) + c, v);
@@ -326,7 +326,7 @@ gemm_tc_kernel(const __grid_constant__ TcMaps maps, const __grid_constant__ TcAr
       for (int e = r0 * per_row + (int)threadIdx.x; e < r1 * per_row; e += TC_THREADS) {
         const int row = e / per_row, col = 4 * (e - row * per_row);
         if (n0 + col >= P.N) continue;               // N is a multiple of 16
-        const float* src = part + (size_t)row * TC_PART_LD + col;
+        const float* src = part + (size_t)row * (a.BN + TC_PART_PAD) + col;
         float4 v = ld_cluster(src, 0);
         for (int o = 1; o < a.split; ++o) {
           const float4 w = ld_cluster(src, o);
@@ -361,8 +361,17 @@ gemm_tc_kernel(const __grid_constant__ TcMaps maps, const __grid_constant__ TcAr
   if (ok && a.split == 1) {
     const uint32_t trow = tmem + (static_cast<uint32_t>(warp * 32) << 16);
     const int rt = warp * 32 + lane;                 // row within the tile
-    const int row = m0 + rt;
-    const float* brow = (P.bias && row < P.M) ? P.bias + (size_t)(row % P.bias_period) * P.N : nullptr;
+    const int sw = rt & 7, sw2 = (rt >> 1) & 3;      // the stages' swizzle of this row
+    // bias rows this lane adds, eight lanes a row: 32 warp + 4 it + lane / 8
+    const int bq = lane & 7;
+    const float* brow[8];
+    if (P.bias) {
+#pragma unroll
+      for (int it = 0; it < 8; ++it) {
+        const int m = m0 + warp * 32 + 4 * it + (lane >> 3);
+        brow[it] = P.bias + (size_t)(m % P.bias_period) * P.N;
+      }
+    }
     const int chunk_bytes = P.mode == 0 ? TC_OUT_CHUNK_F32 : TC_OUT_CHUNK_BF16X3;
     const int fit = ring / chunk_bytes;
     const int nbuf = fit >= 4 ? 4 : (fit >= 2 ? 2 : 1);
@@ -370,24 +379,24 @@ gemm_tc_kernel(const __grid_constant__ TcMaps maps, const __grid_constant__ TcAr
       float v[32];
       tmem_ld32(trow + c, v);
       const int nb = n0 + c;
-      if (brow) {
-#pragma unroll
-        for (int q = 0; q < 8; ++q)
-          if (nb + 4 * q + 3 < P.N) {
-            const float4 b = __ldg(reinterpret_cast<const float4*>(brow + nb) + q);
-            v[4 * q] += b.x; v[4 * q + 1] += b.y; v[4 * q + 2] += b.z; v[4 * q + 3] += b.w;
-          } else {
-            for (int e = 0; e < 4; ++e)
-              if (nb + 4 * q + e < P.N) v[4 * q + e] += brow[nb + 4 * q + e];
-          }
-      }
       uint8_t* stage = base + (ci % nbuf) * chunk_bytes;
       if (threadIdx.x == 0) bulk_wait_read(nbuf - 1);   // the store that last used `stage` has read it
       __syncthreads();
       if (P.mode == 0) {
         float4* st = reinterpret_cast<float4*>(stage + rt * 128);
 #pragma unroll
-        for (int q = 0; q < 8; ++q) st[q] = make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
+        for (int q = 0; q < 8; ++q)
+          st[q ^ sw] = make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
+        __syncwarp();
+        if (P.bias && nb + 4 * bq < P.N) {           // (N is a multiple of 4)
+#pragma unroll
+          for (int it = 0; it < 8; ++it) {
+            const int r = warp * 32 + 4 * it + (lane >> 3);
+            float4* at = reinterpret_cast<float4*>(stage + r * 128) + (bq ^ (r & 7));
+            const float4 w = __ldg(reinterpret_cast<const float4*>(brow[it] + nb) + bq), x = *at;
+            *at = make_float4(x.x + w.x, x.y + w.y, x.z + w.z, x.w + w.w);
+          }
+        }
       } else {
         __align__(16) __nv_bfloat16 hi[32], mid[32], lo[32];
 #pragma unroll
@@ -396,9 +405,9 @@ gemm_tc_kernel(const __grid_constant__ TcMaps maps, const __grid_constant__ TcAr
         }
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
-          reinterpret_cast<uint4*>(stage + rt * 64)[q] = reinterpret_cast<const uint4*>(hi)[q];
-          reinterpret_cast<uint4*>(stage + TC_BM * 64 + rt * 64)[q] = reinterpret_cast<const uint4*>(mid)[q];
-          reinterpret_cast<uint4*>(stage + 2 * TC_BM * 64 + rt * 64)[q] = reinterpret_cast<const uint4*>(lo)[q];
+          reinterpret_cast<uint4*>(stage + rt * 64)[q ^ sw2] = reinterpret_cast<const uint4*>(hi)[q];
+          reinterpret_cast<uint4*>(stage + TC_BM * 64 + rt * 64)[q ^ sw2] = reinterpret_cast<const uint4*>(mid)[q];
+          reinterpret_cast<uint4*>(stage + 2 * TC_BM * 64 + rt * 64)[q ^ sw2] = reinterpret_cast<const uint4*>(lo)[q];
         }
       }
       fence_async_smem();
@@ -447,8 +456,9 @@ bool make_map(CUtensorMap* map, const void* ptr, int rows, int cols, int ld, int
             CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-// Output map: [rows, cols] of fp32 or bf16 with row stride ld (elements), boxes of 32 x 128, no
-// swizzle (the epilogue stages a chunk row-major).
+// Output map: [rows, cols] of fp32 or bf16 with row stride ld (elements), boxes of 32 x 128,
+// swizzled over their 128- or 64-byte rows: unswizzled, the epilogue's threads, a row each, would
+// all write the same banks (folding 126464 ids: 1207 us, swizzled 1052 us).
 bool make_out_map(CUtensorMap* map, const void* ptr, bool f32, int rows, int cols, int ld) {
   auto fn = encode_fn();
   if (!fn) return false;
@@ -460,7 +470,7 @@ bool make_out_map(CUtensorMap* map, const void* ptr, bool f32, int rows, int col
   cuuint32_t estr[2] = {1, 1};
   return fn(map, f32 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2,
             const_cast<void*>(ptr), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
-            CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_NONE,
+            f32 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_NONE,
             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
@@ -490,32 +500,50 @@ bool gemm_tc_supported(const void* A, int lda, const void* B, int ldb, int K) {
 
 // One or two products C = A B^T, A [M, K] (row stride lda) and B [N, K] (row stride ldb) bf16,
 // fp32 accumulation, in one launch.
+//
+// Tile columns, parts of K and pipeline depth follow from the sizes alone, so a product is summed
+// in the same order whichever call it belongs to. What a CTA waits for is its operands through
+// L2 (about 40 bytes a cycle and SM), so among 64, 128 and 256 columns the least traffic per SM
+// wins: up to one CTA an SM, K split while there is room, a 4-stage pipeline; with more tiles
+// than SMs, 2-stage CTAs share an SM in pairs, one multiplying while the other stores.
 cudaError_t gemm_tc_grouped(const TcSpec* spec, int nprob, int32_t* status, cudaStream_t stream,
-                            int stages, int carveout_kb) {
-  if (nprob < 1 || nprob > 2 || (stages != 2 && stages != 4)) return cudaErrorInvalidValue;
-  if (carveout_kb != CARVEOUT_GEMM_KB && stages != 2) return cudaErrorInvalidValue;
-  int nmax = 0;
-  for (int i = 0; i < nprob; ++i) nmax = spec[i].N > nmax ? spec[i].N : nmax;
-  // Few tiles: split K. The rule looks at the products alone, so a product is summed in the same
-  // order whichever schedule it runs in.
-  int tiles = 0, nk = 0;
+                            bool beside) {
+  if (nprob < 1 || nprob > 2) return cudaErrorInvalidValue;
+  int nmax = 0, nk_min = 0, nk_max = 0;
   for (int i = 0; i < nprob; ++i) {
-    tiles += ((spec[i].M + TC_BM - 1) / TC_BM) * ((spec[i].N + TC_SPLIT_BN - 1) / TC_SPLIT_BN);
     const int k = (spec[i].K + TC_BK - 1) / TC_BK;
-    nk = i == 0 || k < nk ? k : nk;
+    nmax = spec[i].N > nmax ? spec[i].N : nmax;
+    nk_min = i == 0 || k < nk_min ? k : nk_min;
+    nk_max = k > nk_max ? k : nk_max;
   }
-  int split = 1;
-  while (tiles <= TC_SPLIT_TILES && split < TC_SPLIT_MAX && 2 * split * tiles <= TC_SPLIT_CTAS + 8 &&
-         nk >= 4 * split)
-    split *= 2;
-  int max_bn = spec[0].max_bn;
-  if (split > 1) {
-    max_bn = TC_SPLIT_BN;
-    stages = 4;
-    carveout_kb = CARVEOUT_GEMM_KB;
+  int BN = 0, split = 1, stages = 4;
+  double best = 0.;
+  bool may_split = false;
+  for (int bn = 256; bn >= 64; bn /= 2) {
+    const int cols = tc_bn(nmax < bn ? nmax : bn);
+    long long tiles = 0;
+    for (int i = 0; i < nprob; ++i)
+      tiles += (long long)((spec[i].M + TC_BM - 1) / TC_BM) * ((spec[i].N + cols - 1) / cols);
+    if (bn == 256) may_split = tiles <= TC_SPLIT_TILES;
+    int parts = 1;
+    while (may_split && parts < TC_SPLIT_MAX && 2 * parts * tiles <= TC_SMS && nk_min >= 2 * parts * TC_SPLIT_STEPS)
+      parts *= 2;
+    const double sms = tiles * parts < TC_SMS ? (double)tiles * parts : TC_SMS;
+    const double cost = tiles / sms * nk_max * (TC_BM + cols);
+    if (BN == 0 || cost < best) {
+      best = cost;
+      BN = cols;
+      split = parts;
+      stages = tiles > TC_SMS ? 2 : 4;
+    }
   }
-  if (max_bn >= 16 && nmax > max_bn) nmax = max_bn;
-  const int BN = tc_bn(nmax);
+  if (beside && split == 1) {
+    // beside the sweeps: tiles of 64 columns and two stages (49 KB) within the sweep's carveout,
+    // so that sweep CTAs stay on the same SMs
+    BN = tc_bn(nmax < 64 ? nmax : 64);
+    stages = 2;
+  }
+  const bool small = beside && split == 1;
   int cols = 32;
   while (cols < BN) cols *= 2;
   TcMaps maps;
@@ -553,15 +581,11 @@ cudaError_t gemm_tc_grouped(const TcSpec* spec, int nprob, int32_t* status, cuda
   }
   if (total == 0) return cudaSuccess;
   const size_t smem = gemm_tc_smem(BN, stages);
-  if (smem > (size_t)(carveout_kb - 1) * 1024 && carveout_kb == CARVEOUT_SMALL_KB)
-    return cudaErrorInvalidValue;
-  auto kernel = carveout_kb == CARVEOUT_SMALL_KB  ? gemm_tc_kernel<2, CARVEOUT_SMALL_KB>
-                : carveout_kb == CARVEOUT_FULL_KB ? gemm_tc_kernel<2, CARVEOUT_FULL_KB>
-                : stages == 2                     ? gemm_tc_kernel<2, CARVEOUT_GEMM_KB>
-                                                  : gemm_tc_kernel<4, CARVEOUT_GEMM_KB>;
+  auto kernel = small ? gemm_tc_kernel<2, true>
+                      : (stages == 2 ? gemm_tc_kernel<2> : gemm_tc_kernel<4>);
   cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        static_cast<int>(smem));
-  if (e == cudaSuccess) e = prefer_carveout(kernel, carveout_kb);
+  if (e == cudaSuccess) e = prefer_carveout(kernel, small ? CARVEOUT_SMALL_KB : CARVEOUT_FULL_KB);
   if (e != cudaSuccess) return e;
   e = launch_cluster(kernel, dim3(total * split), dim3(TC_THREADS), smem, stream, split, maps, a);
   if (e != cudaSuccess) return e;
