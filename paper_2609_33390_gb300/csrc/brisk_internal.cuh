@@ -149,8 +149,10 @@ __device__ __forceinline__ void warp_lse_combine(float& m, float& s) {
 // while a CTA is resident, and the first kernel to land on an idle SM sets it, so a kernel that
 // runs beside another one (the sweep beside the dense products, the verifier-row sweep beside
 // the corrector) must leave room in its split for the other's CTAs. Everything not carved out
-// is L1, which holds the sweep's loads in flight: the sweep is fastest with a small split.
-constexpr int CARVEOUT_SMALL_KB = 64;    // sweep (9 KB a CTA), corrector, verification
+// is L1, which holds the sweep's loads in flight. Sweeps of 128 x 32 x 126464 alone with 32, 64,
+// 100, 132 and 164 KB: 168, 168, 166, 174, 189 us proposal rows; a decode tail of them with 64,
+// 100, 132 KB: 395, 381, 389 us.
+constexpr int CARVEOUT_SMALL_KB = 100;   // sweep (5.5 KB a CTA), corrector, verification
 constexpr int CARVEOUT_FULL_KB = 228;    // dense products, except beside the sweeps
 // Sets the carveout preference of `func` on the current device once (kernels of the same
 // signature are distinct entries: the registry is keyed by the function's address).
@@ -380,7 +382,7 @@ struct ScanArgs {
   int32_t* base_rank;    // [B, L] (base_prefix only)
   int beside_sweep;      // the corrector runs beside the verifier-row sweep
   // set by the launch (see corrector_kernel)
-  int groups, ring_depth, tok_ranks, ask_rows, ask_tokens;
+  int ring_depth, tok_ranks, ask_rows, ask_tokens;
   long long wait_limit;
   // select outputs (or verify inputs when do_select == 0)
   int32_t* sel_tokens;   // [B, L]

@@ -398,9 +398,8 @@ verify_kernel(const __grid_constant__ ScanArgs a) {
 constexpr int CORR_SPAN = 128;   // state elements a computing warp owns, 4 a lane
 constexpr int CORR_PART = 8;     // slots for the dots' parts: S <= 1024, so at most 8 warps
 constexpr int CORR_DEPTH = 4;    // positions the ring holds at most
-constexpr int CORR_AHEAD = 4;    // positions whose table rows are asked into L2 ahead of use
+constexpr int CORR_AHEAD = 3;    // positions whose rows are asked into L2 ahead of use
 constexpr int CORR_OTHERS = 64;  // threads of a sequence that do not compute
-constexpr int CORR_GROUPS = 2;   // sequences a CTA takes at most
 
 struct CorrSmem {
   uint64_t* full;  // [CORR_DEPTH] mbarriers: a stage's rows have landed
@@ -488,13 +487,20 @@ __device__ __forceinline__ void bulk_load(float* dst, const float* src, unsigned
       "l"(src), "r"(bytes), "r"(su32(bar))
       : "memory");
 }
-// Asks for `bytes` (a multiple of 16) at p in L2.
-__device__ __forceinline__ void prefetch_l2(const float* p, unsigned bytes) {
-  asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p), "r"(bytes));
+// Asks for `bytes` (a multiple of 16) at p in L2, to be kept there ahead of streamed data (a
+// concurrent sweep replaces the whole of L2 within 20 us).
+__device__ __forceinline__ uint64_t keep_policy() {
+  uint64_t p;
+  asm volatile("createpolicy.fractional.L2::evict_last.b64 %0, 1.0;" : "=l"(p));
+  return p;
 }
-// Barrier `id` of the block for `threads` of its threads.
-__device__ __forceinline__ void group_sync(int id, int threads) {
-  asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(threads) : "memory");
+__device__ __forceinline__ void prefetch_l2(const float* p, unsigned bytes, uint64_t policy) {
+  asm volatile("cp.async.bulk.prefetch.L2.global.L2::cache_hint [%0], %1, %2;" ::"l"(p), "r"(bytes),
+               "l"(policy));
+}
+// The block's barrier, for code that only some warps run.
+__device__ __forceinline__ void block_sync(int threads) {
+  asm volatile("bar.sync 0, %0;" ::"r"(threads) : "memory");
 }
 // Bounded wait for the phase of the given parity (more than `limit` SM cycles: false).
 __device__ __forceinline__ bool mbar_wait_limit(uint64_t* bar, uint32_t parity, long long limit) {
@@ -545,23 +551,21 @@ __device__ __forceinline__ float sigmoid_hw(float x) { return rcp_hw(1.f + ex2(-
 // load the residual rows themselves. One more warp asks rows into L2 some positions ahead (where
 // the ring is shallow) and stores the outputs. The features of every (position, rank fed
 // forward) pair are tabulated first; the shares of a position that do not depend on the
-// selection are summed before the barrier of the position before. A CTA takes one sequence, or
-// several side by side (a.groups), each with its own warps, barrier and shared memory.
+// selection are summed before the barrier of the position before. (One CTA an SM is asked of the
+// compiler: left to itself it settles on 80 to 103 registers, some spilled on the chain, and one
+// sequence's graph replay takes 61 us, not 51.)
 template <int NP, bool ROWS, bool SAMPLE, bool VERIFY>
-__global__ void __launch_bounds__(384)
+__global__ void __launch_bounds__(32 * CORR_PART + CORR_OTHERS, 1)
 corrector_kernel(const __grid_constant__ ScanArgs a) {
   extern __shared__ __align__(16) char smem_raw[];
   const int L = a.L, K = a.K, S = a.S, V = a.V, R = a.tok_ranks, D = a.ring_depth;
   const int stage = corr_stage(K, S, R, ROWS);
-  const int NT = blockDim.x / a.groups, grp = threadIdx.x / NT;   // threads of a sequence
-  const int b = blockIdx.x * a.groups + grp;
-  if (b >= a.B) return;
-  const int tid = threadIdx.x - grp * NT, warp = tid >> 5, lane = tid & 31;
-  const int NC = NT - CORR_OTHERS;                                 // computing threads
-  auto sync = [&] { group_sync(1 + grp, NT); };
+  const int b = blockIdx.x, NT = blockDim.x;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int NC = NT - CORR_OTHERS;   // computing threads
+  auto sync = [&] { block_sync(NT); };
   CorrSmem sm;
-  const size_t own = corr_layout(L, K, S, V, D, stage, VERIFY, nullptr, nullptr);
-  corr_layout(L, K, S, V, D, stage, VERIFY, smem_raw + grp * own, &sm);
+  corr_layout(L, K, S, V, D, stage, VERIFY, smem_raw, &sm);
   const size_t bL = (size_t)b * L;
   constexpr int MODE = SAMPLE ? BRISK_SELECT_SAMPLE : BRISK_SELECT_GREEDY;
 
@@ -770,10 +774,14 @@ corrector_kernel(const __grid_constant__ ScanArgs a) {
     if (lane == 0)
       for (int p = L - D < 0 ? 0 : L - D; p < L; ++p) mbar_drain(&sm.full[p % D], (p / D) & 1);
   } else {
+    const uint64_t keep = keep_policy();
     auto ask = [&](int p) {
-      if (!a.ask_rows || p >= L || lane >= K) return;
-      prefetch_l2(a.U + (size_t)sm.cid[p * K + lane] * S, S * 4);
-      if (a.ask_tokens && p + 1 < L) prefetch_l2(a.Tzh + (size_t)sm.cid[p * K + lane] * 2 * S, S * 8);
+      if (!a.ask_rows || p >= L) return;
+      if (lane == 0) prefetch_l2(a.G + (bL + p) * 2 * S, S * 8, keep);
+      if (lane >= K) return;
+      prefetch_l2(a.U + (size_t)sm.cid[p * K + lane] * S, S * 4, keep);
+      if ((a.ask_tokens || lane < R) && p + 1 < L)
+        prefetch_l2(a.Tzh + (size_t)sm.cid[p * K + lane] * 2 * S, S * 8, keep);
     };
     for (int p = 0; p < CORR_AHEAD; ++p) ask(p);
     features();
@@ -819,20 +827,22 @@ size_t scan_smem_bytes(int L, int K, int S, int V) {
 
 namespace {
 
-constexpr size_t CORR_SMEM = 220 * 1024;   // shared memory a CTA may take
+// Shared memory a CTA may take; beside the verifier-row sweep (128 sequences, S = 512, K = 8):
+// 377 us a decode tail with the corrector's 69 KB beside sweep CTAs, 382 us with two sequences'
+// 210 KB on half as many SMs, which no sweep CTA shares.
+constexpr size_t CORR_SMEM = 220 * 1024;
+constexpr size_t CORR_SMEM_BESIDE = 76 * 1024;
 
 template <int NP, bool ROWS, bool SAMPLE, bool VERIFY>
 cudaError_t launch_corrector_k(const ScanArgs& a, cudaStream_t stream) {
-  const size_t smem = a.groups * corr_layout(a.L, a.K, a.S, a.V, a.ring_depth,
-                                             corr_stage(a.K, a.S, a.tok_ranks, ROWS), VERIFY,
-                                             nullptr, nullptr);
+  const size_t smem = corr_layout(a.L, a.K, a.S, a.V, a.ring_depth,
+                                  corr_stage(a.K, a.S, a.tok_ranks, ROWS), VERIFY, nullptr, nullptr);
   auto kernel = corrector_kernel<NP, ROWS, SAMPLE, VERIFY>;
   cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e == cudaSuccess) e = prefer_carveout(kernel, CARVEOUT_SMALL_KB);
   if (e != cudaSuccess) return e;
   const int threads = 32 * ((a.S + CORR_SPAN - 1) / CORR_SPAN) + CORR_OTHERS;
-  e = launch_prio(kernel, dim3((a.B + a.groups - 1) / a.groups), dim3(a.groups * threads), smem,
-                  stream, a);
+  e = launch_prio(kernel, dim3(a.B), dim3(threads), smem, stream, a);
   if (e != cudaSuccess) return e;
   return cudaGetLastError();
 }
@@ -849,9 +859,14 @@ cudaError_t launch_corrector_m(const ScanArgs& a, cudaStream_t stream) {
 cudaError_t launch_corrector(const ScanArgs& args, cudaStream_t stream) {
   ScanArgs a = args;
   a.wait_limit = wait_limit_cycles();
-  // Beside the verifier-row sweep, sequences of up to 512 state elements share CTAs: a corrector
-  // CTA keeps the sweep's off its SM, so fewer and fuller ones leave it more SMs.
-  a.groups = a.beside_sweep && a.S <= 512 && !a.do_verify ? CORR_GROUPS : 1;
+  auto bytes = [&](int depth, int ranks, bool rows) {
+    return corr_layout(a.L, a.K, a.S, a.V, depth, corr_stage(a.K, a.S, ranks, rows),
+                       a.do_verify != 0, nullptr, nullptr);
+  };
+  // Beside the verifier-row sweep a CTA stays within the sweep's carveout, with room for sweep CTAs
+  // on its SM, where it can.
+  const size_t room = a.beside_sweep && bytes(2, 1, true) <= CORR_SMEM_BESIDE ? CORR_SMEM_BESIDE
+                                                                              : CORR_SMEM;
   // the ring's depth, the token rows a stage holds, and whether it holds the residual rows: the
   // first of these that fits
   struct Shape { int depth, ranks; bool rows; };
@@ -862,9 +877,7 @@ cudaError_t launch_corrector(const ScanArgs& args, cudaStream_t stream) {
     a.ring_depth = s.depth;
     a.tok_ranks = s.ranks;
     rows = s.rows;
-    if (a.groups * corr_layout(a.L, a.K, a.S, a.V, s.depth, corr_stage(a.K, a.S, s.ranks, s.rows),
-                               a.do_verify != 0, nullptr, nullptr) <= CORR_SMEM)
-      break;
+    if (bytes(s.depth, s.ranks, s.rows) <= room) break;
   }
   a.ask_rows = a.ring_depth < 4;
   a.ask_tokens = !a.beside_sweep;

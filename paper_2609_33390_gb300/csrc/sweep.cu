@@ -100,11 +100,9 @@ __device__ __forceinline__ float key_to_float(unsigned k) {
 
 struct SweepSmem {
   uint4 stash[SWEEP_WARPS][SWEEP_UNROLL];        // one lane's batch
-  float val[SWEEP_WARPS][SWEEP_BUF];             // the warps' buffers
+  float val[SWEEP_WARPS][SWEEP_BUF];             // the warps' buffers, then the entries to merge
   int id[SWEEP_WARPS][SWEEP_BUF];
-  unsigned long long top[SWEEP_WARPS];           // the warps' largest lane maxima so far (packed)
-  float list_v[SWEEP_MERGE];                     // entries to merge
-  int list_i[SWEEP_MERGE];
+  unsigned long long top[2][SWEEP_WARPS];        // the warps' largest lane maxima so far (packed)
   int listed;
   float thr;                                     // the final threshold
   float m[SWEEP_WARPS], s[SWEEP_WARPS];
@@ -123,35 +121,46 @@ struct WarpState {
   int fresh;       // of these, appended since the threshold was last raised
 };
 
-// Publishes this warp's four largest lane maxima (the largest alone for kout == 1), as one word
-// that other warps read whole: 16-bit keys, cut towards smaller values, so still lower bounds.
+// Publishes this warp's four largest lane maxima (the largest alone for kout == 1; the four
+// largest of either half of the warp for kout > 16), each set as one word that other warps read
+// whole, so that no maximum is ever seen twice: 16-bit keys, cut towards smaller values, so still
+// lower bounds. With fewer than kout sets the threshold would hang on the warp whose logits are
+// smallest (32 of 100003 fp32: 224 us with four maxima a warp, 175 with eight).
 __device__ __forceinline__ void publish(SweepSmem& sm, int warp, int kout, float m) {
   const int lane = threadIdx.x & 31;
+  const bool halves = kout > 16;
+  const unsigned mask = !halves ? FULL_MASK : (lane < 16 ? 0x0000ffffu : 0xffff0000u);
   unsigned key = order_key(m);
-  unsigned long long word = __reduce_max_sync(FULL_MASK, key);
+  unsigned long long word = __reduce_max_sync(mask, key);
   if (kout > 1) {
     unsigned top = (unsigned)word;
     word >>= 16;
 #pragma unroll
     for (int j = 1; j < SWEEP_TOPS; ++j) {
-      const unsigned at = __ballot_sync(FULL_MASK, key == top);
+      const unsigned at = __ballot_sync(mask, key == top) & mask;
       if (lane == __ffs(at) - 1) key = 0;
-      top = __reduce_max_sync(FULL_MASK, key);
+      top = __reduce_max_sync(mask, key);
       word = word << 16 | top >> 16;
     }
   }
-  if (lane == 0) *const_cast<volatile unsigned long long*>(&sm.top[warp]) = word;
+  if (lane == 0 || (halves && lane == 16))
+    *const_cast<volatile unsigned long long*>(&sm.top[lane >> 4][warp]) = word;
   __syncwarp();
 }
 
 // K-th largest of the published maxima: a lower bound on the segment's K-th best.
 __device__ __forceinline__ float segment_threshold(const SweepSmem& sm, int kout) {
-  const int lane = threadIdx.x & 31;
-  const volatile unsigned long long* top = sm.top;
+  const int lane = threadIdx.x & 31, w = lane / SWEEP_TOPS, shift = 16 * (lane % SWEEP_TOPS);
+  const volatile unsigned long long* top = &sm.top[0][0];
   if (kout == 1)
     return key_to_float(__reduce_max_sync(FULL_MASK, lane < SWEEP_WARPS ? (unsigned)top[lane] : 0u));
-  const unsigned key = (unsigned)(top[lane / SWEEP_TOPS] >> (16 * (lane % SWEEP_TOPS))) & 0xffffu;
-  const unsigned kth = __shfl_sync(FULL_MASK, warp_sort(key), 32 - kout);
+  unsigned key = warp_sort((unsigned)(top[w] >> shift) & 0xffffu);
+  if (kout > 16) {
+    // the larger 32 of 64: two sorted halves compared end to end
+    const unsigned other = warp_sort((unsigned)(top[SWEEP_WARPS + w] >> shift) & 0xffffu);
+    key = warp_sort(max(key, __shfl_xor_sync(FULL_MASK, other, 31)));
+  }
+  const unsigned kth = __shfl_sync(FULL_MASK, key, 32 - kout);
   return kth <= 0x7fu ? -INFINITY : key_to_float(kth << 16);   // (0x7f: the key of -inf)
 }
 
@@ -364,19 +373,28 @@ __device__ __forceinline__ void sweep_segment(const T* rowp, int V, int split, i
     if (lane == 0) sm.thr = t;
   }
   __syncthreads();
+  // the entries that reach it, through registers: the list takes the buffers' place
   const float thr = sm.thr;
-  for (int e0 = 0; e0 < st.count; e0 += 32) {
-    const int e = e0 + lane;
-    const float v = e < st.count ? sm.val[warp][e] : -INFINITY;
-    const unsigned hit = __ballot_sync(FULL_MASK, e < st.count && v >= thr);
-    int at = 0;
-    if (lane == 0) at = atomicAdd(&sm.listed, __popc(hit));
-    at = __shfl_sync(FULL_MASK, at, 0) + __popc(hit & ((1u << lane) - 1));
-    if (hit >> lane & 1) {
-      sm.list_v[at] = v;
-      sm.list_i[at] = sm.id[warp][e];
-    }
+  float v[SWEEP_BUF / 32];
+  int id[SWEEP_BUF / 32], at[SWEEP_BUF / 32];
+#pragma unroll
+  for (int j = 0; j < SWEEP_BUF / 32; ++j) {
+    const int e = lane + 32 * j;
+    v[j] = sm.val[warp][e];
+    id[j] = sm.id[warp][e];
+    const unsigned hit = __ballot_sync(FULL_MASK, e < st.count && v[j] >= thr);
+    int first = 0;
+    if (lane == 0 && hit) first = atomicAdd(&sm.listed, __popc(hit));
+    first = __shfl_sync(FULL_MASK, first, 0);
+    at[j] = hit >> lane & 1 ? first + __popc(hit & ((1u << lane) - 1)) : -1;
   }
+  __syncthreads();
+#pragma unroll
+  for (int j = 0; j < SWEEP_BUF / 32; ++j)
+    if (at[j] >= 0) {
+      (&sm.val[0][0])[at[j]] = v[j];
+      (&sm.id[0][0])[at[j]] = id[j];
+    }
 }
 
 // The best kout of the n listed entries, best first, into best_v / best_i (-inf, INVALID_ID past
@@ -388,12 +406,14 @@ __device__ __forceinline__ void merge_by_rank(SweepSmem& sm, int n, int kout) {
     sm.best_i[tid] = INVALID_ID;
   }
   __syncthreads();
+  const float* list_v = &sm.val[0][0];
+  const int* list_i = &sm.id[0][0];
   for (int e = tid; e < n; e += SWEEP_WARPS * 32) {
-    const float v = sm.list_v[e];
-    const int i = sm.list_i[e];
+    const float v = list_v[e];
+    const int i = list_i[e];
     int rank = 0;
 #pragma unroll 4
-    for (int o = 0; o < n; ++o) rank += better(sm.list_v[o], sm.list_i[o], v, i) ? 1 : 0;
+    for (int o = 0; o < n; ++o) rank += better(list_v[o], list_i[o], v, i) ? 1 : 0;
     if (i != INVALID_ID && rank < kout) {
       sm.best_v[rank] = v;
       sm.best_i[rank] = i;
@@ -454,8 +474,8 @@ sweep_kernel(const __grid_constant__ SweepLaunch a) {
     __threadfence();
     for (int e = tid; e < nsplit * kout; e += SWEEP_WARPS * 32) {
       const size_t q = (p0 + e / kout) * a.KP + e % kout;
-      sm.list_v[e] = __ldcg(sg.part_val + q);
-      sm.list_i[e] = __ldcg(sg.part_id + q);
+      (&sm.val[0][0])[e] = __ldcg(sg.part_val + q);
+      (&sm.id[0][0])[e] = __ldcg(sg.part_id + q);
     }
     merge_by_rank(sm, nsplit * kout, kout);
     if (warp == 0) {
