@@ -283,6 +283,28 @@ __device__ __forceinline__ float4 ld_cluster(const float* p, unsigned rank) {
   return v;
 }
 
+// Stores x at this CTA's shared address p, in the shared memory of CTA `rank` of the cluster.
+__device__ __forceinline__ void st_cluster(float* p, unsigned rank, float x) {
+  uint32_t addr;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(addr) : "r"(su32(p)), "r"(rank));
+  asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(addr), "f"(x) : "memory");
+}
+// Sum, in rank order, of the 16 bytes at this CTA's shared address p in the first n (at most 8)
+// CTAs of the cluster, all loads in flight at once.
+__device__ __forceinline__ float4 sum_cluster(const float* p, int n) {
+  float4 v[8];
+#pragma unroll
+  for (int o = 0; o < 8; ++o)
+    if (o < n) v[o] = ld_cluster(p, o);
+  float4 t = v[0];
+#pragma unroll
+  for (int o = 1; o < 8; ++o)
+    if (o < n) {
+      t.x += v[o].x; t.y += v[o].y; t.z += v[o].z; t.w += v[o].w;
+    }
+  return t;
+}
+
 __device__ __forceinline__ void set_status(int32_t* status, int code) {
   if (status) atomicCAS(status, 0, code);
 }
@@ -383,6 +405,7 @@ struct ScanArgs {
   int beside_sweep;      // the corrector runs beside the verifier-row sweep
   // set by the launch (see corrector_kernel)
   int ring_depth, tok_ranks, ask_rows, ask_tokens;
+  int parts;             // CTAs that share a verification's residual walk
   long long wait_limit;
   // select outputs (or verify inputs when do_select == 0)
   int32_t* sel_tokens;   // [B, L]

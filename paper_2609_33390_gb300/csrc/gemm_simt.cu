@@ -8,7 +8,7 @@ namespace brisk {
 namespace {
 
 // One CTA computes a 128 x 64 tile of one product on 256 threads, 8 x 4 outputs a thread in
-// packed fp32 pairs, over 16-wide K slices double-buffered in shared memory (the next slice's
+// packed fp32 pairs, over 16-wide K slices double-buffered in shared memory (the next two slices'
 // global loads are in flight while the present one is multiplied). Large products are bound by
 // the FMA pipes. A product with few tiles is bound by the K loop's latency instead (12 sequences
 // x 24 positions x 1000 by 96: 10 tiles, 145 us on 64 x 64 tiles over the whole K), so there a
@@ -87,30 +87,32 @@ gemm_simt_kernel(const __grid_constant__ SimtProblem P) {
   const TA* brow_a = A + (m0 + (rb ? r + 64 : 0)) * P.lda;
   const TB* brow = B + (P.transB ? 0 : (n0 + (rn ? r : 0)) * P.ldb);
   const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
-  float4 va, vb, vn;
+  struct Slice { float4 a, b, n; };
   auto load = [&](int s) {
+    Slice v;
     const int k = s * TK + 4 * q;
-    va = ra ? row4(arow, k, K, P.vecA) : zero;
-    vb = rb ? row4(brow_a, k, K, P.vecA) : zero;
+    v.a = ra ? row4(arow, k, K, P.vecA) : zero;
+    v.b = rb ? row4(brow_a, k, K, P.vecA) : zero;
     if (!P.transB) {
-      vn = rn ? row4(brow, k, K, P.vecB) : zero;
+      v.n = rn ? row4(brow, k, K, P.vecB) : zero;
     } else {
       const int kt = s * TK + kk;
-      vn = kt < K ? row4(B + (long long)kt * P.ldb + n0, 4 * c, (int)min((long long)TN, N - n0), P.vecB)
+      v.n = kt < K ? row4(B + (long long)kt * P.ldb + n0, 4 * c, (int)min((long long)TN, N - n0), P.vecB)
                   : zero;
     }
+    return v;
   };
-  auto store = [&](int buf) {
+  auto store = [&](int buf, const Slice& v) {
     SimtSlices& z = sm.s;
-    z.a[buf][4 * q][r] = va.x; z.a[buf][4 * q + 1][r] = va.y;
-    z.a[buf][4 * q + 2][r] = va.z; z.a[buf][4 * q + 3][r] = va.w;
-    z.a[buf][4 * q][r + 64] = vb.x; z.a[buf][4 * q + 1][r + 64] = vb.y;
-    z.a[buf][4 * q + 2][r + 64] = vb.z; z.a[buf][4 * q + 3][r + 64] = vb.w;
+    z.a[buf][4 * q][r] = v.a.x; z.a[buf][4 * q + 1][r] = v.a.y;
+    z.a[buf][4 * q + 2][r] = v.a.z; z.a[buf][4 * q + 3][r] = v.a.w;
+    z.a[buf][4 * q][r + 64] = v.b.x; z.a[buf][4 * q + 1][r + 64] = v.b.y;
+    z.a[buf][4 * q + 2][r + 64] = v.b.z; z.a[buf][4 * q + 3][r + 64] = v.b.w;
     if (!P.transB) {
-      z.b[buf][4 * q][r] = vn.x; z.b[buf][4 * q + 1][r] = vn.y;
-      z.b[buf][4 * q + 2][r] = vn.z; z.b[buf][4 * q + 3][r] = vn.w;
+      z.b[buf][4 * q][r] = v.n.x; z.b[buf][4 * q + 1][r] = v.n.y;
+      z.b[buf][4 * q + 2][r] = v.n.z; z.b[buf][4 * q + 3][r] = v.n.w;
     } else {
-      *reinterpret_cast<float4*>(&z.b[buf][kk][4 * c]) = vn;
+      *reinterpret_cast<float4*>(&z.b[buf][kk][4 * c]) = v.n;
     }
   };
   // outputs: rows 8 ty .. 8 ty + 7 in pairs, columns 4 tx .. 4 tx + 3
@@ -120,14 +122,14 @@ gemm_simt_kernel(const __grid_constant__ SimtProblem P) {
   for (int i = 0; i < 4; ++i)
 #pragma unroll
     for (int j = 0; j < 4; ++j) acc[i][j] = make_float2(0.f, 0.f);
-  if (s0 < s1) {
-    load(s0);
-    store(0);
-  }
+  // two slices on their way while one is multiplied
+  Slice next{}, after{};
+  if (s0 < s1) store(0, load(s0));
+  if (s0 + 1 < s1) next = load(s0 + 1);
   __syncthreads();
   for (int s = s0; s < s1; ++s) {
     const int buf = (s - s0) & 1;
-    if (s + 1 < s1) load(s + 1);
+    if (s + 2 < s1) after = load(s + 2);
 #pragma unroll
     for (int k = 0; k < TK; ++k) {
       const float4 x0 = *reinterpret_cast<const float4*>(&sm.s.a[buf][k][8 * ty]);
@@ -142,7 +144,8 @@ gemm_simt_kernel(const __grid_constant__ SimtProblem P) {
         for (int j = 0; j < 4; ++j)
           acc[i][j] = __ffma2_rn(x[i], make_float2(yv[j], yv[j]), acc[i][j]);
     }
-    if (s + 1 < s1) store(buf ^ 1);
+    if (s + 1 < s1) store(buf ^ 1, next);
+    next = after;
     __syncthreads();
   }
   auto bias = [&](long long m, long long n) {
@@ -176,11 +179,7 @@ gemm_simt_kernel(const __grid_constant__ SimtProblem P) {
   const int r0 = part * share, r1 = min(rows, r0 + share);
   for (int e = r0 * 16 + tid; e < r1 * 16; e += SIMT_THREADS) {
     const int row = e >> 4, col = 4 * (e & 15);
-    float4 v = ld_cluster(&sm.part[row][col], 0);
-    for (int o = 1; o < split; ++o) {
-      const float4 w = ld_cluster(&sm.part[row][col], o);
-      v.x += w.x; v.y += w.y; v.z += w.z; v.w += w.w;
-    }
+    const float4 v = sum_cluster(&sm.part[row][col], split);
     const float x[4] = {v.x, v.y, v.z, v.w};
     float* dst = P.C + (m0 + row) * P.ldc + n0 + col;
 #pragma unroll

@@ -327,11 +327,7 @@ gemm_tc_kernel(const __grid_constant__ TcMaps maps, const __grid_constant__ TcAr
         const int row = e / per_row, col = 4 * (e - row * per_row);
         if (n0 + col >= P.N) continue;               // N is a multiple of 16
         const float* src = part + (size_t)row * (a.BN + TC_PART_PAD) + col;
-        float4 v = ld_cluster(src, 0);
-        for (int o = 1; o < a.split; ++o) {
-          const float4 w = ld_cluster(src, o);
-          v.x += w.x; v.y += w.y; v.z += w.z; v.w += w.w;
-        }
+        float4 v = sum_cluster(src, a.split);
         if (P.bias) {
           const float* w = P.bias + (size_t)((m0 + row) % P.bias_period) * P.N + n0 + col;
           v.x += w[0]; v.y += w[1]; v.z += w[2]; v.w += w[3];

@@ -27,6 +27,8 @@ namespace {
 // loads and the hardware one).
 constexpr int VERIFY_THREADS = 128;
 constexpr int VERIFY_THREADS_MAX = 512;
+constexpr int VERIFY_CTAS = 152;       // CTAs up to which a residual walk is shared
+constexpr int VERIFY_SHARE = 4096;     // ids of it a CTA has at least
 
 struct Smem {
   int* cid;        // [L][K]
@@ -80,9 +82,11 @@ __device__ __forceinline__ float redux_max(float x) {
   return r;
 }
 
-// Select with lane k holding refined score k (lanes >= K hold -inf); the same in every lane.
+// Select with lane k holding refined score k (lanes >= K hold -inf), K <= NP; the same in every
+// lane.
 // Greedy: argmax, the lowest rank on ties. Sample: the first rank whose cumulative softmax mass
 // exceeds u * total (warp prefix sums), else the last rank with mass.
+template <int NP = 32>
 __device__ __forceinline__ int select_warp(float ref, int K, int mode, float u) {
   const int lane = threadIdx.x & 31;
   if (mode == BRISK_SELECT_GREEDY) {
@@ -97,11 +101,11 @@ __device__ __forceinline__ int select_warp(float ref, int K, int mode, float u) 
   const float w = lane < K ? expf(ref - mx) : 0.f;
   float cum = w;
 #pragma unroll
-  for (int off = 1; off < 32; off <<= 1) {
+  for (int off = 1; off < NP; off <<= 1) {
     const float o = __shfl_up_sync(FULL_MASK, cum, off);
     if (lane >= off) cum += o;
   }
-  const float tot = __shfl_sync(FULL_MASK, cum, 31);
+  const float tot = __shfl_sync(FULL_MASK, cum, NP - 1);
   const unsigned hit = __ballot_sync(FULL_MASK, lane < K && cum > u * tot);
   if (hit) return __ffs(hit) - 1;
   const unsigned pos = __ballot_sync(FULL_MASK, w > 0.f);
@@ -169,9 +173,11 @@ __device__ __forceinline__ void residual8(const float (&l)[8], float lse, int v0
 
 // Draw from the normalised [p - pi]_+ of verifier row `rowp` with uniform u, walking ids in
 // ascending order; the verifier argmax when the residual mass is <= RESID_Z_FLOOR. CTA-wide.
+// With `parts` CTAs of a cluster sharing the walk, each sums every parts-th run of blocks into the
+// first CTA's shared memory, which goes on alone (the others return -1).
 __device__ int residual_sample(const Smem& sm, const void* rowp, int dt, int V, float lse,
                                const int* cid, const float* ref, int K, int select_mode,
-                               int sel_rank, float u, int argmax_p) {
+                               int sel_rank, float u, int argmax_p, int part, int parts) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int nblk = (V + RES_BLOCK - 1) / RES_BLOCK;
   // candidate k's proposal mass, held by lane k
@@ -185,8 +191,8 @@ __device__ int residual_sample(const Smem& sm, const void* rowp, int dt, int V, 
   // pass 1: block sums, blocks interleaved over warps, the logits of RES_FLIGHT blocks on their
   // way at once (one at a time, the walk of a 126464-entry row waited 31 times for memory:
   // a call waits for memory most of the time)
-  const int nw = (int)(blockDim.x >> 5);
-  for (int base = warp; base < nblk; base += RES_FLIGHT * nw) {
+  const int nw = (int)(blockDim.x >> 5) * parts;
+  for (int base = part * (int)(blockDim.x >> 5) + warp; base < nblk; base += RES_FLIGHT * nw) {
     float l[RES_FLIGHT][8];
 #pragma unroll
     for (int u = 0; u < RES_FLIGHT; ++u)   // (a block past the row reads as -inf)
@@ -201,8 +207,16 @@ __device__ int residual_sample(const Smem& sm, const void* rowp, int dt, int V, 
 #pragma unroll
       for (int e = 0; e < 8; ++e) t += R[e];
       t = warp_sum(t);
-      if (lane == 0) sm.bsum[blk] = t;
+      if (lane == 0) {
+        if (parts > 1) st_cluster(sm.bsum + blk, 0, t);
+        else sm.bsum[blk] = t;
+      }
     }
+  }
+  if (parts > 1) {
+    __syncwarp();
+    cluster_sync();
+    if (part) return -1;
   }
   __syncthreads();
   // warp 0: total mass and the block holding the target
@@ -311,8 +325,11 @@ __device__ int residual_sample(const Smem& sm, const void* rowp, int dt, int V, 
   return sm.imisc[1];
 }
 
-// Left-to-right verification of sm.sel against the verifier rows of sequence b.
-__device__ void verify_sequence(const ScanArgs& a, const Smem& sm, int b) {
+// Left-to-right verification of sm.sel against the verifier rows of sequence b. part of parts:
+// this CTA's place in a cluster that shares the residual walk (all of them find the same first
+// rejection).
+__device__ void verify_sequence(const ScanArgs& a, const Smem& sm, int b, int part = 0,
+                                int parts = 1) {
   const int tid = threadIdx.x;
   const int L = a.L, K = a.K;
   if (tid == 0) sm.imisc[2] = L;
@@ -345,9 +362,10 @@ __device__ void verify_sequence(const ScanArgs& a, const Smem& sm, int b) {
                              : (const void*)(reinterpret_cast<const float*>(a.logits_p) + bj * a.V);
       corr = residual_sample(sm, rowp, a.logits_dt, a.V, a.lse_p[bj], sm.cid + (size_t)j * K,
                              sm.ref + (size_t)j * K, K, a.select_mode, sm.rank[j], a.u_res[bj],
-                             a.argmax_p[bj]);
+                             a.argmax_p[bj], part, parts);
     }
   }
+  if (part) return;
   if (tid == 0) {
     a.accepted_len[b] = j;
     a.correction[b] = (j < L) ? corr : -1;
@@ -364,10 +382,11 @@ verify_kernel(const __grid_constant__ ScanArgs a) {
   extern __shared__ __align__(16) char smem_raw[];
   Smem sm;
   smem_layout(a.L, a.K, a.S, a.V, smem_raw, &sm);
-  const int b = blockIdx.x;
+  const int b = blockIdx.x / a.parts;
   const int tid = threadIdx.x;
   const int L = a.L, K = a.K, V = a.V;
   const size_t bL = (size_t)b * L;
+  if (a.parts > 1) cluster_sync();   // every CTA runs before its shared memory is written
   // Ids are gathered with below, so out-of-range ones (a row with no finite logit leaves
   // placeholder ids; caller-provided ids may be anything) are replaced by 0 and reported.
   const int nt = (int)blockDim.x;
@@ -391,7 +410,7 @@ verify_kernel(const __grid_constant__ ScanArgs a) {
     sm.rank[i] = r;
   }
   __syncthreads();
-  verify_sequence(a, sm, b);
+  verify_sequence(a, sm, b, (int)blockIdx.x - b * a.parts, a.parts);
 }
 
 // ---------------------------------------------------------------- corrector
@@ -409,6 +428,7 @@ struct CorrSmem {
                    //         and the gate's share of all five features
   float2* gap;     // [L]     features 0 and 1
   float* usel;     // [L]
+  int* base;       // [L]     base selections (same-state replay)
   float* red;      // [2][32][CORR_PART] the residual dots' parts, zero past the computing warps
   float* gpart;    // [2][CORR_PART]     the gate's parts
   float* ring;     // [depth][stage]: the token rows and residual rows of a position
@@ -436,6 +456,7 @@ __host__ __device__ inline size_t corr_layout(int L, int K, int S, int V, int de
   char* pf = take(sizeof(float4) * L * K);
   char* pg = take(sizeof(float2) * L);
   char* pu = take(sizeof(float) * L);
+  char* pq = take(sizeof(int) * L);
   char* pr = take(sizeof(float) * 2 * 32 * CORR_PART);
   char* pp = take(sizeof(float) * 2 * CORR_PART);
   char* pt = take(sizeof(float) * depth * stage);
@@ -443,7 +464,7 @@ __host__ __device__ inline size_t corr_layout(int L, int K, int S, int V, int de
   if (sm) {
     sm->full = (uint64_t*)pb;
     sm->cid = (int*)pc + K; sm->clp = (float*)pl; sm->feat = (float4*)pf; sm->gap = (float2*)pg;
-    sm->usel = (float*)pu; sm->red = (float*)pr; sm->gpart = (float*)pp; sm->ring = (float*)pt;
+    sm->usel = (float*)pu; sm->base = (int*)pq; sm->red = (float*)pr; sm->gpart = (float*)pp; sm->ring = (float*)pt;
   }
   // with verification in the same CTA its tables follow (the candidate table is the corrector's)
   if (!verify) return off;
@@ -634,13 +655,20 @@ corrector_kernel(const __grid_constant__ ScanArgs a) {
       gs += (q1.x + q1.y) + (q1.z + q1.w);
     }
     ref = fmaf(sig_alpha * sigmoid_hw(share + gs), dk, lp);   // (lanes past K: dk = 0)
-    return select_warp(ref, K, MODE, SAMPLE ? sm.usel[i] : 0.f);
+    return select_warp<NP>(ref, K, MODE, SAMPLE ? sm.usel[i] : 0.f);
   };
   // the token fed forward: the head's selection, or in a same-state replay the base selection
-  // (the Select rule on the base scores log q, same draw)
-  auto base_pick = [&](int i) {
-    return select_warp(lane < K ? sm.clp[i * K + lane] : -INFINITY, K, MODE,
-                       SAMPLE ? sm.usel[i] : 0.f);
+  // (the Select rule on the base scores log q, same draw), which is tabulated too
+  auto base_ranks = [&] {
+    if (!a.base_prefix) return;
+    for (int i = warp; i < L; i += NT / 32) {
+      const int pick = select_warp<NP>(lane < K ? sm.clp[i * K + lane] : -INFINITY, K, MODE,
+                                       SAMPLE ? sm.usel[i] : 0.f);
+      if (lane == 0) {
+        sm.base[i] = pick;
+        a.base_rank[bL + i] = pick;
+      }
+    }
   };
 
   if (tid < NC) {
@@ -667,6 +695,7 @@ corrector_kernel(const __grid_constant__ ScanArgs a) {
     }
     const float4 wg = ld4(a.wg + e4);
     features();
+    base_ranks();
     float4 s = make_float4(0.f, 0.f, 0.f, 0.f);   // s_{-1} = u_0 = Init(h_c, E(x0))
     if (owns) s = make_float4(tanhf(g0.x + t0.x), tanhf(g0.y + t0.y), tanhf(g0.z + t0.z),
                               tanhf(g0.w + t0.w));
@@ -744,7 +773,7 @@ corrector_kernel(const __grid_constant__ ScanArgs a) {
       sync();
       float ref;
       const int pick = decide(i, ft.w, ref);
-      prank = a.base_prefix ? base_pick(i) : pick;
+      prank = a.base_prefix ? sm.base[i] : pick;
     }
     if (!alive) set_status(a.status, BRISK_ERR_TIMEOUT);
   } else if (tid < NC + 32) {
@@ -763,6 +792,7 @@ corrector_kernel(const __grid_constant__ ScanArgs a) {
     };
     for (int p = 0; p < D - 1; ++p) fetch(p, p);
     features();
+    base_ranks();
     sync();
     int slot = D - 1;                     // of position i + D - 1
     for (int i = 0; i < L; ++i) {
@@ -785,6 +815,7 @@ corrector_kernel(const __grid_constant__ ScanArgs a) {
     };
     for (int p = 0; p < CORR_AHEAD; ++p) ask(p);
     features();
+    base_ranks();
     sync();
     int prank = 0;
     bool bad = false;
@@ -803,11 +834,7 @@ corrector_kernel(const __grid_constant__ ScanArgs a) {
           sm.v.rank[i] = pick;
         }
       }
-      prank = pick;
-      if (a.base_prefix) {
-        prank = base_pick(i);
-        if (lane == 0) a.base_rank[bL + i] = prank;
-      }
+      prank = a.base_prefix ? sm.base[i] : pick;
     }
     if (bad) set_status(a.status, BRISK_ERR_NUMERIC);
   }
@@ -894,13 +921,20 @@ cudaError_t launch_corrector(const ScanArgs& args, cudaStream_t stream) {
 // verification alone (do_verify) for every sequence.
 cudaError_t launch_scan(const ScanArgs& a, cudaStream_t stream) {
   if (a.do_select) return launch_corrector(a, stream);
+  ScanArgs v = a;
+  // A rejection walks a whole vocabulary row: clusters of up to 8 CTAs a sequence while there are
+  // SMs for them (16 sequences: 28 us alone, 12 us so).
+  v.parts = 1;
+  if (a.verify_mode == BRISK_VERIFY_STOCHASTIC)
+    while (v.parts < 8 && 2 * v.parts * a.B <= VERIFY_CTAS && a.V >= 2 * v.parts * VERIFY_SHARE)
+      v.parts *= 2;
   const size_t smem = scan_smem_bytes(a.L, a.K, a.S, a.V);
   cudaError_t e = cudaFuncSetAttribute(verify_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        (int)smem);
   if (e == cudaSuccess) e = prefer_carveout(verify_kernel, CARVEOUT_SMALL_KB);
   if (e != cudaSuccess) return e;
   const int threads = a.verify_mode == BRISK_VERIFY_STOCHASTIC ? VERIFY_THREADS_MAX : VERIFY_THREADS;
-  e = launch_prio(verify_kernel, dim3(a.B), dim3(threads), smem, stream, a);
+  e = launch_cluster(verify_kernel, dim3(a.B * v.parts), dim3(threads), smem, stream, v.parts, v);
   if (e != cudaSuccess) return e;
   return cudaGetLastError();
 }
