@@ -314,8 +314,9 @@ gemm_tc_kernel(const __grid_constant__ TcMaps maps, const __grid_constant__ TcAr
         tmem_ld32(tmem + (static_cast<uint32_t>(warp * 32) << 16) + c, v);
 #pragma unroll
         for (int q = 0; q < 8; ++q)
-          *reinterpret_cast<float4*>(mine + c + 4 * q) =
-              make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
+          if (c + 4 * q < a.BN)   // (the last 32 columns may reach past the tile's)
+            *reinterpret_cast<float4*>(mine + c + 4 * q) =
+                make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
       }
     }
     cluster_sync();
