@@ -129,6 +129,14 @@ TbLayout tb_layout(const brisk_dims* d) {
   return t;
 }
 
+// Whether the hidden products take the form that shares SMs with a sweep. Not in the fused
+// schedule (the sweep is as short as they are), nor for wide states beside whole-chip sweeps,
+// whose second product is four times larger (64 sequences, S = 1024: 525 us a tail, 625 so).
+inline bool products_beside(const WsLayout& w, const brisk_dims* d) {
+  if (w.schedule == SCHEDULE_FUSED) return false;
+  return w.schedule == SCHEDULE_SEPARATE || 2 * d->r <= BESIDE_STATE;
+}
+
 template <typename T>
 inline T* at(void* base, size_t off) { return reinterpret_cast<T*>(static_cast<char*>(base) + off); }
 template <typename T>
@@ -560,7 +568,7 @@ brisk_status brisk::decode_tail_locked(const brisk_dims* d, const brisk_params* 
   if (overlap) BRISK_CUDA(cudaStreamWaitEvent(m, ss->ev[0], 0));
   if (w.schedule != SCHEDULE_FUSED) BRISK_CUDA(cudaStreamWaitEvent(ss->lo, ss->ev[0], 0));
   s = hidden_products(d, p, tables, io->hidden, io->h_ctx, w, ws, ss->hi,
-                      overlap && 2 * d->r <= BESIDE_STATE);
+                      products_beside(w, d));
   if (s != BRISK_OK) return s;
   BRISK_CUDA(cudaEventRecord(ss->ev[1], ss->hi));
 
@@ -738,13 +746,15 @@ brisk_status brisk_replay_diagnostics(const brisk_dims* d, const brisk_params* p
   // Three independent parts meet in two places: the hidden products and the candidates in the
   // corrector, the corrector and the verifier rows' log-partition in the comparison. The products
   // run beside the proposal rows' sweep and the verifier rows' sweep beside the corrector, on side
-  // streams forked from the caller's (32 sequences: 213 us one after another, 158 us so).
+  // streams forked from the caller's, by priority (32 sequences: 213 us one after another, 155 us
+  // on the caller's stream and two more without priority for the corrector, 138 us so).
   std::lock_guard<std::mutex> lock(side_stream_mutex());
   SideStream* ss = side_stream();
   if (!ss) return BRISK_ERR_CUDA;
   BRISK_CUDA(cudaEventRecord(ss->ev[0], st));
   BRISK_CUDA(cudaStreamWaitEvent(ss->hi, ss->ev[0], 0));
-  s = hidden_products(d, p, tables, hidden, h_ctx, w, ws, ss->hi);
+  BRISK_CUDA(cudaStreamWaitEvent(ss->mid, ss->ev[0], 0));
+  s = hidden_products(d, p, tables, hidden, h_ctx, w, ws, ss->hi, products_beside(w, d));
   if (s != BRISK_OK) return s;
   BRISK_CUDA(cudaEventRecord(ss->ev[1], ss->hi));
   SweepLaunch sq{};
@@ -755,8 +765,8 @@ brisk_status brisk_replay_diagnostics(const brisk_dims* d, const brisk_params* p
   sq.KP = w.KP;
   sq.dtype = d->logits_dtype;
   sq.status = at<int32_t>(ws, w.status);
-  BRISK_CUDA(launch_sweep(sq, st));
-  BRISK_CUDA(cudaEventRecord(ss->ev[2], st));
+  BRISK_CUDA(launch_sweep(sq, ss->mid));
+  BRISK_CUDA(cudaEventRecord(ss->ev[2], ss->mid));
   BRISK_CUDA(cudaStreamWaitEvent(ss->lo, ss->ev[2], 0));
   SweepLaunch sp = sq;
   sp.seg[0] = make_seg(w, ws, 1, logits_p, BL, 1, at<int32_t>(ws, w.argmax_p), nullptr,
@@ -764,7 +774,7 @@ brisk_status brisk_replay_diagnostics(const brisk_dims* d, const brisk_params* p
   BRISK_CUDA(launch_sweep(sp, ss->lo));
   BRISK_CUDA(cudaEventRecord(ss->ev[3], ss->lo));
   // the head along the factual base prefix
-  BRISK_CUDA(cudaStreamWaitEvent(st, ss->ev[1], 0));
+  BRISK_CUDA(cudaStreamWaitEvent(ss->mid, ss->ev[1], 0));
   ScanArgs a = scan_args(d, p, tables, w, ws);
   a.select_mode = select_mode;
   a.do_select = 1;
@@ -777,9 +787,9 @@ brisk_status brisk_replay_diagnostics(const brisk_dims* d, const brisk_params* p
   a.refined = ref;
   a.base_prefix = 1;
   a.base_rank = at<int32_t>(ws, w.base_rank);
-  a.beside_sweep = w.schedule == SCHEDULE_OVERLAP;
-  BRISK_CUDA(launch_scan(a, st));
-  BRISK_CUDA(cudaStreamWaitEvent(st, ss->ev[3], 0));
+  a.beside_sweep = 1;
+  BRISK_CUDA(launch_scan(a, ss->mid));
+  BRISK_CUDA(cudaStreamWaitEvent(ss->mid, ss->ev[3], 0));
   ReplayArgs r{};
   r.B = d->B; r.L = d->L; r.V = d->V; r.K = d->K; r.logits_dt = d->logits_dtype;
   r.logits_p = logits_p;
@@ -792,7 +802,9 @@ brisk_status brisk_replay_diagnostics(const brisk_dims* d, const brisk_params* p
   r.flags = flags;
   r.first_breaker = first_breaker;
   r.status = at<int32_t>(ws, w.status);
-  BRISK_CUDA(launch_replay(r, st));
+  BRISK_CUDA(launch_replay(r, ss->mid));
+  BRISK_CUDA(cudaEventRecord(ss->ev[4], ss->mid));
+  BRISK_CUDA(cudaStreamWaitEvent(st, ss->ev[4], 0));
   return BRISK_OK;
 }
 

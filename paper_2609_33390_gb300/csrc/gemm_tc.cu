@@ -195,7 +195,8 @@ constexpr int TC_PART_PAD = 4;      // floats between the rows of a part in shar
 // SMALL_CARVEOUT does not change the code: it makes a separate kernel whose shared-memory
 // carveout preference (a per-kernel attribute) is the sweep's.
 template <int TC_STAGES, bool SMALL_CARVEOUT = false>
-__global__ void __launch_bounds__(TC_THREADS, 1)
+// At most 128 registers a thread: a CTA fits beside three sweep CTAs.
+__global__ void __launch_bounds__(TC_THREADS, 4)
 gemm_tc_kernel(const __grid_constant__ TcMaps maps, const __grid_constant__ TcArgs a) {
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   // 1024-byte alignment of every stage buffer (required by the 128-byte swizzle atoms)
@@ -534,13 +535,12 @@ cudaError_t gemm_tc_grouped(const TcSpec* spec, int nprob, int32_t* status, cuda
       stages = tiles > TC_SMS ? 2 : 4;
     }
   }
-  if (beside && split == 1) {
+  if (beside) {
     // beside the sweeps: tiles of 64 columns and two stages (49 KB) within the sweep's carveout,
-    // so that sweep CTAs stay on the same SMs
+    // so that both kernels' CTAs find room on the same SMs (the same parts of K: the same sums)
     BN = tc_bn(nmax < 64 ? nmax : 64);
     stages = 2;
   }
-  const bool small = beside && split == 1;
   int cols = 32;
   while (cols < BN) cols *= 2;
   TcMaps maps;
@@ -578,11 +578,11 @@ cudaError_t gemm_tc_grouped(const TcSpec* spec, int nprob, int32_t* status, cuda
   }
   if (total == 0) return cudaSuccess;
   const size_t smem = gemm_tc_smem(BN, stages);
-  auto kernel = small ? gemm_tc_kernel<2, true>
+  auto kernel = beside ? gemm_tc_kernel<2, true>
                       : (stages == 2 ? gemm_tc_kernel<2> : gemm_tc_kernel<4>);
   cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        static_cast<int>(smem));
-  if (e == cudaSuccess) e = prefer_carveout(kernel, small ? CARVEOUT_SMALL_KB : CARVEOUT_FULL_KB);
+  if (e == cudaSuccess) e = prefer_carveout(kernel, beside ? CARVEOUT_SMALL_KB : CARVEOUT_FULL_KB);
   if (e != cudaSuccess) return e;
   e = launch_cluster(kernel, dim3(total * split), dim3(TC_THREADS), smem, stream, split, maps, a);
   if (e != cudaSuccess) return e;
