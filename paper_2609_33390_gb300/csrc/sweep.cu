@@ -29,23 +29,13 @@ constexpr int SWEEP_MERGE = SWEEP_WARPS * SWEEP_BUF;    // entries merged at mos
 constexpr int SWEEP_TOPS = 32 / SWEEP_WARPS;            // maxima a warp publishes
 constexpr int SWEEP_RAISE = 3;                          // entries between raises of the threshold
 
-// Online log-sum-exp of one group of N logits whose max is mx.
-template <int N>
-__device__ __forceinline__ void lse_update(const float (&f)[N], float mx, float& m, float& s) {
-  if (mx > m) {
-    s *= ex2((m - mx) * LOG2E);
-    m = mx;
+// Online log-sum-exp of one logit.
+__device__ __forceinline__ void lse_update(float f, float& m, float& s) {
+  if (f > m) {
+    s *= ex2((m - f) * LOG2E);
+    m = f;
   }
-  if (m != -INFINITY) {
-    const float mb = m * LOG2E;
-    float a0 = 0.f, a1 = 0.f;
-#pragma unroll
-    for (int j = 0; j < N; j += 2) {
-      a0 += ex2(fmaf(f[j], LOG2E, -mb));
-      if (j + 1 < N) a1 += ex2(fmaf(f[j + 1], LOG2E, -mb));
-    }
-    s += a0 + a1;
-  }
+  if (m != -INFINITY) s += ex2((f - m) * LOG2E);
 }
 
 // The warp's values in ascending lane order (bitonic sort).
@@ -87,6 +77,21 @@ __device__ __forceinline__ float batch_max(const uint4 (&w)[SWEEP_UNROLL], float
 #pragma unroll
   for (int u = 1; u < SWEEP_UNROLL; ++u) m = fmaxf(m, vec_max(w[u], 0.f));
   return m;
+}
+
+// Logits past this are so far apart that only equal ones count in a sum of exp(x - max).
+constexpr float HUGE_LOGIT = 1e37f;
+template <typename T>
+__device__ __forceinline__ float count_equal(const uint4 (&w)[SWEEP_UNROLL], float m, T) {
+  int n = 0;
+#pragma unroll
+  for (int u = 0; u < SWEEP_UNROLL; ++u) {
+    float f[Vec<T>::N];
+    unpack(w[u], f, T());
+#pragma unroll
+    for (int j = 0; j < Vec<T>::N; ++j) n += f[j] == m ? 1 : 0;
+  }
+  return (float)n;
 }
 
 // Order-preserving map of a float (not NaN) to an unsigned key; -0 and +0 map alike.
@@ -271,7 +276,10 @@ __device__ __forceinline__ void sweep_batch(const uint4 (&w)[SWEEP_UNROLL], int 
     st.m = mx;
   }
   if constexpr (FIRST) publish(sm, warp, kout, st.m);
-  if (st.m != -INFINITY) {
+  if (fabsf(st.m) > HUGE_LOGIT) {
+    // m log2 e can overflow (a mask of the type's lowest value), and no other logit is close
+    if (st.m != -INFINITY) st.s += count_equal(w, st.m, T());
+  } else {
     const float nmb = -st.m * LOG2E;
     const float2 l2e = make_float2(LOG2E, LOG2E), off = make_float2(nmb, nmb);
     float2 acc0 = make_float2(0.f, 0.f), acc1 = make_float2(0.f, 0.f);
@@ -324,8 +332,7 @@ __device__ __forceinline__ void sweep_segment(const T* rowp, int V, int split, i
     float f = -INFINITY;
     if (in) {
       f = to_f32(rowp[lane]);
-      const float ff[1] = {f};
-      lse_update<1>(ff, f, st.m, st.s);
+      lse_update(f, st.m, st.s);
     }
     append(sm, warp, kout, in, f, lane, st);
   }
@@ -360,8 +367,7 @@ __device__ __forceinline__ void sweep_segment(const T* rowp, int V, int split, i
     float f = -INFINITY;
     if (e < V) {
       f = to_f32(rowp[e]);
-      const float ff[1] = {f};
-      lse_update<1>(ff, f, st.m, st.s);
+      lse_update(f, st.m, st.s);
     }
     append(sm, warp, kout, e < V, f, e, st);
   }

@@ -1,5 +1,5 @@
-"""GPU tests of the branches that the sizes of a call choose: the dense products' split of K and
-narrow tiles."""
+"""GPU tests of the branches that the sizes of a call choose: the sweep's buffers, threshold and
+segments on rows that stress them, the dense products' split of K and narrow tiles."""
 import numpy as np
 import pytest
 import torch
@@ -11,6 +11,57 @@ from test_parity_gpu import _run_and_check, _to, brisk  # noqa: F401  (brisk: a 
 pytestmark = pytest.mark.gpu
 
 BF16, F32 = torch.bfloat16, torch.float32
+
+
+def _rows(V, kind, dtype):
+    """[n, V] logits of one kind."""
+    g = torch.Generator().manual_seed(V)
+    x = torch.randn((5, V), generator=g)
+    if kind == "sorted":          # every logit raises the threshold / none after the first does
+        x = torch.sort(x, dim=1, descending=False).values
+        x[1::2] = x[1::2].flip(1)
+    elif kind == "masked":        # a few allowed ids, the rest at the type's lowest value
+        m = torch.full_like(x, torch.finfo(dtype).min)
+        for r in range(5):
+            at = torch.randperm(V, generator=g)[:6 + 9 * r]
+            m[r, at] = x[r, at]
+        x = m
+    elif kind == "infinite":      # fewer finite logits than candidates
+        m = torch.full_like(x, float("-inf"))
+        m[:, V // 2:V // 2 + 3] = x[:, :3]
+        x = m
+    elif kind == "ties":          # a handful of values
+        x = torch.round(x)
+    elif kind == "constant":
+        x = torch.full_like(x, 1.5)
+    return x.to(dtype).cuda()
+
+
+@pytest.mark.parametrize("K", [4, 8, 17, 32])
+@pytest.mark.parametrize("kind", ["normal", "sorted", "masked", "infinite", "ties", "constant"])
+@pytest.mark.parametrize("V,dtype", [(33, BF16), (2047, BF16), (16384 + 7, BF16), (70001, BF16),
+                                     (1000, F32), (8192, F32), (66000, F32)])
+def test_topk_against_a_stable_sort(brisk, V, dtype, kind, K):  # noqa: F811
+    """Rows shorter than one batch of one warp, of one batch a warp, and split into segments."""
+    x = _rows(V, kind, dtype)
+    B, L = 5, 1
+    tail = brisk.DecodeTail(B, L, V, 16, K, 16, dtype, BF16, _params(V))
+    got = tail.topk(x.view(B, L, V))
+    torch.cuda.synchronize()
+    want = torch.sort(x.float(), dim=1, descending=True, stable=True).indices[:, :K]
+    assert torch.equal(got["cand_ids"].view(B, K).long(), want)
+    lse = torch.logsumexp(x.double(), 1)
+    # sums of V positive fp32 terms, pairwise over lanes and warps: below 20 roundings of 2^-24
+    # each on the path of a term, and the logarithm's
+    assert torch.allclose(got["lse_q"].view(B).double(), lse, rtol=2e-6, atol=4e-6)
+    again = tail.topk(x.view(B, L, V))
+    assert all(torch.equal(got[k], again[k]) for k in got)
+
+
+def _params(V):
+    t = torch.zeros(8, dtype=BF16, device="cuda")
+    names = ("E_in", "E_out", "P_h", "P_e", "P_phi", "pos", "W0", "Wz", "Wh", "W_s", "W_c", "w_g")
+    return dict({n: t for n in names}, b_g=0.0, alpha=0.0)
 
 
 @pytest.mark.parametrize("dtype", [BF16, F32])
