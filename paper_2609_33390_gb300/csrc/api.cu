@@ -184,9 +184,12 @@ SweepSeg make_seg(const WsLayout& w, void* ws, int seg, const void* logits, int 
 // G = Hm[:BL] [W_z[:, :r] ; W_h[:, :r]]^T and G0 = Hm[BL:] W0[:, :r]^T. With bf16 weights the
 // products run on the tensor cores: the first one writes Hm as three bf16 parts, which the
 // second one multiplies by the weight blocks written three times along k (fp32-level accuracy).
+// `part` 1 enqueues the first products and 2 the second ones (both together: 1 | 2).
+enum { HIDDEN_FIRST = 1, HIDDEN_SECOND = 2, HIDDEN_BOTH = 3 };
 brisk_status hidden_products(const brisk_dims* d, const brisk_params* p, const void* tables,
                              const void* hidden, const void* h_ctx, const WsLayout& w, void* ws,
-                             cudaStream_t st, bool beside = false) {
+                             int part, cudaStream_t st, bool beside = false,
+                             cudaStream_t ctx_st = nullptr) {
   const TbLayout t = tb_layout(d);
   const int BL = d->B * d->L, r = d->r, S = 2 * d->r, hd = d->hidden_dtype;
   int32_t* status = at<int32_t>(ws, w.status);
@@ -197,23 +200,28 @@ brisk_status hidden_products(const brisk_dims* d, const brisk_params* p, const v
     const TcSpec first[2] = {
         {BL, r, d->d, hidden, d->d, p->P_h, d->d, 1, Hs, r3, nullptr, 0},
         {d->B, r, d->d, h_ctx, d->d, p->P_h, d->d, 1, Hs + (size_t)BL * r3, r3, nullptr, 0}};
-    BRISK_CUDA(gemm_tc_grouped(first, 2, status, st, beside));
+    if (part & HIDDEN_FIRST) BRISK_CUDA(gemm_tc_grouped(first, 2, status, st, beside));
     const TcSpec second[2] = {
         {BL, 2 * S, r3, Hs, r3, at<__nv_bfloat16>(tables, t.W2s), r3, 0, at<float>(ws, w.G), 2 * S,
          at<float>(tables, t.posG), d->L},
         {d->B, S, r3, Hs + (size_t)BL * r3, r3, at<__nv_bfloat16>(tables, t.W0s), r3, 0,
          at<float>(ws, w.G0), S, nullptr, 0}};
-    BRISK_CUDA(gemm_tc_grouped(second, 2, status, st, beside));
+    if (part & HIDDEN_SECOND) BRISK_CUDA(gemm_tc_grouped(second, 2, status, st, beside));
     return BRISK_OK;
   }
   float* Hm = at<float>(ws, w.Hm);
-  BRISK_CUDA(gemm_simt(BL, r, d->d, hidden, hd, d->d, p->P_h, hd, d->d, false, Hm, r, st));
-  BRISK_CUDA(gemm_simt(d->B, r, d->d, h_ctx, hd, d->d, p->P_h, hd, d->d, false,
-                       Hm + (size_t)BL * r, r, st));
-  BRISK_CUDA(gemm_simt(BL, 2 * S, r, Hm, BRISK_DT_F32, r, at<float>(tables, t.W2), BRISK_DT_F32, r,
-                       false, at<float>(ws, w.G), 2 * S, st, at<float>(tables, t.posG), d->L));
-  BRISK_CUDA(gemm_simt(d->B, S, r, Hm + (size_t)BL * r, BRISK_DT_F32, r, at<float>(tables, t.W0h),
-                       BRISK_DT_F32, r, false, at<float>(ws, w.G0), S, st));
+  float* Hc = Hm + (size_t)BL * r;
+  cudaStream_t cs = ctx_st ? ctx_st : st;   // the context's two products wait for no other
+  if (part & HIDDEN_FIRST) {
+    BRISK_CUDA(gemm_simt(BL, r, d->d, hidden, hd, d->d, p->P_h, hd, d->d, false, Hm, r, st));
+    BRISK_CUDA(gemm_simt(d->B, r, d->d, h_ctx, hd, d->d, p->P_h, hd, d->d, false, Hc, r, cs));
+  }
+  if (part & HIDDEN_SECOND) {
+    BRISK_CUDA(gemm_simt(BL, 2 * S, r, Hm, BRISK_DT_F32, r, at<float>(tables, t.W2), BRISK_DT_F32,
+                         r, false, at<float>(ws, w.G), 2 * S, st, at<float>(tables, t.posG), d->L));
+    BRISK_CUDA(gemm_simt(d->B, S, r, Hc, BRISK_DT_F32, r, at<float>(tables, t.W0h), BRISK_DT_F32, r,
+                         false, at<float>(ws, w.G0), S, cs));
+  }
   return BRISK_OK;
 }
 
@@ -439,7 +447,7 @@ brisk_status brisk_corrector_select(const brisk_dims* d, const brisk_params* p, 
   const WsLayout w = ws_layout(d);
   brisk_status s = clear_ws(w, d, ws, st);
   if (s != BRISK_OK) return s;
-  s = hidden_products(d, p, tables, hidden, h_ctx, w, ws, st);
+  s = hidden_products(d, p, tables, hidden, h_ctx, w, ws, HIDDEN_BOTH, st);
   if (s != BRISK_OK) return s;
   ScanArgs a = scan_args(d, p, tables, w, ws);
   a.select_mode = select_mode;
@@ -567,10 +575,25 @@ brisk_status brisk::decode_tail_locked(const brisk_dims* d, const brisk_params* 
   BRISK_CUDA(cudaStreamWaitEvent(ss->hi, ss->ev[0], 0));
   if (overlap) BRISK_CUDA(cudaStreamWaitEvent(m, ss->ev[0], 0));
   if (w.schedule != SCHEDULE_FUSED) BRISK_CUDA(cudaStreamWaitEvent(ss->lo, ss->ev[0], 0));
-  s = hidden_products(d, p, tables, io->hidden, io->h_ctx, w, ws, ss->hi,
-                      products_beside(w, d));
+  // without tensor cores the products are two chains of two; the middle stream is free for the
+  // shorter one unless the proposal rows are swept on it
+  const bool two_chains = !overlap && d->hidden_dtype == BRISK_DT_F32;
+  if (two_chains) BRISK_CUDA(cudaStreamWaitEvent(ss->mid, ss->ev[0], 0));
+  // The first products are enqueued before the proposal sweep, the second ones after it: a sweep
+  // that is enqueued last starts late (the host takes longer than the first product).
+  auto products = [&](int part) {
+    return hidden_products(d, p, tables, io->hidden, io->h_ctx, w, ws, part, ss->hi,
+                           products_beside(w, d), two_chains ? ss->mid : nullptr);
+  };
+  auto products_done = [&]() -> brisk_status {
+    const brisk_status r = products(HIDDEN_SECOND);
+    if (r != BRISK_OK) return r;
+    BRISK_CUDA(cudaEventRecord(ss->ev[1], ss->hi));
+    if (two_chains) BRISK_CUDA(cudaEventRecord(ss->ev[4], ss->mid));
+    return BRISK_OK;
+  };
+  s = products(HIDDEN_FIRST);
   if (s != BRISK_OK) return s;
-  BRISK_CUDA(cudaEventRecord(ss->ev[1], ss->hi));
 
   SweepLaunch sq{};
   sq.seg[0] = make_seg(w, ws, 0, io->logits_q, BL, d->K, cand_ids, cand_lp, lse_q);
@@ -607,8 +630,11 @@ brisk_status brisk::decode_tail_locked(const brisk_dims* d, const brisk_params* 
     BRISK_CUDA(launch_sweep(both, st));
     if (ev && ev->sweep_q_end) BRISK_CUDA(cudaEventRecord(static_cast<cudaEvent_t>(ev->sweep_q_end), st));
     if (ev && ev->sweep_p_end) BRISK_CUDA(cudaEventRecord(static_cast<cudaEvent_t>(ev->sweep_p_end), st));
+    s = products_done();
+    if (s != BRISK_OK) return s;
     // the corrector once the hidden products are done, verifying in the same CTA
     BRISK_CUDA(cudaStreamWaitEvent(st, ss->ev[1], 0));
+    if (two_chains) BRISK_CUDA(cudaStreamWaitEvent(st, ss->ev[4], 0));
     a.do_verify = 1;
     a.logits_p = io->logits_p;
     a.u_acc = io->u_acc;
@@ -624,6 +650,8 @@ brisk_status brisk::decode_tail_locked(const brisk_dims* d, const brisk_params* 
   if (ev && ev->sweep_q_begin) BRISK_CUDA(cudaEventRecord(static_cast<cudaEvent_t>(ev->sweep_q_begin), m));
   BRISK_CUDA(launch_sweep(sq, m));
   if (ev && ev->sweep_q_end) BRISK_CUDA(cudaEventRecord(static_cast<cudaEvent_t>(ev->sweep_q_end), m));
+  s = products_done();
+  if (s != BRISK_OK) return s;
   if (!overlap) {
     // SEPARATE: the verifier rows after the proposal rows, beside the corrector
     BRISK_CUDA(cudaEventRecord(ss->ev[2], m));
@@ -639,6 +667,7 @@ brisk_status brisk::decode_tail_locked(const brisk_dims* d, const brisk_params* 
 
   // the corrector once the proposal candidates and the hidden products are done
   BRISK_CUDA(cudaStreamWaitEvent(m, ss->ev[1], 0));
+  if (two_chains) BRISK_CUDA(cudaStreamWaitEvent(m, ss->ev[4], 0));
   BRISK_CUDA(launch_scan(a, m));
   BRISK_CUDA(cudaStreamWaitEvent(m, ss->ev[3], 0));
 
@@ -754,7 +783,7 @@ brisk_status brisk_replay_diagnostics(const brisk_dims* d, const brisk_params* p
   BRISK_CUDA(cudaEventRecord(ss->ev[0], st));
   BRISK_CUDA(cudaStreamWaitEvent(ss->hi, ss->ev[0], 0));
   BRISK_CUDA(cudaStreamWaitEvent(ss->mid, ss->ev[0], 0));
-  s = hidden_products(d, p, tables, hidden, h_ctx, w, ws, ss->hi, products_beside(w, d));
+  s = hidden_products(d, p, tables, hidden, h_ctx, w, ws, HIDDEN_BOTH, ss->hi, products_beside(w, d));
   if (s != BRISK_OK) return s;
   BRISK_CUDA(cudaEventRecord(ss->ev[1], ss->hi));
   SweepLaunch sq{};
