@@ -201,14 +201,11 @@ brisk_status brisk_verify_block(const brisk_dims *dims, const void *logits_p,
  * results, bit for bit, as brisk_topk_candidates + brisk_corrector_select + brisk_verify_block on
  * the same inputs. The work runs on library side streams of decreasing priority: the
  * hidden-state products; the proposal sweep, corrector and verification (the critical path);
- * the verifier-row sweep, which starts at once and fills the SMs the others leave free (this
- * applies whenever each proposal row is swept as one task: many rows, or rows too short to
- * split). When the batch is small enough that the proposal rows are swept in several chunks
- * each, the critical
- * path runs on `stream` itself: the verifier sweep starts after the proposal sweep, beside the
- * corrector; or, when both logit tensors together hold at most 64 MB, one sweep launch covers
- * the rows of both and the corrector kernel also verifies (brisk_kernels_per_tail counts the
- * launches). The call
+ * the verifier-row sweep, which starts at once (with fp32 hidden states and fewer than 2432
+ * rows after the proposal sweep) and fills the room the others leave free. When both logit
+ * tensors together hold at most 64 MB and their rows are not short, one sweep launch on `stream`
+ * covers the rows of both and the corrector kernel also verifies (brisk_kernels_per_tail counts
+ * the launches). The call
  * only enqueues work and the results are ordered on `stream` (the side streams fork from and
  * join back to it, also under graph capture). The first call in a CUDA context creates the side
  * streams and their events: make it before any stream capture. Calls from several host threads
@@ -256,9 +253,9 @@ int32_t brisk_kernels_per_tail(const brisk_dims *dims);
  * bounds). With clear != 0 the word is reset to BRISK_OK afterwards. */
 brisk_status brisk_last_device_status(void *workspace, int32_t clear, void *stream);
 
-/* Sets the limit, in SM clock cycles, of the bounded device-side waits (the tensor-core
- * products' pipeline and accumulator waits, which no other kernel has: the sweep, corrector and
- * verification kernels never wait on another CTA or on a copy). cycles <= 0 restores the default
+/* Sets the limit, in SM clock cycles, of the bounded device-side waits: the tensor-core
+ * products' pipeline and accumulator waits, and the corrector's waits for its candidates' table
+ * rows (the sweep and the verification kernel have none). cycles <= 0 restores the default
  * of 4e9 cycles (about 2 s). Returns the previous limit. The value is read when a launch is
  * enqueued and passed to the kernel (a captured graph keeps the value it was captured with); it
  * is process-wide. When a wait gives up, the call records BRISK_ERR_TIMEOUT in the device status,

@@ -30,14 +30,17 @@ bool dims_ok(const brisk_dims* d) {
 inline size_t esize(int dt) { return dt == BRISK_DT_BF16 ? 2 : 4; }
 
 // ---------------------------------------------------------------- workspace layout
-enum TailSchedule { SCHEDULE_OVERLAP = 0, SCHEDULE_SEPARATE = 1, SCHEDULE_FUSED = 2 };
-// Largest pair of logit tensors (bytes) for the fused small-batch schedule. Measured per block
-// (direct calls / graph replays): one sequence (16 MB) 124.9 / 106.4 us separate, 117.7 / 102.5
-// us fused; 16 sequences (259 MB, stochastic) 188.9 / 175.2 us separate, 243.6 / 210.6 fused.
+enum TailSchedule { SCHEDULE_OVERLAP = 0, SCHEDULE_FUSED = 1 };
+// Largest pair of logit tensors (bytes) for the fused schedule. Measured a tail of 32 positions,
+// V = 126464 bf16, greedy (fused / both sweeps overlapping): one sequence (16 MB) 56 / 58 us, four
+// (65 MB) 67 / 70, sixteen (259 MB) 101 / 88.
 constexpr size_t FUSE_MAX_BYTES = size_t(64) << 20;
-constexpr size_t OVERLAP_ROWS = 2432;      // proposal rows from which the sweeps overlap
+constexpr size_t FUSE_MIN_VECTORS = 2048;  // 16-byte vectors a row below which it does not pay
+// Rows below which fp32 products keep the verifier rows' sweep waiting: they run on the same units as
+// it and slow down beside two sweeps (16 sequences, d = 2048, S = 512: 115 us a tail, up to 126
+// with both from the start; 100 sequences: 355 with both from the start).
+constexpr size_t F32_ROWS = 2432;
 constexpr int BESIDE_STATE = 512;          // state width up to which the products share SMs with them
-constexpr size_t OVERLAP_VECTORS = 2048;   // 16-byte vectors a row below which they do
 
 struct WsLayout {
   size_t status, counters, part_val, part_id, part_m, part_s, argmax_p, lse_p;
@@ -53,13 +56,13 @@ WsLayout ws_layout(const brisk_dims* d) {
   w.nsplit = sweep_splits((int)BL, d->V, d->logits_dtype, d->K);
   // Schedule of the fused tail (every entry point sweeps a row the same way, so fused and separate
   // calls give the same bits):
-  //  OVERLAP  many rows, or rows of few vectors: the verifier rows' sweep from the start, on the
-  //           lowest priority;
-  //  FUSED    few rows and both logit tensors within FUSE_MAX_BYTES: both in one sweep launch;
-  //  SEPARATE otherwise: the verifier rows' sweep after the proposal rows', beside the corrector.
+  //  FUSED    few rows of many vectors, both logit tensors within FUSE_MAX_BYTES: both in one
+  //           sweep launch;
+  //  OVERLAP  otherwise: the verifier rows' sweep from the start, on the lowest priority (after the
+  //           proposal rows' sweep, 16 sequences took 99 us instead of 88, 48 194 instead of 164).
   const size_t row_bytes = (size_t)d->V * esize(d->logits_dtype);
-  if (BL >= OVERLAP_ROWS || row_bytes / 16 < OVERLAP_VECTORS) w.schedule = SCHEDULE_OVERLAP;
-  else w.schedule = 2 * BL * row_bytes <= FUSE_MAX_BYTES ? SCHEDULE_FUSED : SCHEDULE_SEPARATE;
+  const bool fused = row_bytes / 16 >= FUSE_MIN_VECTORS && 2 * BL * row_bytes <= FUSE_MAX_BYTES;
+  w.schedule = fused ? SCHEDULE_FUSED : SCHEDULE_OVERLAP;
   w.KP = kp_for(d->K);
   const size_t np = 2 * BL * (size_t)w.nsplit;
   size_t o = 0;
@@ -130,11 +133,10 @@ TbLayout tb_layout(const brisk_dims* d) {
 }
 
 // Whether the hidden products take the form that shares SMs with a sweep. Not in the fused
-// schedule (the sweep is as short as they are), nor for wide states beside whole-chip sweeps,
-// whose second product is four times larger (64 sequences, S = 1024: 525 us a tail, 625 so).
+// schedule (the sweep is as short as they are), nor for wide states, whose second product is four
+// times larger (64 sequences, S = 1024: 525 us a tail, 625 so).
 inline bool products_beside(const WsLayout& w, const brisk_dims* d) {
-  if (w.schedule == SCHEDULE_FUSED) return false;
-  return w.schedule == SCHEDULE_SEPARATE || 2 * d->r <= BESIDE_STATE;
+  return w.schedule == SCHEDULE_OVERLAP && 2 * d->r <= BESIDE_STATE;
 }
 
 template <typename T>
@@ -231,19 +233,22 @@ brisk_status hidden_products(const brisk_dims* d, const brisk_params* p, const v
 struct SideStream {
   unsigned long long ctx = 0;   // id of the context the streams belong to
   cudaStream_t hi = nullptr;    // highest priority: the hidden-state products
+  cudaStream_t hi2 = nullptr;   // highest priority: the context products where they are their own chain
   cudaStream_t mid = nullptr;   // middle priority: proposal sweep, corrector, verification
   cudaStream_t lo = nullptr;    // lowest priority: the verifier-row sweep
   cudaEvent_t ev[5] = {};
 };
 std::deque<SideStream> g_side;   // guarded by side_stream_mutex(); elements never move
 
-// The current context's side streams; the caller holds side_stream_mutex().
-SideStream* side_stream() {
+// The current context's side streams (with create false: only if they exist already); the caller
+// holds side_stream_mutex().
+SideStream* side_stream(bool create = true) {
   unsigned long long ctx = 0;
   if (!brisk::current_context_id(&ctx)) return nullptr;
   SideStream* found = nullptr;
   for (auto& e : g_side)
     if (e.ctx == ctx) found = &e;
+  if ((!found || !found->hi) && !create) return nullptr;
   if (!found) {
     g_side.emplace_back();
     found = &g_side.back();
@@ -253,8 +258,9 @@ SideStream* side_stream() {
   if (!ss.hi) {
     int least = 0, greatest = 0;
     if (cudaDeviceGetStreamPriorityRange(&least, &greatest) != cudaSuccess) return nullptr;
-    cudaStream_t hi = nullptr, mid = nullptr, lo = nullptr;
+    cudaStream_t hi = nullptr, hi2 = nullptr, mid = nullptr, lo = nullptr;
     if (cudaStreamCreateWithPriority(&hi, cudaStreamNonBlocking, greatest) != cudaSuccess ||
+        cudaStreamCreateWithPriority(&hi2, cudaStreamNonBlocking, greatest) != cudaSuccess ||
         cudaStreamCreateWithPriority(&mid, cudaStreamNonBlocking, (least + greatest) / 2) !=
             cudaSuccess ||
         cudaStreamCreateWithPriority(&lo, cudaStreamNonBlocking, least) != cudaSuccess)
@@ -263,6 +269,7 @@ SideStream* side_stream() {
       if (cudaEventCreateWithFlags(&e, cudaEventDisableTiming) != cudaSuccess) return nullptr;
     ss.lo = lo;
     ss.mid = mid;
+    ss.hi2 = hi2;
     ss.hi = hi;
   }
   return &ss;
@@ -554,19 +561,14 @@ brisk_status brisk::decode_tail_locked(const brisk_dims* d, const brisk_params* 
   //   H (highest): hidden products -----.
   //   M (middle) : proposal sweep ---- join -> corrector --- join -> verification -> join A
   //   W (lowest) : verifier sweep ---------------------------'
-  // The block scheduler places ready blocks of higher priority first. The products take their
-  // SMs first; the proposal sweep, on the critical path (proposal candidates -> corrector ->
-  // verification), takes the rest; the verifier sweep, needed only by the verification, starts
-  // at once but only fills room the other two leave: the proposal sweep's ragged end (one
-  // long task per row, ending over tens of microseconds) and the SMs beside the corrector.
-  // In this mode the products use wide tiles (fewer SMs held at the start).
-  // With chunked proposal rows (few rows) the short tasks end together and the critical path
-  // stays on A, the products (on the critical path there) using narrow tiles (more CTAs):
-  //  SEPARATE the verifier sweep starts after the proposal sweep, beside the corrector, which
-  //           saves the extra fork and keeps the SMs free for the corrector's start;
-  //  FUSED    (small tensors) one sweep launch on A covers the rows of both tensors, and the
-  //           corrector that follows it verifies its sequence in the same CTA (four launches
-  //           with two products, against six).
+  // The block scheduler places ready blocks of higher priority first. The products, tensor-core
+  // work within the sweep's carveout, share SMs with the proposal sweep, which is on the critical
+  // path (proposal candidates -> corrector -> verification); the verifier sweep, needed only by the
+  // verification, starts at once but only fills room the others leave: the proposal sweep's end
+  // and the SMs beside the corrector.
+  // FUSED (small tensors): one sweep launch on A covers the rows of both tensors, and the corrector
+  // that follows it verifies its sequence in the same CTA (four launches with two products, against
+  // six).
   const bool overlap = w.schedule == SCHEDULE_OVERLAP;
   SideStream* ss = side_stream();
   if (!ss) return BRISK_ERR_CUDA;
@@ -574,22 +576,22 @@ brisk_status brisk::decode_tail_locked(const brisk_dims* d, const brisk_params* 
   BRISK_CUDA(cudaEventRecord(ss->ev[0], st));
   BRISK_CUDA(cudaStreamWaitEvent(ss->hi, ss->ev[0], 0));
   if (overlap) BRISK_CUDA(cudaStreamWaitEvent(m, ss->ev[0], 0));
-  if (w.schedule != SCHEDULE_FUSED) BRISK_CUDA(cudaStreamWaitEvent(ss->lo, ss->ev[0], 0));
-  // without tensor cores the products are two chains of two; the middle stream is free for the
-  // shorter one unless the proposal rows are swept on it
-  const bool two_chains = !overlap && d->hidden_dtype == BRISK_DT_F32;
-  if (two_chains) BRISK_CUDA(cudaStreamWaitEvent(ss->mid, ss->ev[0], 0));
+  if (overlap) BRISK_CUDA(cudaStreamWaitEvent(ss->lo, ss->ev[0], 0));
+  // without tensor cores the products are two chains of two (8 sequences, d = 1024: 93 us a tail
+  // on one stream)
+  const bool two_chains = d->hidden_dtype == BRISK_DT_F32;
+  if (two_chains) BRISK_CUDA(cudaStreamWaitEvent(ss->hi2, ss->ev[0], 0));
   // The first products are enqueued before the proposal sweep, the second ones after it: a sweep
   // that is enqueued last starts late (the host takes longer than the first product).
   auto products = [&](int part) {
     return hidden_products(d, p, tables, io->hidden, io->h_ctx, w, ws, part, ss->hi,
-                           products_beside(w, d), two_chains ? ss->mid : nullptr);
+                           products_beside(w, d), two_chains ? ss->hi2 : nullptr);
   };
   auto products_done = [&]() -> brisk_status {
     const brisk_status r = products(HIDDEN_SECOND);
     if (r != BRISK_OK) return r;
     BRISK_CUDA(cudaEventRecord(ss->ev[1], ss->hi));
-    if (two_chains) BRISK_CUDA(cudaEventRecord(ss->ev[4], ss->mid));
+    if (two_chains) BRISK_CUDA(cudaEventRecord(ss->ev[4], ss->hi2));
     return BRISK_OK;
   };
   s = products(HIDDEN_FIRST);
@@ -618,7 +620,7 @@ brisk_status brisk::decode_tail_locked(const brisk_dims* d, const brisk_params* 
   a.u_sel = io->u_sel;
   a.sel_tokens = sel;
   a.refined = refined;
-  a.beside_sweep = w.schedule == SCHEDULE_OVERLAP;
+  a.beside_sweep = overlap;
 
   if (w.schedule == SCHEDULE_FUSED) {
     // both tensors' rows in one launch (the same layout and chunks as the separate calls)
@@ -652,13 +654,11 @@ brisk_status brisk::decode_tail_locked(const brisk_dims* d, const brisk_params* 
   if (ev && ev->sweep_q_end) BRISK_CUDA(cudaEventRecord(static_cast<cudaEvent_t>(ev->sweep_q_end), m));
   s = products_done();
   if (s != BRISK_OK) return s;
-  if (!overlap) {
-    // SEPARATE: the verifier rows after the proposal rows, beside the corrector
+  // verifier rows on the low-priority stream
+  if (d->hidden_dtype == BRISK_DT_F32 && BL < F32_ROWS) {
     BRISK_CUDA(cudaEventRecord(ss->ev[2], m));
     BRISK_CUDA(cudaStreamWaitEvent(ss->lo, ss->ev[2], 0));
   }
-
-  // verifier rows on the low-priority stream
   if (ev && ev->sweep_p_begin) BRISK_CUDA(cudaEventRecord(static_cast<cudaEvent_t>(ev->sweep_p_begin), ss->lo));
   BRISK_CUDA(launch_sweep(sp, ss->lo));
   // the join first: a timing record ahead of it would delay the verification behind it
@@ -687,10 +687,8 @@ brisk_status brisk::decode_tail_locked(const brisk_dims* d, const brisk_params* 
   v.correction = io->correction;
   v.next_anchor = io->next_anchor;
   BRISK_CUDA(launch_scan(v, m));
-  if (overlap) {
-    BRISK_CUDA(cudaEventRecord(ss->ev[4], m));
-    BRISK_CUDA(cudaStreamWaitEvent(st, ss->ev[4], 0));
-  }
+  BRISK_CUDA(cudaEventRecord(ss->ev[4], m));
+  BRISK_CUDA(cudaStreamWaitEvent(st, ss->ev[4], 0));
   return BRISK_OK;
 }
 
@@ -774,18 +772,26 @@ brisk_status brisk_replay_diagnostics(const brisk_dims* d, const brisk_params* p
   float* ref = refined ? refined : at<float>(ws, w.refined);
   // Three independent parts meet in two places: the hidden products and the candidates in the
   // corrector, the corrector and the verifier rows' log-partition in the comparison. The products
-  // run beside the proposal rows' sweep and the verifier rows' sweep beside the corrector, on side
-  // streams forked from the caller's, by priority (32 sequences: 213 us one after another, 155 us
-  // on the caller's stream and two more without priority for the corrector, 138 us so).
+  // run beside the proposal rows' sweep and the verifier rows' sweep beside the corrector, on the
+  // decode tail's side streams (32 sequences: 213 us one after another, 129 us so; 131 us with the
+  // verifier rows from the start, as little follows them here).
+  // A call under stream capture does not create them: without them everything stays on `stream`.
   std::lock_guard<std::mutex> lock(side_stream_mutex());
-  SideStream* ss = side_stream();
-  if (!ss) return BRISK_ERR_CUDA;
-  BRISK_CUDA(cudaEventRecord(ss->ev[0], st));
-  BRISK_CUDA(cudaStreamWaitEvent(ss->hi, ss->ev[0], 0));
-  BRISK_CUDA(cudaStreamWaitEvent(ss->mid, ss->ev[0], 0));
-  s = hidden_products(d, p, tables, hidden, h_ctx, w, ws, HIDDEN_BOTH, ss->hi, products_beside(w, d));
+  cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+  BRISK_CUDA(cudaStreamIsCapturing(st, &capture));
+  SideStream* ss = side_stream(capture == cudaStreamCaptureStatusNone);
+  if (!ss && capture == cudaStreamCaptureStatusNone) return BRISK_ERR_CUDA;
+  cudaStream_t hi = ss ? ss->hi : st, mid = ss ? ss->mid : st, lo = ss ? ss->lo : st;
+  // `to` goes on after everything enqueued on `from` so far
+  auto after = [&](cudaStream_t to, cudaStream_t from, int ev) {
+    if (!ss) return cudaSuccess;
+    const cudaError_t e = cudaEventRecord(ss->ev[ev], from);
+    return e != cudaSuccess ? e : cudaStreamWaitEvent(to, ss->ev[ev], 0);
+  };
+  BRISK_CUDA(after(hi, st, 0));
+  if (ss) BRISK_CUDA(cudaStreamWaitEvent(mid, ss->ev[0], 0));
+  s = hidden_products(d, p, tables, hidden, h_ctx, w, ws, HIDDEN_BOTH, hi, ss && products_beside(w, d));
   if (s != BRISK_OK) return s;
-  BRISK_CUDA(cudaEventRecord(ss->ev[1], ss->hi));
   SweepLaunch sq{};
   sq.seg[0] = make_seg(w, ws, 0, logits_q, BL, d->K, cand_ids, cand_lp, at<float>(ws, w.lse_q));
   sq.nseg = 1;
@@ -794,16 +800,14 @@ brisk_status brisk_replay_diagnostics(const brisk_dims* d, const brisk_params* p
   sq.KP = w.KP;
   sq.dtype = d->logits_dtype;
   sq.status = at<int32_t>(ws, w.status);
-  BRISK_CUDA(launch_sweep(sq, ss->mid));
-  BRISK_CUDA(cudaEventRecord(ss->ev[2], ss->mid));
-  BRISK_CUDA(cudaStreamWaitEvent(ss->lo, ss->ev[2], 0));
+  BRISK_CUDA(launch_sweep(sq, mid));
+  BRISK_CUDA(after(lo, mid, 2));
   SweepLaunch sp = sq;
   sp.seg[0] = make_seg(w, ws, 1, logits_p, BL, 1, at<int32_t>(ws, w.argmax_p), nullptr,
                        at<float>(ws, w.lse_p));
-  BRISK_CUDA(launch_sweep(sp, ss->lo));
-  BRISK_CUDA(cudaEventRecord(ss->ev[3], ss->lo));
+  BRISK_CUDA(launch_sweep(sp, lo));
   // the head along the factual base prefix
-  BRISK_CUDA(cudaStreamWaitEvent(ss->mid, ss->ev[1], 0));
+  BRISK_CUDA(after(mid, hi, 1));
   ScanArgs a = scan_args(d, p, tables, w, ws);
   a.select_mode = select_mode;
   a.do_select = 1;
@@ -816,9 +820,9 @@ brisk_status brisk_replay_diagnostics(const brisk_dims* d, const brisk_params* p
   a.refined = ref;
   a.base_prefix = 1;
   a.base_rank = at<int32_t>(ws, w.base_rank);
-  a.beside_sweep = 1;
-  BRISK_CUDA(launch_scan(a, ss->mid));
-  BRISK_CUDA(cudaStreamWaitEvent(ss->mid, ss->ev[3], 0));
+  a.beside_sweep = ss != nullptr;
+  BRISK_CUDA(launch_scan(a, mid));
+  BRISK_CUDA(after(mid, lo, 3));
   ReplayArgs r{};
   r.B = d->B; r.L = d->L; r.V = d->V; r.K = d->K; r.logits_dt = d->logits_dtype;
   r.logits_p = logits_p;
@@ -831,9 +835,8 @@ brisk_status brisk_replay_diagnostics(const brisk_dims* d, const brisk_params* p
   r.flags = flags;
   r.first_breaker = first_breaker;
   r.status = at<int32_t>(ws, w.status);
-  BRISK_CUDA(launch_replay(r, ss->mid));
-  BRISK_CUDA(cudaEventRecord(ss->ev[4], ss->mid));
-  BRISK_CUDA(cudaStreamWaitEvent(st, ss->ev[4], 0));
+  BRISK_CUDA(launch_replay(r, mid));
+  BRISK_CUDA(after(st, mid, 4));
   return BRISK_OK;
 }
 
