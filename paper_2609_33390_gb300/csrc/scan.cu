@@ -23,8 +23,8 @@ namespace {
 
 // Verification CTA: 128 threads, or 512 under stochastic verification, where a rejection
 // resamples from a residual over the whole vocabulary row (a 126464-entry row: 112 us on 128
-// threads with element loads and the precise exponential, a few us with 512 threads, vector
-// loads and the hardware one).
+// threads with element loads and the precise exponential, 28 with 512 threads, vector loads and
+// the hardware one, 12 with a cluster of 8 CTAs).
 constexpr int VERIFY_THREADS = 128;
 constexpr int VERIFY_THREADS_MAX = 512;
 constexpr int VERIFY_CTAS = 152;       // CTAs up to which a residual walk is shared
@@ -559,9 +559,10 @@ __device__ __forceinline__ float rcp_hw(float x) {
 __device__ __forceinline__ float sigmoid_hw(float x) { return rcp_hw(1.f + ex2(-LOG2E * x)); }
 
 // The sequential corrector (Sec. 3.3 Eqs. 4-5; App. C.3 Eq. 9; Algorithm 1(b) loop). What bounds
-// it is the number of instructions on the dependent chain of a position, and beside it the ones
-// that every warp repeats; so few warps compute and the rest of the work is done by others or
-// beforehand. A sequence has ceil(S / 128) computing warps that own four state elements a lane.
+// it is the number of instructions on the dependent chain of a position (a lone warp issues one
+// about every 8 cycles), and beside it the ones that every warp repeats; so few warps compute and
+// the rest of the work is done by others or beforehand (32 positions, S = 512, K = 8: one sequence
+// 41 us with eight computing warps that load for themselves, now 27; 16 sampled ones 63, now 41). A sequence has ceil(S / 128) computing warps that own four state elements a lane.
 // A position is:
 //  - the minimal-GRU step on the lane's elements, its residual-dot and gate partials (packed
 //    fp32 pairs), a warp reduce-scatter, the warps' parts to shared memory, one barrier;
