@@ -191,7 +191,7 @@ enum { HIDDEN_FIRST = 1, HIDDEN_SECOND = 2, HIDDEN_BOTH = 3 };
 brisk_status hidden_products(const brisk_dims* d, const brisk_params* p, const void* tables,
                              const void* hidden, const void* h_ctx, const WsLayout& w, void* ws,
                              int part, cudaStream_t st, bool beside = false,
-                             cudaStream_t ctx_st = nullptr) {
+                             cudaStream_t ctx_st = nullptr, cudaEvent_t started = nullptr) {
   const TbLayout t = tb_layout(d);
   const int BL = d->B * d->L, r = d->r, S = 2 * d->r, hd = d->hidden_dtype;
   int32_t* status = at<int32_t>(ws, w.status);
@@ -202,7 +202,7 @@ brisk_status hidden_products(const brisk_dims* d, const brisk_params* p, const v
     const TcSpec first[2] = {
         {BL, r, d->d, hidden, d->d, p->P_h, d->d, 1, Hs, r3, nullptr, 0},
         {d->B, r, d->d, h_ctx, d->d, p->P_h, d->d, 1, Hs + (size_t)BL * r3, r3, nullptr, 0}};
-    if (part & HIDDEN_FIRST) BRISK_CUDA(gemm_tc_grouped(first, 2, status, st, beside));
+    if (part & HIDDEN_FIRST) BRISK_CUDA(gemm_tc_grouped(first, 2, status, st, beside, started));
     const TcSpec second[2] = {
         {BL, 2 * S, r3, Hs, r3, at<__nv_bfloat16>(tables, t.W2s), r3, 0, at<float>(ws, w.G), 2 * S,
          at<float>(tables, t.posG), d->L},
@@ -236,7 +236,7 @@ struct SideStream {
   cudaStream_t hi2 = nullptr;   // highest priority: the context products where they are their own chain
   cudaStream_t mid = nullptr;   // middle priority: proposal sweep, corrector, verification
   cudaStream_t lo = nullptr;    // lowest priority: the verifier-row sweep
-  cudaEvent_t ev[5] = {};
+  cudaEvent_t ev[6] = {};
 };
 std::deque<SideStream> g_side;   // guarded by side_stream_mutex(); elements never move
 
@@ -789,9 +789,15 @@ brisk_status brisk_replay_diagnostics(const brisk_dims* d, const brisk_params* p
     return e != cudaSuccess ? e : cudaStreamWaitEvent(to, ss->ev[ev], 0);
   };
   BRISK_CUDA(after(hi, st, 0));
-  if (ss) BRISK_CUDA(cudaStreamWaitEvent(mid, ss->ev[0], 0));
-  s = hidden_products(d, p, tables, hidden, h_ctx, w, ws, HIDDEN_BOTH, hi, ss && products_beside(w, d));
+  // A sweep that is placed first leaves the products no room until its rows end (129 us in some
+  // processes, 134 to 144 in others), so it waits until they have begun (130 in all; under capture
+  // until their fork: the graph orders the launches).
+  const bool live = ss && capture == cudaStreamCaptureStatusNone;
+  if (ss) BRISK_CUDA(cudaEventRecord(ss->ev[5], hi));
+  s = hidden_products(d, p, tables, hidden, h_ctx, w, ws, HIDDEN_BOTH, hi, ss && products_beside(w, d),
+                      nullptr, live ? ss->ev[5] : nullptr);
   if (s != BRISK_OK) return s;
+  if (ss) BRISK_CUDA(cudaStreamWaitEvent(mid, ss->ev[5], 0));
   SweepLaunch sq{};
   sq.seg[0] = make_seg(w, ws, 0, logits_q, BL, d->K, cand_ids, cand_lp, at<float>(ws, w.lse_q));
   sq.nseg = 1;

@@ -238,10 +238,11 @@ __device__ __forceinline__ void fence_async_smem() {
 // into a CUDA graph keep launch attributes, but not the priority of the stream they were captured
 // from, so without it a replay of the tail's three-priority schedule runs every kernel at the
 // default priority.
-// With cluster > 1 the grid runs as clusters of that many CTAs.
+// With cluster > 1 the grid runs as clusters of that many CTAs. `started`, if not null, is recorded
+// to fire once all of them have begun.
 template <typename... KArgs, typename... Args>
-inline cudaError_t launch_cluster(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem,
-                                  cudaStream_t stream, int cluster, Args&&... args) {
+inline cudaError_t launch_started(cudaEvent_t started, void (*kernel)(KArgs...), dim3 grid, dim3 block,
+                                  size_t smem, cudaStream_t stream, int cluster, Args&&... args) {
   int prio = 0;
   cudaError_t e = cudaStreamGetPriority(stream, &prio);
   if (e != cudaSuccess) return e;
@@ -250,15 +251,30 @@ inline cudaError_t launch_cluster(void (*kernel)(KArgs...), dim3 grid, dim3 bloc
   cfg.blockDim = block;
   cfg.dynamicSmemBytes = smem;
   cfg.stream = stream;
-  cudaLaunchAttribute attr[2];
+  cudaLaunchAttribute attr[3];
   attr[0].id = cudaLaunchAttributePriority;
   attr[0].val.priority = prio;
-  attr[1].id = cudaLaunchAttributeClusterDimension;
-  attr[1].val.clusterDim.x = (unsigned)cluster;
-  attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
   cfg.attrs = attr;
-  cfg.numAttrs = cluster > 1 ? 2 : 1;
+  cfg.numAttrs = 1;
+  if (cluster > 1) {
+    cudaLaunchAttribute& c = attr[cfg.numAttrs++];
+    c.id = cudaLaunchAttributeClusterDimension;
+    c.val.clusterDim.x = (unsigned)cluster;
+    c.val.clusterDim.y = c.val.clusterDim.z = 1;
+  }
+  if (started) {
+    cudaLaunchAttribute& c = attr[cfg.numAttrs++];
+    c.id = cudaLaunchAttributeLaunchCompletionEvent;
+    c.val.launchCompletionEvent.event = started;
+    c.val.launchCompletionEvent.flags = 0;
+  }
   return cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...);
+}
+template <typename... KArgs, typename... Args>
+inline cudaError_t launch_cluster(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem,
+                                  cudaStream_t stream, int cluster, Args&&... args) {
+  return launch_started(nullptr, kernel, grid, block, smem, stream, cluster,
+                        std::forward<Args>(args)...);
 }
 template <typename... KArgs, typename... Args>
 inline cudaError_t launch_prio(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem,
@@ -363,9 +379,9 @@ struct TcSpec {
   int bias_period;
 };
 // beside: the products run beside the sweeps and should share SMs with them (the results are the
-// same bit for bit).
+// same bit for bit). started: recorded to fire once every CTA has begun.
 cudaError_t gemm_tc_grouped(const TcSpec* spec, int nprob, int32_t* status, cudaStream_t stream,
-                            bool beside = false);
+                            bool beside = false, cudaEvent_t started = nullptr);
 bool gemm_tc_supported(const void* A, int lda, const void* B, int ldb, int K);
 // The folds that read the corrector's weights alone, in one launch: see brisk_corrector_prepare.
 struct PackArgs {

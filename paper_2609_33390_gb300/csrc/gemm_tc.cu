@@ -512,7 +512,7 @@ bool gemm_tc_supported(const void* A, int lda, const void* B, int ldb, int K) {
 // wins: up to one CTA an SM, K split while there is room, a 4-stage pipeline; with more tiles
 // than SMs, 2-stage CTAs share an SM in pairs, one multiplying while the other stores.
 cudaError_t gemm_tc_grouped(const TcSpec* spec, int nprob, int32_t* status, cudaStream_t stream,
-                            bool beside) {
+                            bool beside, cudaEvent_t started) {
   if (nprob < 1 || nprob > 2) return cudaErrorInvalidValue;
   int nmax = 0, nk_min = 0, nk_max = 0;
   for (int i = 0; i < nprob; ++i) {
@@ -591,7 +591,7 @@ cudaError_t gemm_tc_grouped(const TcSpec* spec, int nprob, int32_t* status, cuda
                                        static_cast<int>(smem));
   if (e == cudaSuccess) e = prefer_carveout(kernel, beside ? CARVEOUT_SMALL_KB : CARVEOUT_FULL_KB);
   if (e != cudaSuccess) return e;
-  e = launch_cluster(kernel, dim3(total * split), dim3(TC_THREADS), smem, stream, split, maps, a);
+  e = launch_started(started, kernel, dim3(total * split), dim3(TC_THREADS), smem, stream, split, maps, a);
   if (e != cudaSuccess) return e;
   return cudaGetLastError();
 }
