@@ -86,19 +86,23 @@ __device__ __forceinline__ float batch_max(const uint4 (&w)[SWEEP_UNROLL], float
   return m;
 }
 
-// Logits past this are so far apart that only equal ones count in a sum of exp(x - max).
-constexpr float HUGE_LOGIT = 1e37f;
+// Sum of exp(x - m) of a lane's batch for m past FAR_LOGIT in size. The main path multiplies first,
+// fma(x, log2 e, -(m log2 e)), and so returns the rounding of m log2 e where x equals m: up to half
+// an ulp of m, as the log-partition's own rounding, but 2^-25 of m as an exponent, which overflows
+// on a lane whose logits are all a mask of -1e10 (and spoils the row: inf times zero, later). Here
+// the difference comes first, which is exact for logits close enough to count.
+constexpr float FAR_LOGIT = 1e6f;
 template <typename T>
-__device__ __forceinline__ float count_equal(const uint4 (&w)[SWEEP_UNROLL], float m, T) {
-  int n = 0;
+__device__ __forceinline__ float sum_far(const uint4 (&w)[SWEEP_UNROLL], float m, T) {
+  float s = 0.f;
 #pragma unroll
   for (int u = 0; u < SWEEP_UNROLL; ++u) {
     float f[Vec<T>::N];
     unpack(w[u], f, T());
 #pragma unroll
-    for (int j = 0; j < Vec<T>::N; ++j) n += f[j] == m ? 1 : 0;
+    for (int j = 0; j < Vec<T>::N; ++j) s += ex2((f[j] - m) * LOG2E);
   }
-  return (float)n;
+  return s;
 }
 
 // Order-preserving map of a float (not NaN) to an unsigned key; -0 and +0 map alike.
@@ -283,9 +287,8 @@ __device__ __forceinline__ void sweep_batch(const uint4 (&w)[SWEEP_UNROLL], int 
     st.m = mx;
   }
   if constexpr (FIRST) publish(sm, warp, kout, st.m);
-  if (fabsf(st.m) > HUGE_LOGIT) {
-    // m log2 e can overflow (a mask of the type's lowest value), and no other logit is close
-    if (st.m != -INFINITY) st.s += count_equal(w, st.m, T());
+  if (fabsf(st.m) > FAR_LOGIT) {
+    if (st.m != -INFINITY) st.s += sum_far(w, st.m, T());
   } else {
     const float nmb = -st.m * LOG2E;
     const float2 l2e = make_float2(LOG2E, LOG2E), off = make_float2(nmb, nmb);

@@ -58,6 +58,30 @@ def test_topk_against_a_stable_sort(brisk, V, dtype, kind, K):  # noqa: F811
     assert all(torch.equal(got[k], again[k]) for k in got)
 
 
+@pytest.mark.parametrize("dtype", [BF16, F32])
+@pytest.mark.parametrize("V", [1000, 16384 + 7, 70001])
+@pytest.mark.parametrize("mask", [-1e4, -1e9, -1e10, -1e20, -1e30, 1e10])
+def test_masked_ranges(brisk, mask, V, dtype):  # noqa: F811
+    """A whole range of the vocabulary at one far value (every lane of some batches holds nothing
+    else; last, every logit of a row), so that no exponential of the others is lost or spoilt."""
+    g = torch.Generator().manual_seed(V)
+    x = torch.randn((4, V), generator=g)
+    x[0, V // 8:] = mask
+    x[1, :V - 100] = mask
+    x[2] = mask
+    x[3, ::2] = mask
+    x = x.to(dtype).cuda()
+    tail = brisk.DecodeTail(4, 1, V, 16, 8, 16, dtype, BF16, _params(V))
+    got = tail.topk(x.view(4, 1, V))
+    torch.cuda.synchronize()
+    assert tail.device_status() == brisk.OK
+    want = torch.sort(x.float(), dim=1, descending=True, stable=True).indices[:, :8]
+    assert torch.equal(got["cand_ids"].view(4, 8).long(), want)
+    lse = torch.logsumexp(x.double(), 1)
+    # as above, and the rounding of the far value's product with log2 e: an ulp of it
+    assert torch.allclose(got["lse_q"].view(4).double(), lse, rtol=2e-6, atol=4e-6)
+
+
 def _params(V):
     t = torch.zeros(8, dtype=BF16, device="cuda")
     names = ("E_in", "E_out", "P_h", "P_e", "P_phi", "pos", "W0", "Wz", "Wh", "W_s", "W_c", "w_g")
