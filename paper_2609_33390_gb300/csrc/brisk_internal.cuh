@@ -346,7 +346,7 @@ struct SweepLaunch {
   SweepSeg seg[2];
   int nseg;
   int V;
-  int nsplit;             // segments (CTAs) per row
+  int nsplit;             // segments (CTAs) per row; 1 where a warp sweeps a row
   int KP;
   int dtype;              // brisk_dtype of the logits
   int32_t* status;

@@ -2,24 +2,24 @@
 // (Sec. 3.3 "C_i = TopK(q_i, K)"; App. C.3 ordered candidate set), and for
 // verifier rows the argmax (lowest id on ties) and the log-partition.
 //
-// Work unit: one CTA of SWEEP_WARPS warps sweeps one row, or one of nsplit equal segments of a
-// row when there are too few rows to fill the chip. Its warps take the segment's batches in turn
-// (32 lanes x SWEEP_UNROLL 16-byte streaming loads, all in flight at once). Each lane keeps a
-// running (max, sum of exp) pair. The lanes' maxima also give the top-K's threshold: every warp
-// publishes its few largest, each of them a logit of the segment, and the K-th largest of all
-// published ones is a lower bound on the segment's K-th best. A batch whose largest logit is
-// below the threshold costs one comparison; a logit that reaches it (about K (1 + ln(batches)) of
-// them a row) is appended to the warp's buffer. At the end every buffered entry that reaches the
-// final threshold counts the entries that precede it, which is its place. The segments of a row
-// are merged the same way by the last of them to finish (arrival counter, no waiting). Which
-// logits are buffered depends on timing; the outputs do not.
+// Two layouts, by the rows and their length (by_warp). Many rows, or short ones: a warp sweeps a row
+// alone (sweep_rows_kernel). Else one CTA of SWEEP_WARPS warps sweeps one row, or one of nsplit
+// equal segments of a row when there are too few rows to fill the chip:
 //
-// Large tensors are bound by the rate at which an SM takes and handles 16-byte vectors (about 45
-// GB/s of logits each, 0.86 to 1 of a copy's rate over the chip), small ones by the threshold's
-// and the merge's latency. A threshold shared by the CTA's warps is why a row is one CTA's: with a
-// list of its own in every warp, each warp paid for its own insertions (128 x 32 rows of 126464
-// bf16: proposal rows, K = 8, 175 us, now 170; verifier rows 181, now 152; 16 x 32 proposal rows
-// 50, now 28; 32 proposal rows 29, now 10).
+// Its warps take the segment's batches in turn (32 lanes x SWEEP_UNROLL 16-byte streaming loads, all
+// in flight at once). Each lane keeps a running (max, sum of exp) pair. The lanes' maxima also give
+// the top-K's threshold: every warp publishes its few largest, each of them a logit of the segment,
+// and the K-th largest of all published ones is a lower bound on the segment's K-th best. A batch
+// whose largest logit is below the threshold costs one comparison; a logit that reaches it (about
+// K (1 + ln(batches)) of them a row) is appended to the warp's buffer. At the end every buffered
+// entry that reaches the final threshold counts the entries that precede it, which is its place. The
+// segments of a row are merged the same way by the last of them to finish (arrival counter, no
+// waiting). Which logits are buffered depends on timing; the outputs do not.
+//
+// Large tensors are bound by memory (see by_warp), small ones by the threshold's and the merge's
+// latency. A threshold shared by the CTA's warps is why a row is one CTA's where there are few rows:
+// with a list of its own in every warp, each warp paid for its own insertions (16 x 32 rows of 126464
+// bf16, K = 8: 50 us, now 28; 32 rows 29, now 10).
 #include "brisk_internal.cuh"
 
 namespace brisk {
@@ -35,6 +35,14 @@ constexpr int SWEEP_BUF = 64;                           // entries a warp buffer
 constexpr int SWEEP_MERGE = SWEEP_WARPS * SWEEP_BUF;    // entries merged at most
 constexpr int SWEEP_TOPS = 32 / SWEEP_WARPS;            // maxima a warp publishes
 constexpr int SWEEP_RAISE = 3;                          // entries between raises of the threshold
+
+// The warp-a-row layout.
+constexpr int ROW_WARPS = 2;                            // rows a CTA sweeps
+constexpr int ROW_CARVEOUT_KB = 64;
+constexpr int ROW_SHORT = 3 * SWEEP_BATCH + 33;         // vectors below which every row takes it
+constexpr int ROW_MANY = 152 * 16;                      // rows from which every length takes it
+constexpr int ROW_MID = 152 * 12;                       // rows from which ROW_MID_VECTORS do
+constexpr int ROW_MID_VECTORS = 8192;
 
 // Online log-sum-exp of one logit.
 __device__ __forceinline__ void lse_update(float f, float& m, float& s) {
@@ -67,6 +75,12 @@ __device__ __forceinline__ float vec_max(const uint4& w, float) {
                fmaxf(__uint_as_float(w.z), __uint_as_float(w.w)));
 }
 
+__device__ __forceinline__ float vec_max(const uint4& w, __nv_bfloat16) {
+  const __nv_bfloat162* v = reinterpret_cast<const __nv_bfloat162*>(&w);
+  const __nv_bfloat162 c = __hmax2(__hmax2(v[0], v[1]), __hmax2(v[2], v[3]));
+  return fmaxf(__low2float(c), __high2float(c));
+}
+
 // Max of a lane's whole batch (bf16: packed maxima, 4 instructions a vector).
 __device__ __forceinline__ float batch_max(const uint4 (&w)[SWEEP_UNROLL], __nv_bfloat16) {
   __nv_bfloat162 m[4];
@@ -94,15 +108,57 @@ __device__ __forceinline__ float batch_max(const uint4 (&w)[SWEEP_UNROLL], float
 constexpr float FAR_LOGIT = 1e6f;
 template <typename T>
 __device__ __forceinline__ float sum_far(const uint4 (&w)[SWEEP_UNROLL], float m, T) {
-  float s = 0.f;
+  const float2 off = make_float2(-m, -m), l2e = make_float2(LOG2E, LOG2E);
+  float2 s = make_float2(0.f, 0.f);
 #pragma unroll
   for (int u = 0; u < SWEEP_UNROLL; ++u) {
     float f[Vec<T>::N];
     unpack(w[u], f, T());
 #pragma unroll
-    for (int j = 0; j < Vec<T>::N; ++j) s += ex2((f[j] - m) * LOG2E);
+    for (int j = 0; j < Vec<T>::N; j += 2) {
+      const float2 arg = __fmul2_rn(__fadd2_rn(make_float2(f[j], f[j + 1]), off), l2e);
+      s = __fadd2_rn(s, make_float2(ex2(arg.x), ex2(arg.y)));
+    }
   }
-  return s;
+  return s.x + s.y;
+}
+
+// A batch in a lane's running (max, sum of exp): the max first (returns the batch's own), which moves
+// once per batch, so that all of its exponentials share one offset; then the sum, arguments and
+// parts in packed fp32 pairs.
+template <typename T>
+__device__ __forceinline__ float raise_max(const uint4 (&w)[SWEEP_UNROLL], float& m, float& s) {
+  const float mx = batch_max(w, T());
+  if (mx > m) {
+    s *= ex2((m - mx) * LOG2E);
+    m = mx;
+  }
+  return mx;
+}
+template <typename T>
+__device__ __forceinline__ void add_batch(const uint4 (&w)[SWEEP_UNROLL], float m, float& s) {
+  constexpr int VN = Vec<T>::N;
+  if (fabsf(m) > FAR_LOGIT) {
+    if (m != -INFINITY) s += sum_far(w, m, T());
+  } else {
+    const float nmb = -m * LOG2E;
+    const float2 l2e = make_float2(LOG2E, LOG2E), off = make_float2(nmb, nmb);
+    float2 acc0 = make_float2(0.f, 0.f), acc1 = make_float2(0.f, 0.f);
+#pragma unroll
+    for (int u = 0; u < SWEEP_UNROLL; ++u) {
+      float f[VN];
+      unpack(w[u], f, T());
+#pragma unroll
+      for (int j = 0; j < VN; j += 2) {
+        const float2 arg = __ffma2_rn(make_float2(f[j], f[j + 1]), l2e, off);
+        const float2 e = make_float2(ex2(arg.x), ex2(arg.y));
+        if ((j / 2 + u) & 1) acc1 = __fadd2_rn(acc1, e);
+        else acc0 = __fadd2_rn(acc0, e);
+      }
+    }
+    const float2 acc = __fadd2_rn(acc0, acc1);
+    s += acc.x + acc.y;
+  }
 }
 
 // Order-preserving map of a float (not NaN) to an unsigned key; -0 and +0 map alike.
@@ -273,41 +329,14 @@ __device__ __forceinline__ void offer_batch(const uint4 (&w)[SWEEP_UNROLL], floa
 }
 
 // One batch: SWEEP_UNROLL vectors per lane, lane's vector u holding ids id0_lane + 32 u VN + j;
-// vectors u >= valid are padding (-inf) and are never appended. The running max moves once per
-// batch, so all of the batch's exponentials share one offset; arguments and sums use packed fp32
-// pairs.
+// vectors u >= valid are padding (-inf) and are never appended.
 template <typename T, bool FIRST>
 __device__ __forceinline__ void sweep_batch(const uint4 (&w)[SWEEP_UNROLL], int id0_lane, int valid,
                                             int kout, SweepSmem& sm, WarpState& st) {
-  constexpr int VN = Vec<T>::N;
   const int warp = threadIdx.x >> 5;
-  const float mx = batch_max(w, T());
-  if (mx > st.m) {
-    st.s *= ex2((st.m - mx) * LOG2E);
-    st.m = mx;
-  }
+  const float mx = raise_max<T>(w, st.m, st.s);
   if constexpr (FIRST) publish(sm, warp, kout, st.m);
-  if (fabsf(st.m) > FAR_LOGIT) {
-    if (st.m != -INFINITY) st.s += sum_far(w, st.m, T());
-  } else {
-    const float nmb = -st.m * LOG2E;
-    const float2 l2e = make_float2(LOG2E, LOG2E), off = make_float2(nmb, nmb);
-    float2 acc0 = make_float2(0.f, 0.f), acc1 = make_float2(0.f, 0.f);
-#pragma unroll
-    for (int u = 0; u < SWEEP_UNROLL; ++u) {
-      float f[VN];
-      unpack(w[u], f, T());
-#pragma unroll
-      for (int j = 0; j < VN; j += 2) {
-        const float2 arg = __ffma2_rn(make_float2(f[j], f[j + 1]), l2e, off);
-        const float2 e = make_float2(ex2(arg.x), ex2(arg.y));
-        if ((j / 2 + u) & 1) acc1 = __fadd2_rn(acc1, e);
-        else acc0 = __fadd2_rn(acc0, e);
-      }
-    }
-    const float2 acc = __fadd2_rn(acc0, acc1);
-    st.s += acc.x + acc.y;
-  }
+  add_batch<T>(w, st.m, st.s);
   if constexpr (FIRST) {   // every warp has published its maxima before anyone needs them
     __syncthreads();
     st.thr = segment_threshold(sm, kout);
@@ -438,6 +467,19 @@ __device__ __forceinline__ void merge_by_rank(SweepSmem& sm, int n, int kout) {
   __syncthreads();
 }
 
+// A row's outputs, by one warp: its (max, sum of exp) and, in lane k < kout, the k-th best.
+__device__ __forceinline__ void write_row(const SweepSeg& sg, size_t row, int kout, float m, float s,
+                                          float v, int id, int32_t* status) {
+  const int lane = threadIdx.x & 31;
+  const float lse = m + logf(s);
+  if (!isfinite(lse) && lane == 0) set_status(status, BRISK_ERR_NUMERIC);
+  if (lane < kout) {
+    sg.out_ids[row * kout + lane] = id;
+    if (sg.out_logprob) sg.out_logprob[row * kout + lane] = v - lse;
+  }
+  if (lane == 0) sg.out_lse[row] = lse;
+}
+
 // At most 64 registers a thread: four CTAs of eight warps an SM.
 template <typename T>
 __global__ void __launch_bounds__(SWEEP_WARPS * 32, SWEEP_RESIDENT)
@@ -508,20 +550,164 @@ sweep_kernel(const __grid_constant__ SweepLaunch a) {
       if (lane == 0) sg.counters[row] = 0;
     }
   }
-  if (warp != 0) return;
-  const float lse = m + logf(s);
-  if (!isfinite(lse) && lane == 0) set_status(a.status, BRISK_ERR_NUMERIC);
-  if (lane < kout) {
-    sg.out_ids[(size_t)row * kout + lane] = sm.best_i[lane];
-    if (sg.out_logprob) sg.out_logprob[(size_t)row * kout + lane] = sm.best_v[lane] - lse;
+  if (warp == 0) write_row(sg, row, kout, m, s, sm.best_v[lane], sm.best_i[lane], a.status);
+}
+
+
+// ---------------------------------------------------------------- a warp a row
+// Many rows, or short ones: a warp sweeps a row alone and keeps its best-first list over the lanes
+// (lane k holds the k-th best), into which the few logits that reach the K-th best are inserted one
+// by one. Bound by memory from some 3000 rows (4096 rows of 126464 bf16, K = 8: 6.7 TB/s) given L1 for
+// its loads in flight, 128 KB an SM: with 100 KB of shared memory carved out instead of 64, 185 us
+// instead of 156.
+struct RowState {
+  float m, s;      // this lane's running max and sum of exp(x - max)
+  float wv;        // this lane's entry of the list
+  int wi;
+  float thr;       // lower bound on the row's K-th best, the same in all lanes
+};
+
+// Inserts (v, id), the same in all lanes; entries past kout keep (-inf, INVALID_ID).
+__device__ __forceinline__ void list_insert(float v, int id, int kout, RowState& st) {
+  const int lane = threadIdx.x & 31;
+  const bool ahead = lane < kout && !better(v, id, st.wv, st.wi);   // entries that stay before it
+  const int pos = __popc(__ballot_sync(FULL_MASK, ahead));
+  const float uv = __shfl_up_sync(FULL_MASK, st.wv, 1);
+  const int ui = __shfl_up_sync(FULL_MASK, st.wi, 1);
+  if (lane < kout && lane >= pos) {
+    st.wv = lane == pos ? v : uv;
+    st.wi = lane == pos ? id : ui;
   }
-  if (lane == 0) sg.out_lse[row] = lse;
+  st.thr = fmaxf(st.thr, __shfl_sync(FULL_MASK, st.wv, kout - 1));
+}
+
+// Inserts the lanes' elements f (ids id) that reach the threshold and come before the list's last
+// (not the many at a mask's value once the list is full of them).
+__device__ __forceinline__ void insert_lanes(bool in, float f, int id, int kout, RowState& st) {
+  const float last_v = __shfl_sync(FULL_MASK, st.wv, kout - 1);
+  const int last_i = __shfl_sync(FULL_MASK, st.wi, kout - 1);
+  unsigned hit = __ballot_sync(FULL_MASK, in && f >= st.thr && better(f, id, last_v, last_i));
+  while (hit) {
+    const int src = __ffs(hit) - 1;
+    hit &= hit - 1;
+    const float v = __shfl_sync(FULL_MASK, f, src);
+    const int i = __shfl_sync(FULL_MASK, id, src);
+    if (v >= st.thr) list_insert(v, i, kout, st);
+  }
+}
+
+// One batch (as in sweep_batch). stash: 32 vectors of shared memory.
+template <typename T>
+__device__ __forceinline__ void row_batch(const uint4 (&w)[SWEEP_UNROLL], int id0_lane, int valid,
+                                          int kout, uint4* stash, RowState& st) {
+  constexpr int VN = Vec<T>::N;
+  const int lane = threadIdx.x & 31;
+  const float mx = raise_max<T>(w, st.m, st.s);
+  add_batch<T>(w, st.m, st.s);
+  const unsigned lanes = __ballot_sync(FULL_MASK, valid > 0 && mx >= st.thr);
+  if (!lanes) return;
+  if (__popc(lanes) >= kout) {   // kout lanes each hold a logit at least as large as this
+    const unsigned key = order_key(mx);
+    const unsigned kth = kout == 1 ? __reduce_max_sync(FULL_MASK, key)
+                                   : __shfl_sync(FULL_MASK, warp_sort(key), 32 - kout);
+    st.thr = fmaxf(st.thr, key_to_float(kth));
+  }
+#pragma unroll
+  for (int u = 0; u < SWEEP_UNROLL; ++u) {
+    unsigned hit = __ballot_sync(FULL_MASK, u < valid && vec_max(w[u], T()) >= st.thr);
+    if (!hit) continue;
+    stash[lane] = w[u];
+    __syncwarp();
+    do {   // lane j < VN reads logit j of the vector of lane src
+      const int src = __ffs(hit) - 1;
+      hit &= hit - 1;
+      const T* e = reinterpret_cast<const T*>(stash + src);
+      const float f = lane < VN ? to_f32(e[lane]) : -INFINITY;
+      const int id = __shfl_sync(FULL_MASK, id0_lane, src) + u * 32 * VN + lane;
+      insert_lanes(lane < VN, f, id, kout, st);
+    } while (hit);
+    __syncwarp();
+  }
+  // ids only grow from one batch to the next: a later logit has to exceed a full list's last
+  const float last = __shfl_sync(FULL_MASK, st.wv, kout - 1);
+  if (__shfl_sync(FULL_MASK, st.wi, kout - 1) != INVALID_ID)
+    st.thr = fmaxf(st.thr, nextafterf(last, INFINITY));
+}
+
+// At most 64 registers a thread: 32 rows an SM.
+template <typename T>
+__global__ void __launch_bounds__(ROW_WARPS * 32, 32 / ROW_WARPS)
+sweep_rows_kernel(const __grid_constant__ SweepSeg sg, int V, int32_t* status) {
+  constexpr int VN = Vec<T>::N;
+  __shared__ uint4 stash[ROW_WARPS][32];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int row = (int)blockIdx.x * ROW_WARPS + warp;
+  if (row >= sg.rows) return;
+  const int kout = sg.kout;
+  const T* rowp = reinterpret_cast<const T*>(sg.logits) + (size_t)row * V;
+  const uintptr_t addr = reinterpret_cast<uintptr_t>(rowp);
+  const int head = min(V, (int)(((16u - (unsigned)(addr & 15u)) & 15u) / sizeof(T)));
+  const int nvec = (V - head) / VN;
+  RowState st{-INFINITY, 0.f, -INFINITY, INVALID_ID, -INFINITY};
+  // the unaligned head and, at the end, the ragged tail: fewer than VN logits each
+  auto ragged = [&](int first, int n) {
+    const bool in = lane < n;
+    const float f = in ? to_f32(rowp[first + lane]) : -INFINITY;
+    if (in) lse_update(f, st.m, st.s);
+    insert_lanes(in, f, first + lane, kout, st);
+  };
+  ragged(0, head);
+  const uint4* vp = reinterpret_cast<const uint4*>(rowp + head) + lane;
+  const uint32_t ninf = VN == 8 ? 0xff80ff80u : 0xff800000u;
+  uint4 w[SWEEP_UNROLL];
+  int base = 0;
+  auto load = [&]() -> int {   // padded with -inf past the row
+    const int left = nvec - base - lane;
+    const int valid = left <= 0 ? 0 : min(SWEEP_UNROLL, (left + 31) / 32);
+#pragma unroll
+    for (int u = 0; u < SWEEP_UNROLL; ++u)
+      w[u] = u < valid ? ld_stream_v4(vp + base + 32 * u) : make_uint4(ninf, ninf, ninf, ninf);
+    return valid;
+  };
+  int valid = load();
+  row_batch<T>(w, head + lane * VN, valid, kout, stash[warp], st);
+  // full batches: no bounds checks
+  for (base = SWEEP_BATCH; base + SWEEP_BATCH <= nvec; base += SWEEP_BATCH) {
+#pragma unroll
+    for (int u = 0; u < SWEEP_UNROLL; ++u) w[u] = ld_stream_v4(vp + base + 32 * u);
+    row_batch<T>(w, head + (base + lane) * VN, SWEEP_UNROLL, kout, stash[warp], st);
+  }
+  if (base < nvec) {
+    valid = load();
+    row_batch<T>(w, head + (base + lane) * VN, valid, kout, stash[warp], st);
+  }
+  ragged(head + nvec * VN, V - head - nvec * VN);
+  warp_lse_combine(st.m, st.s);
+  write_row(sg, row, kout, st.m, st.s, st.wv, st.wi, status);
+}
+
+// Whether a warp sweeps a row alone. In short rows fewer than four warps of a CTA have a logit in
+// every lane, too few for K <= 32 maxima to be published, and nothing would be screened out (4096 bf16
+// rows of 1000, K = 8: 161 us on a CTA a row, 16 so; 32 rows of 4000, K = 32: 91, 27). And where one warp a row fills the chip it
+// spares the CTA's barriers and merge (4096 rows of 16000, K = 8: 53 us, 33; of 126464: 175, 156).
+// With fewer rows a long one wants more warps (2048 rows, K = 8: of 32000 44 us, 40; of 64000 62, 62;
+// of 126464 98, 101; 1536 of 32000: 36, 38; 1024 of 16000: 20, 24).
+bool by_warp(int rows, int V, int dtype) {
+  const int nvec = V / (dtype == BRISK_DT_BF16 ? 8 : 4);
+  return nvec < ROW_SHORT || rows >= ROW_MANY || (rows >= ROW_MID && nvec <= ROW_MID_VECTORS);
 }
 
 template <typename T>
 cudaError_t launch_t(const SweepLaunch& a, cudaStream_t stream) {
   long long rows = a.seg[0].rows;
   if (a.nseg > 1) rows += a.seg[1].rows;
+  if (by_warp(a.seg[0].rows, a.V, a.dtype)) {
+    cudaError_t e = prefer_carveout(sweep_rows_kernel<T>, ROW_CARVEOUT_KB);
+    for (int i = 0; i < a.nseg && e == cudaSuccess; ++i)
+      e = launch_prio(sweep_rows_kernel<T>, dim3((unsigned)((a.seg[i].rows + ROW_WARPS - 1) / ROW_WARPS)),
+                      dim3(ROW_WARPS * 32), 0, stream, a.seg[i], a.V, a.status);
+    return e != cudaSuccess ? e : cudaGetLastError();
+  }
   cudaError_t e = prefer_carveout(sweep_kernel<T>, CARVEOUT_SMALL_KB);
   if (e != cudaSuccess) return e;
   e = launch_prio(sweep_kernel<T>, dim3((unsigned)(rows * a.nsplit)), dim3(SWEEP_WARPS * 32), 0, stream, a);
@@ -544,6 +730,7 @@ int kp_for(int K) {
 int sweep_splits(int rows_per_tensor, int V, int dtype, int K) {
   const int vn = dtype == BRISK_DT_BF16 ? 8 : 4;
   const int batches = (V / vn + SWEEP_BATCH - 1) / SWEEP_BATCH;
+  if (by_warp(rows_per_tensor, V, dtype)) return 1;
   int c = SWEEP_CTAS / rows_per_tensor;
   const int most = (batches + SWEEP_WARPS - 1) / SWEEP_WARPS;
   if (c > most) c = most;

@@ -82,6 +82,28 @@ def test_masked_ranges(brisk, mask, V, dtype):  # noqa: F811
     assert torch.allclose(got["lse_q"].view(4).double(), lse, rtol=2e-6, atol=4e-6)
 
 
+@pytest.mark.parametrize("K", [8, 32])
+@pytest.mark.parametrize("rows,V,dtype", [(5, 6407, BF16), (5, 6415, BF16), (1823, 9001, BF16),
+                                          (1824, 9001, BF16), (1824, 65601, BF16),
+                                          (2431, 70001, BF16), (2432, 70001, BF16),
+                                          (3, 3203, F32), (3, 3207, F32), (2433, 4999, F32)])
+def test_layout_borders(brisk, rows, V, dtype, K):  # noqa: F811
+    """Both sides of the rows and lengths at which a warp, not a CTA, takes a row."""
+    g = torch.Generator("cuda").manual_seed(V + rows)
+    x = torch.randn((rows, V), generator=g, device="cuda").to(dtype)
+    tail = brisk.DecodeTail(rows, 1, V, 16, K, 16, dtype, BF16, _params(V))
+    got = tail.topk(x.view(rows, 1, V))
+    step = 512
+    for s in range(0, rows, step):
+        part = x[s:s + step]
+        want = torch.sort(part.float(), dim=1, descending=True, stable=True).indices[:, :K]
+        assert torch.equal(got["cand_ids"].view(rows, K)[s:s + step].long(), want)
+        lse = torch.logsumexp(part.double(), 1)
+        # sums as above
+        assert torch.allclose(got["lse_q"].view(rows)[s:s + step].double(), lse, rtol=2e-6,
+                              atol=4e-6)
+
+
 def _params(V):
     t = torch.zeros(8, dtype=BF16, device="cuda")
     names = ("E_in", "E_out", "P_h", "P_e", "P_phi", "pos", "W0", "Wz", "Wh", "W_s", "W_c", "w_g")
