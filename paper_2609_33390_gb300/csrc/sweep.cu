@@ -275,7 +275,7 @@ __device__ __forceinline__ void append(SweepSmem& sm, int warp, int kout, bool i
   const bool want = in && f >= st.thr && better(f, id, st.kv, st.ki);
   unsigned hit = __ballot_sync(FULL_MASK, want);
   if (!hit) return;
-  if (st.count + 32 > SWEEP_BUF) {
+  if (st.count + __popc(hit) > SWEEP_BUF) {
     trim_buffer(sm, warp, kout, st);
     hit = __ballot_sync(FULL_MASK, want && better(f, id, st.kv, st.ki));
   }
