@@ -145,6 +145,12 @@ __device__ __forceinline__ void warp_lse_combine(float& m, float& s) {
   s = t;
 }
 
+// ---------------------------------------------------------------- contexts
+// Unique id of the CUDA context current on this thread (cuCtxGetId; ids are never reused, so a
+// device reset, which creates a new context, gives a new id). False when no context is current
+// or the driver entry points are unavailable.
+bool current_context_id(unsigned long long* id);
+
 // Shared-memory carveouts (KB) the kernels ask for. An SM cannot change its L1/shared split
 // while a CTA is resident, and the first kernel to land on an idle SM sets it, so a kernel that
 // runs beside another one (the sweep beside the dense products, the verifier-row sweep beside
@@ -154,30 +160,39 @@ __device__ __forceinline__ void warp_lse_combine(float& m, float& s) {
 // 100, 132 KB: 395, 381, 389 us.
 constexpr int CARVEOUT_SMALL_KB = 100;   // sweep (5.5 KB a CTA), corrector, verification
 constexpr int CARVEOUT_FULL_KB = 228;    // dense products, except beside the sweeps
-// Sets the carveout preference of `func` on the current device once (kernels of the same
-// signature are distinct entries: the registry is keyed by the function's address).
-inline cudaError_t prefer_carveout_fn(const void* func, int kb) {
+// Prepares `func` in the current context, once: its carveout preference and, for a kernel with dynamic
+// shared memory, the most that a block of it may have (process-wide state that another thread's call
+// must not lower between this one's and its launch). cudaErrorInvalidValue if `smem` bytes do not fit.
+inline cudaError_t set_up_kernel_fn(const void* func, int kb, size_t smem) {
+  struct Entry { const void* func; unsigned long long ctx; size_t most; };
   static std::mutex mu;
-  static std::vector<std::pair<const void*, int>> done;
-  int dev = 0;
-  cudaError_t e = cudaGetDevice(&dev);
-  if (e != cudaSuccess) return e;
+  static std::vector<Entry> done;
   std::lock_guard<std::mutex> lock(mu);
+  unsigned long long ctx = 0;
+  const bool known = current_context_id(&ctx);   // (a device reset makes a new context)
   for (const auto& d : done)
-    if (d.first == func && d.second == dev) return cudaSuccess;
-  int max_smem = 0;
-  e = cudaDeviceGetAttribute(&max_smem, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev);
+    if (known && d.func == func && d.ctx == ctx) return smem <= d.most ? cudaSuccess : cudaErrorInvalidValue;
+  int dev = 0, per_sm = 0, per_block = 0;
+  cudaFuncAttributes fa;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, func);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&per_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&per_block, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
   if (e != cudaSuccess) return e;
-  int pct = max_smem > 0 ? (kb * 1024 * 100 + max_smem - 1) / max_smem : 100;
+  int pct = per_sm > 0 ? (kb * 1024 * 100 + per_sm - 1) / per_sm : 100;
   if (pct > 100) pct = 100;
   e = cudaFuncSetAttribute(func, cudaFuncAttributePreferredSharedMemoryCarveout, pct);
-  if (e == cudaSuccess) done.emplace_back(func, dev);
-  return e;
+  const size_t most = smem > 0 ? (size_t)per_block - fa.sharedSizeBytes : 0;
+  if (e == cudaSuccess && smem > 0)
+    e = cudaFuncSetAttribute(func, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most);
+  if (e != cudaSuccess) return e;
+  if (known) done.push_back({func, ctx, most});
+  return smem <= most ? cudaSuccess : cudaErrorInvalidValue;
 }
 
 template <typename Kernel>
-inline cudaError_t prefer_carveout(Kernel kernel, int kb) {
-  return prefer_carveout_fn(reinterpret_cast<const void*>(kernel), kb);
+inline cudaError_t set_up_kernel(Kernel kernel, int kb, size_t smem = 0) {
+  return set_up_kernel_fn(reinterpret_cast<const void*>(kernel), kb, smem);
 }
 
 // ---------------------------------------------------------------- mbarriers and bulk copies
@@ -474,12 +489,6 @@ cudaError_t launch_replay(const ReplayArgs& a, cudaStream_t stream);
 
 size_t scan_smem_bytes(int L, int K, int S, int V);
 cudaError_t launch_scan(const ScanArgs& a, cudaStream_t stream);
-
-// ---------------------------------------------------------------- contexts
-// Unique id of the CUDA context current on this thread (cuCtxGetId; ids are never reused, so a
-// device reset, which creates a new context, gives a new id). False when no context is current
-// or the driver entry points are unavailable.
-bool current_context_id(unsigned long long* id);
 
 // ---------------------------------------------------------------- fused tail
 // Serialises the use of the library's side streams: held while one call enqueues on them, and

@@ -587,9 +587,7 @@ cudaError_t gemm_tc_grouped(const TcSpec* spec, int nprob, int32_t* status, cuda
   const size_t smem = gemm_tc_smem(BN, stages);
   auto kernel = beside ? gemm_tc_kernel<2, true>
                       : (stages == 2 ? gemm_tc_kernel<2> : gemm_tc_kernel<4>);
-  cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       static_cast<int>(smem));
-  if (e == cudaSuccess) e = prefer_carveout(kernel, beside ? CARVEOUT_SMALL_KB : CARVEOUT_FULL_KB);
+  cudaError_t e = set_up_kernel(kernel, beside ? CARVEOUT_SMALL_KB : CARVEOUT_FULL_KB, smem);
   if (e != cudaSuccess) return e;
   e = launch_started(started, kernel, dim3(total * split), dim3(TC_THREADS), smem, stream, split, maps, a);
   if (e != cudaSuccess) return e;

@@ -886,8 +886,7 @@ cudaError_t launch_corrector_k(const ScanArgs& a, cudaStream_t stream) {
   const size_t smem = corr_layout(a.L, a.K, a.S, a.V, a.ring_depth,
                                   corr_stage(a.K, a.S, a.tok_ranks, ROWS), VERIFY, nullptr, nullptr);
   auto kernel = corrector_kernel<NP, ROWS, SAMPLE, VERIFY>;
-  cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e == cudaSuccess) e = prefer_carveout(kernel, CARVEOUT_SMALL_KB);
+  cudaError_t e = set_up_kernel(kernel, CARVEOUT_SMALL_KB, smem);
   if (e != cudaSuccess) return e;
   const int threads = 32 * ((a.S + CORR_SPAN - 1) / CORR_SPAN) + CORR_OTHERS;
   e = launch_prio(kernel, dim3(a.B), dim3(threads), smem, stream, a);
@@ -950,9 +949,7 @@ cudaError_t launch_scan(const ScanArgs& a, cudaStream_t stream) {
     while (v.parts < 8 && 2 * v.parts * a.B <= VERIFY_CTAS && a.V >= 2 * v.parts * VERIFY_SHARE)
       v.parts *= 2;
   const size_t smem = scan_smem_bytes(a.L, a.K, a.S, a.V);
-  cudaError_t e = cudaFuncSetAttribute(verify_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)smem);
-  if (e == cudaSuccess) e = prefer_carveout(verify_kernel, CARVEOUT_SMALL_KB);
+  cudaError_t e = set_up_kernel(verify_kernel, CARVEOUT_SMALL_KB, smem);
   if (e != cudaSuccess) return e;
   const int threads = a.verify_mode == BRISK_VERIFY_STOCHASTIC ? VERIFY_THREADS_MAX : VERIFY_THREADS;
   e = launch_cluster(verify_kernel, dim3(a.B * v.parts), dim3(threads), smem, stream, v.parts, v);

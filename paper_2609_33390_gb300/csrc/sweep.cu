@@ -702,13 +702,13 @@ cudaError_t launch_t(const SweepLaunch& a, cudaStream_t stream) {
   long long rows = a.seg[0].rows;
   if (a.nseg > 1) rows += a.seg[1].rows;
   if (by_warp(a.seg[0].rows, a.V, a.dtype)) {
-    cudaError_t e = prefer_carveout(sweep_rows_kernel<T>, ROW_CARVEOUT_KB);
+    cudaError_t e = set_up_kernel(sweep_rows_kernel<T>, ROW_CARVEOUT_KB);
     for (int i = 0; i < a.nseg && e == cudaSuccess; ++i)
       e = launch_prio(sweep_rows_kernel<T>, dim3((unsigned)((a.seg[i].rows + ROW_WARPS - 1) / ROW_WARPS)),
                       dim3(ROW_WARPS * 32), 0, stream, a.seg[i], a.V, a.status);
     return e != cudaSuccess ? e : cudaGetLastError();
   }
-  cudaError_t e = prefer_carveout(sweep_kernel<T>, CARVEOUT_SMALL_KB);
+  cudaError_t e = set_up_kernel(sweep_kernel<T>, CARVEOUT_SMALL_KB);
   if (e != cudaSuccess) return e;
   e = launch_prio(sweep_kernel<T>, dim3((unsigned)(rows * a.nsplit)), dim3(SWEEP_WARPS * 32), 0, stream, a);
   if (e != cudaSuccess) return e;
