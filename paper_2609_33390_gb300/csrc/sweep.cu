@@ -40,9 +40,8 @@ constexpr int SWEEP_RAISE = 3;                          // entries between raise
 constexpr int ROW_WARPS = 2;                            // rows a CTA sweeps
 constexpr int ROW_CARVEOUT_KB = 64;
 constexpr int ROW_SHORT = 3 * SWEEP_BATCH + 33;         // vectors below which every row takes it
-constexpr int ROW_MANY = 152 * 16;                      // rows from which every length takes it
-constexpr int ROW_MID = 152 * 12;                       // rows from which ROW_MID_VECTORS do
-constexpr int ROW_MID_VECTORS = 8192;
+constexpr int ROW_MID = 152 * 12;                       // rows from which three times as many vectors do
+constexpr int ROW_MANY = 152 * 16;                      // rows from which every length does for K > 16
 
 // Online log-sum-exp of one logit.
 __device__ __forceinline__ void lse_update(float f, float& m, float& s) {
@@ -686,22 +685,26 @@ sweep_rows_kernel(const __grid_constant__ SweepSeg sg, int V, int32_t* status) {
   write_row(sg, row, kout, st.m, st.s, st.wv, st.wi, status);
 }
 
-// Whether a warp sweeps a row alone. In short rows fewer than four warps of a CTA have a logit in
-// every lane, too few for K <= 32 maxima to be published, and nothing would be screened out (4096 bf16
-// rows of 1000, K = 8: 161 us on a CTA a row, 16 so; 32 rows of 4000, K = 32: 91, 27). And where one warp a row fills the chip it
-// spares the CTA's barriers and merge (4096 rows of 16000, K = 8: 53 us, 33; of 126464: 175, 156).
-// With fewer rows a long one wants more warps (2048 rows, K = 8: of 32000 44 us, 40; of 64000 62, 62;
-// of 126464 98, 101; 1536 of 32000: 36, 38; 1024 of 16000: 20, 24).
-bool by_warp(int rows, int V, int dtype) {
+// Whether a warp sweeps a row alone (KP: K or a power of two above it). In short rows fewer than four
+// warps of a CTA have a logit in every lane, too few for K <= 32 maxima to be published, and nothing
+// would be screened out (4096 bf16 rows of 1000, K = 8: 161 us on a CTA a row, 16 so; 32 rows of
+// 4000, K = 32: 91, 27). And where one warp a row fills the chip it spares the CTA's barriers and merge
+// (4096 rows of 16000, K = 8: 53 us, 33; 2048 of 32000: 44, 40; of 64000: 62, 62; of 126464: 98, 101;
+// 1536 of 32000: 36, 38). Past 3 vectors a row's length for every row a call of these rows alone
+// still gains (4096 of 126464, K = 8: 175 us, 156), but beside the products of a tail it depends on
+// which kernel is placed first (128 sequences: 372 or 374 us on a CTA a row, 352 or 379 so; 64 of 64
+// rows of 151936: 524 or 533, 539 or 534; 2560 rows of 104000: 222, 234); with K > 16 it stays well
+// ahead (4096 of 126464: 326, 197).
+bool by_warp(int rows, int V, int dtype, int KP) {
   const int nvec = V / (dtype == BRISK_DT_BF16 ? 8 : 4);
-  return nvec < ROW_SHORT || rows >= ROW_MANY || (rows >= ROW_MID && nvec <= ROW_MID_VECTORS);
+  return nvec < ROW_SHORT || (rows >= ROW_MID && nvec <= 3ll * rows) || (rows >= ROW_MANY && KP > 16);
 }
 
 template <typename T>
 cudaError_t launch_t(const SweepLaunch& a, cudaStream_t stream) {
   long long rows = a.seg[0].rows;
   if (a.nseg > 1) rows += a.seg[1].rows;
-  if (by_warp(a.seg[0].rows, a.V, a.dtype)) {
+  if (by_warp(a.seg[0].rows, a.V, a.dtype, a.KP)) {
     cudaError_t e = set_up_kernel(sweep_rows_kernel<T>, ROW_CARVEOUT_KB);
     for (int i = 0; i < a.nseg && e == cudaSuccess; ++i)
       e = launch_prio(sweep_rows_kernel<T>, dim3((unsigned)((a.seg[i].rows + ROW_WARPS - 1) / ROW_WARPS)),
@@ -730,7 +733,7 @@ int kp_for(int K) {
 int sweep_splits(int rows_per_tensor, int V, int dtype, int K) {
   const int vn = dtype == BRISK_DT_BF16 ? 8 : 4;
   const int batches = (V / vn + SWEEP_BATCH - 1) / SWEEP_BATCH;
-  if (by_warp(rows_per_tensor, V, dtype)) return 1;
+  if (by_warp(rows_per_tensor, V, dtype, K)) return 1;
   int c = SWEEP_CTAS / rows_per_tensor;
   const int most = (batches + SWEEP_WARPS - 1) / SWEEP_WARPS;
   if (c > most) c = most;

@@ -86,6 +86,7 @@ def test_masked_ranges(brisk, mask, V, dtype):  # noqa: F811
 @pytest.mark.parametrize("rows,V,dtype", [(5, 6407, BF16), (5, 6415, BF16), (1823, 9001, BF16),
                                           (1824, 9001, BF16), (1824, 65601, BF16),
                                           (2431, 70001, BF16), (2432, 70001, BF16),
+                                          (2433, 58381, BF16), (2433, 58401, BF16),
                                           (3, 3203, F32), (3, 3207, F32), (2433, 4999, F32)])
 def test_layout_borders(brisk, rows, V, dtype, K):  # noqa: F811
     """Both sides of the rows and lengths at which a warp, not a CTA, takes a row."""
