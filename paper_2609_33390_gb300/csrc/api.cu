@@ -275,6 +275,22 @@ SideStream* side_stream(bool create = true) {
   return &ss;
 }
 
+// Joins what a call that fails between its fork and its join has enqueued on the side streams back to
+// its own stream, so that the caller's next work there may reuse the buffers.
+struct SideJoin {
+  SideStream* ss;
+  cudaStream_t st;
+  bool joined = false;
+  ~SideJoin() {
+    cudaStreamCaptureStatus own, side;
+    if (joined || !ss || cudaStreamIsCapturing(st, &own) != cudaSuccess) return;
+    for (cudaStream_t s : {ss->hi, ss->hi2, ss->mid, ss->lo}) {
+      if (cudaStreamIsCapturing(s, &side) != cudaSuccess || side != own) continue;   // not forked
+      if (cudaEventRecord(ss->ev[0], s) == cudaSuccess) (void)cudaStreamWaitEvent(st, ss->ev[0], 0);
+    }
+  }
+};
+
 ScanArgs scan_args(const brisk_dims* d, const brisk_params* p, const void* tables, const WsLayout& w,
                    void* ws) {
   ScanArgs a{};
@@ -572,6 +588,7 @@ brisk_status brisk::decode_tail_locked(const brisk_dims* d, const brisk_params* 
   const bool overlap = w.schedule == SCHEDULE_OVERLAP;
   SideStream* ss = side_stream();
   if (!ss) return BRISK_ERR_CUDA;
+  SideJoin join{ss, st};
   cudaStream_t m = overlap ? ss->mid : st;
   BRISK_CUDA(cudaEventRecord(ss->ev[0], st));
   BRISK_CUDA(cudaStreamWaitEvent(ss->hi, ss->ev[0], 0));
@@ -646,6 +663,7 @@ brisk_status brisk::decode_tail_locked(const brisk_dims* d, const brisk_params* 
     a.correction = io->correction;
     a.next_anchor = io->next_anchor;
     BRISK_CUDA(launch_scan(a, st));
+    join.joined = true;
     return BRISK_OK;
   }
 
@@ -689,6 +707,7 @@ brisk_status brisk::decode_tail_locked(const brisk_dims* d, const brisk_params* 
   BRISK_CUDA(launch_scan(v, m));
   BRISK_CUDA(cudaEventRecord(ss->ev[4], m));
   BRISK_CUDA(cudaStreamWaitEvent(st, ss->ev[4], 0));
+  join.joined = true;
   return BRISK_OK;
 }
 
@@ -781,6 +800,7 @@ brisk_status brisk_replay_diagnostics(const brisk_dims* d, const brisk_params* p
   BRISK_CUDA(cudaStreamIsCapturing(st, &capture));
   SideStream* ss = side_stream(capture == cudaStreamCaptureStatusNone);
   if (!ss && capture == cudaStreamCaptureStatusNone) return BRISK_ERR_CUDA;
+  SideJoin join{ss, st};
   cudaStream_t hi = ss ? ss->hi : st, mid = ss ? ss->mid : st, lo = ss ? ss->lo : st;
   // `to` goes on after everything enqueued on `from` so far
   auto after = [&](cudaStream_t to, cudaStream_t from, int ev) {
@@ -843,6 +863,7 @@ brisk_status brisk_replay_diagnostics(const brisk_dims* d, const brisk_params* p
   r.status = at<int32_t>(ws, w.status);
   BRISK_CUDA(launch_replay(r, mid));
   BRISK_CUDA(after(st, mid, 4));
+  join.joined = true;
   return BRISK_OK;
 }
 
