@@ -207,7 +207,8 @@ brisk_status brisk_verify_block(const brisk_dims *dims, const void *logits_p,
  * covers the rows of both and the corrector kernel also verifies (brisk_kernels_per_tail counts
  * the launches). The call
  * only enqueues work and the results are ordered on `stream` (the side streams fork from and
- * join back to it, also under graph capture). The first call in a CUDA context creates the side
+ * join back to it, also under graph capture, where they belong to the capture until it ends: no other
+ * tail may be enqueued meanwhile). The first call in a CUDA context creates the side
  * streams and their events: make it before any stream capture. Calls from several host threads
  * are serialised while they enqueue, and brisk_tail_graph_create holds that serialisation for
  * the whole of its capture. `ev` may be NULL.
@@ -309,7 +310,11 @@ brisk_status brisk_acceptance_weights(int32_t M, const double *a, const double *
  * rejects), bit 3 = intervention (head token != base token), bit 4 = rescue (J(base) = 0 and
  * J(head) = 1 at the first breaker), bit 5 = regression (J(head) = 0 at a position before the
  * first breaker, where J(base) = 1); first_breaker [B] int32 (L if none); refined [B, L, K]
- * f32 or NULL. */
+ * f32 or NULL.
+ * The sweeps and products run concurrently on the side streams of brisk_decode_tail, forked from
+ * `stream` and joined back to it, so that calls from several host threads are serialised while they
+ * enqueue and their work shares those streams. Under capture, and while a caller's own capture of a
+ * tail holds the side streams, all of it runs on `stream`, one after another, with the same results. */
 brisk_status brisk_replay_diagnostics(const brisk_dims *dims, const brisk_params *params,
                                       const void *tables, const void *hidden, const void *h_ctx,
                                       const int32_t *x0, const void *logits_q,

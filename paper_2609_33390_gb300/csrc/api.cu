@@ -240,15 +240,13 @@ struct SideStream {
 };
 std::deque<SideStream> g_side;   // guarded by side_stream_mutex(); elements never move
 
-// The current context's side streams (with create false: only if they exist already); the caller
-// holds side_stream_mutex().
-SideStream* side_stream(bool create = true) {
+// The current context's side streams; the caller holds side_stream_mutex().
+SideStream* side_stream() {
   unsigned long long ctx = 0;
   if (!brisk::current_context_id(&ctx)) return nullptr;
   SideStream* found = nullptr;
   for (auto& e : g_side)
     if (e.ctx == ctx) found = &e;
-  if ((!found || !found->hi) && !create) return nullptr;
   if (!found) {
     g_side.emplace_back();
     found = &g_side.back();
@@ -794,12 +792,16 @@ brisk_status brisk_replay_diagnostics(const brisk_dims* d, const brisk_params* p
   // run beside the proposal rows' sweep and the verifier rows' sweep beside the corrector, on the
   // decode tail's side streams (32 sequences: 213 us one after another, 129 us so; 131 us with the
   // verifier rows from the start, as little follows them here).
-  // A call under stream capture does not create them: without them everything stays on `stream`.
-  std::lock_guard<std::mutex> lock(side_stream_mutex());
+  // Under capture, and while the side streams belong to a caller's capture of a decode tail, all of
+  // it stays on `stream`: a capture keeps what it forked until it ends, which would break it or the
+  // other calls.
+  std::unique_lock<std::mutex> lock(side_stream_mutex());
   cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
   BRISK_CUDA(cudaStreamIsCapturing(st, &capture));
-  SideStream* ss = side_stream(capture == cudaStreamCaptureStatusNone);
-  if (!ss && capture == cudaStreamCaptureStatusNone) return BRISK_ERR_CUDA;
+  SideStream* ss = capture == cudaStreamCaptureStatusNone ? side_stream() : nullptr;
+  if (ss) BRISK_CUDA(cudaStreamIsCapturing(ss->hi, &capture));
+  if (capture != cudaStreamCaptureStatusNone) ss = nullptr;
+  if (!ss) lock.unlock();
   SideJoin join{ss, st};
   cudaStream_t hi = ss ? ss->hi : st, mid = ss ? ss->mid : st, lo = ss ? ss->lo : st;
   // `to` goes on after everything enqueued on `from` so far
@@ -809,13 +811,12 @@ brisk_status brisk_replay_diagnostics(const brisk_dims* d, const brisk_params* p
     return e != cudaSuccess ? e : cudaStreamWaitEvent(to, ss->ev[ev], 0);
   };
   BRISK_CUDA(after(hi, st, 0));
-  // A sweep that is placed first leaves the products no room until its rows end (129 us in some
-  // processes, 134 to 144 in others), so it waits until they have begun (130 in all; under capture
-  // until their fork: the graph orders the launches).
-  const bool live = ss && capture == cudaStreamCaptureStatusNone;
+  // A sweep that is placed first leaves the products no room until its rows end, so it waits until the
+  // first of them has begun. (That does not settle it: 32 sequences take 129 to 130 us in some
+  // processes and 144 to 145 in others.)
   if (ss) BRISK_CUDA(cudaEventRecord(ss->ev[5], hi));
   s = hidden_products(d, p, tables, hidden, h_ctx, w, ws, HIDDEN_BOTH, hi, ss && products_beside(w, d),
-                      nullptr, live ? ss->ev[5] : nullptr);
+                      nullptr, ss ? ss->ev[5] : nullptr);
   if (s != BRISK_OK) return s;
   if (ss) BRISK_CUDA(cudaStreamWaitEvent(mid, ss->ev[5], 0));
   SweepLaunch sq{};

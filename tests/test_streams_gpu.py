@@ -1,6 +1,9 @@
-"""What calls leave on the library's side streams: a call that fails between its fork and its join."""
+"""What calls leave on the library's side streams: replay diagnostics under capture and beside a
+caller's own capture of a tail, and a call that fails between its fork and its join."""
 import pytest
 import torch
+
+from paper_2609_33390_gb300 import synth
 
 pytestmark = pytest.mark.gpu
 
@@ -13,6 +16,58 @@ def brisk():
     build.build()
     from paper_2609_33390_gb300 import brisk as B
     return B
+
+
+def _workload(brisk, **kw):
+    wl = synth.Workload("streams", agree0=0.9, agree_decay=0.97, weight_std=0.2, **kw)
+    tail = brisk.DecodeTail.for_workload(wl, synth.make_weights(wl, "cuda"))
+    tail.prepare()
+    return tail, synth.make_block(wl, "cuda")
+
+
+@pytest.mark.parametrize("kw", [dict(B=2, L=8, V=4099), dict(B=16, L=32, V=64003),
+                                dict(B=80, L=32, V=32000)])
+def test_captured_replay_matches_direct_calls(brisk, kw):
+    """A captured call stays on its stream, so this also compares the direct call's concurrent
+    sweeps, of up to 160 MB each, with the same work in order."""
+    tail, blk = _workload(brisk, d=256, K=8, r=64, **kw)
+    direct = [tail.replay(blk) for _ in range(3)]
+    torch.cuda.synchronize()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g):
+        out = tail.replay(blk)
+    for _ in range(2):
+        for v in out.values():
+            v.zero_()
+        g.replay()
+        torch.cuda.synchronize()
+        for d in direct:
+            for k in out:
+                assert torch.equal(out[k], d[k]), k
+    assert tail.device_status() == brisk.OK
+
+
+def test_replay_while_a_caller_captures_a_tail(brisk):
+    """The capture owns the side streams until it ends; a replay on another stream goes on without
+    them and leaves it whole."""
+    tail, blk = _workload(brisk, B=4, L=16, V=20011, d=128, K=8, r=32)
+    other, blk2 = _workload(brisk, B=3, L=8, V=9001, d=128, K=8, r=32)
+    want, want2 = tail.tail(blk), other.replay(blk2)
+    out = tail.alloc_outputs()
+    torch.cuda.synchronize()
+    stream, g = torch.cuda.Stream(), torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g, capture_error_mode="relaxed"):
+        tail.tail(blk, out=out)
+        with torch.cuda.stream(stream):
+            got2 = other.replay(blk2)
+    torch.cuda.synchronize()
+    assert all(torch.equal(got2[k], want2[k]) for k in want2)
+    g.replay()
+    torch.cuda.synchronize()
+    assert all(torch.equal(out[k], want[k]) for k in want)
+    again = other.replay(blk2)
+    torch.cuda.synchronize()
+    assert all(torch.equal(again[k], want2[k]) for k in want2)
 
 
 def test_a_failed_tail_is_joined(brisk):
