@@ -435,7 +435,7 @@ struct ScanArgs {
   int32_t* base_rank;    // [B, L] (base_prefix only)
   int beside_sweep;      // the corrector runs beside the verifier-row sweep
   // set by the launch (see corrector_kernel)
-  int ring_depth, tok_ranks, ask_rows, ask_tokens;
+  int ring_depth, tok_ranks, ask_rows;
   int parts;             // CTAs that share a verification's residual walk
   long long wait_limit;
   // select outputs (or verify inputs when do_select == 0)

@@ -565,8 +565,8 @@ __device__ __forceinline__ float sigmoid_hw(float x) { return rcp_hw(1.f + ex2(-
 // it is the number of instructions on the dependent chain of a position (a lone warp issues one
 // about every 8 cycles), and beside it the ones that every warp repeats; so few warps compute and
 // the rest of the work is done by others or beforehand (32 positions, S = 512, K = 8: one sequence
-// 41 us with eight computing warps that load for themselves, now 27; 16 sampled ones 63, now 41). A sequence has ceil(S / 128) computing warps that own four state elements a lane.
-// A position is:
+// 41 us with eight computing warps that load for themselves, now 27; 16 sampled ones 63, now 41). A
+// sequence has ceil(S / 128) computing warps that own four state elements a lane. A position is:
 //  - the minimal-GRU step on the lane's elements, its residual-dot and gate partials (packed
 //    fp32 pairs), a warp reduce-scatter, the warps' parts to shared memory, one barrier;
 //  - gate, refined scores and Select, in every warp alike: lane k adds the parts of candidate k.
@@ -574,11 +574,13 @@ __device__ __forceinline__ float sigmoid_hw(float x) { return rcp_hw(1.f + ex2(-
 // forward) and, with ROWS, the residual rows into a ring of `depth` positions by bulk copies, a
 // row a lane; a rank past R reads its token row through L2, and without ROWS the computing warps
 // load the residual rows themselves. One more warp asks rows into L2 some positions ahead (where
-// the ring is shallow) and stores the outputs. The features of every (position, rank fed
-// forward) pair are tabulated first; the shares of a position that do not depend on the
-// selection are summed before the barrier of the position before. (One CTA an SM is asked of the
-// compiler: left to itself it settles on 80 to 103 registers, some spilled on the chain, and one
-// sequence's graph replay takes 61 us, not 51.)
+// the ring is shallow) and stores the outputs. A warp issues a copy or an ask in some 50 cycles,
+// which bounds positions with many candidates, so it asks for no token rows past the first R (with all K of
+// them 128 sequences of K = 32, S = 512 took 173 us, now 115; K = 16, S = 1024 123, now 113). The
+// features of every (position, rank fed forward) pair are tabulated first; the shares of a position
+// that do not depend on the selection are summed before the barrier of the position before. (One CTA
+// an SM is asked of the compiler: left to itself it settles on 80 to 103 registers, some spilled on
+// the chain, and one sequence's graph replay takes 61 us, not 51.)
 template <int NP, bool ROWS, bool SAMPLE, bool VERIFY>
 __global__ void __launch_bounds__(32 * CORR_PART + CORR_OTHERS, 1)
 corrector_kernel(const __grid_constant__ ScanArgs a) {
@@ -831,7 +833,7 @@ corrector_kernel(const __grid_constant__ ScanArgs a) {
       if (lane == 0) prefetch_l2(a.G + (bL + p) * 2 * S, S * 8, keep);
       if (lane >= K) return;
       prefetch_l2(a.U + (size_t)sm.cid[p * K + lane] * S, S * 4, keep);
-      if ((a.ask_tokens || lane < R) && p + 1 < L)
+      if (lane < R && p + 1 < L)
         prefetch_l2(a.Tzh + (size_t)sm.cid[p * K + lane] * 2 * S, S * 8, keep);
     };
     for (int p = 0; p < CORR_AHEAD; ++p) ask(p);
@@ -927,7 +929,6 @@ cudaError_t launch_corrector(const ScanArgs& args, cudaStream_t stream) {
     if (bytes(s.depth, s.ranks, s.rows) <= room) break;
   }
   a.ask_rows = a.ring_depth < 4;
-  a.ask_tokens = !a.beside_sweep;
   if (a.K <= 8)
     return rows ? launch_corrector_m<8, true>(a, stream) : launch_corrector_m<8, false>(a, stream);
   if (a.K <= 16)
