@@ -575,13 +575,15 @@ __device__ __forceinline__ float sigmoid_hw(float x) { return rcp_hw(1.f + ex2(-
 // row a lane; a rank past R reads its token row through L2, and without ROWS the computing warps
 // load the residual rows themselves. One more warp asks rows into L2 some positions ahead (where
 // the ring is shallow) and stores the outputs. A warp issues a copy or an ask in some 50 cycles,
-// which bounds positions with many candidates, so it asks for no token rows past the first R (with all K of
-// them 128 sequences of K = 32, S = 512 took 173 us, now 115; K = 16, S = 1024 123, now 113). The
+// which bounds positions with many candidates, so it asks for no token rows past the first R (with
+// all K of them 128 sequences of K = 32, S = 512 took 173 us, now 115; K = 16, S = 1024 123, now 113). The
 // features of every (position, rank fed forward) pair are tabulated first; the shares of a position
 // that do not depend on the selection are summed before the barrier of the position before. (One CTA
 // an SM is asked of the compiler: left to itself it settles on 80 to 103 registers, some spilled on
 // the chain, and one sequence's graph replay takes 61 us, not 51.)
-template <int NP, bool ROWS, bool SAMPLE, bool VERIFY>
+// LONE does not change the code: it makes a separate kernel whose shared-memory carveout preference
+// leaves a call without a sweep beside it all that an SM has.
+template <int NP, bool ROWS, bool SAMPLE, bool VERIFY, bool LONE>
 __global__ void __launch_bounds__(32 * CORR_PART + CORR_OTHERS, 1)
 corrector_kernel(const __grid_constant__ ScanArgs a) {
   extern __shared__ __align__(16) char smem_raw[];
@@ -882,13 +884,14 @@ namespace {
 // 210 KB on half as many SMs, which no sweep CTA shares.
 constexpr size_t CORR_SMEM = 220 * 1024;
 constexpr size_t CORR_SMEM_BESIDE = 76 * 1024;
+constexpr int CORR_SMS = 152;
 
-template <int NP, bool ROWS, bool SAMPLE, bool VERIFY>
+template <int NP, bool ROWS, bool SAMPLE, bool VERIFY, bool LONE>
 cudaError_t launch_corrector_k(const ScanArgs& a, cudaStream_t stream) {
   const size_t smem = corr_layout(a.L, a.K, a.S, a.V, a.ring_depth,
                                   corr_stage(a.K, a.S, a.tok_ranks, ROWS), VERIFY, nullptr, nullptr);
-  auto kernel = corrector_kernel<NP, ROWS, SAMPLE, VERIFY>;
-  cudaError_t e = set_up_kernel(kernel, CARVEOUT_SMALL_KB, smem);
+  auto kernel = corrector_kernel<NP, ROWS, SAMPLE, VERIFY, LONE>;
+  cudaError_t e = set_up_kernel(kernel, LONE ? CARVEOUT_FULL_KB : CARVEOUT_SMALL_KB, smem);
   if (e != cudaSuccess) return e;
   const int threads = 32 * ((a.S + CORR_SPAN - 1) / CORR_SPAN) + CORR_OTHERS;
   e = launch_prio(kernel, dim3(a.B), dim3(threads), smem, stream, a);
@@ -896,13 +899,19 @@ cudaError_t launch_corrector_k(const ScanArgs& a, cudaStream_t stream) {
   return cudaGetLastError();
 }
 
-template <int NP, bool ROWS>
+template <int NP, bool ROWS, bool SAMPLE>
 cudaError_t launch_corrector_m(const ScanArgs& a, cudaStream_t stream) {
+  if (a.do_verify) return launch_corrector_k<NP, ROWS, SAMPLE, true, true>(a, stream);
+  return a.beside_sweep ? launch_corrector_k<NP, ROWS, SAMPLE, false, false>(a, stream)
+                        : launch_corrector_k<NP, ROWS, SAMPLE, false, true>(a, stream);
+}
+template <int NP>
+cudaError_t launch_corrector_n(const ScanArgs& a, bool rows, cudaStream_t stream) {
   if (a.select_mode == BRISK_SELECT_SAMPLE)
-    return a.do_verify ? launch_corrector_k<NP, ROWS, true, true>(a, stream)
-                       : launch_corrector_k<NP, ROWS, true, false>(a, stream);
-  return a.do_verify ? launch_corrector_k<NP, ROWS, false, true>(a, stream)
-                     : launch_corrector_k<NP, ROWS, false, false>(a, stream);
+    return rows ? launch_corrector_m<NP, true, true>(a, stream)
+                : launch_corrector_m<NP, false, true>(a, stream);
+  return rows ? launch_corrector_m<NP, true, false>(a, stream)
+              : launch_corrector_m<NP, false, false>(a, stream);
 }
 
 cudaError_t launch_corrector(const ScanArgs& args, cudaStream_t stream) {
@@ -913,9 +922,18 @@ cudaError_t launch_corrector(const ScanArgs& args, cudaStream_t stream) {
                        a.do_verify != 0, nullptr, nullptr);
   };
   // Beside the verifier-row sweep a CTA stays within the sweep's carveout, with room for sweep CTAs
-  // on its SM, where it can.
-  const size_t room = a.beside_sweep && bytes(2, 1, true) <= CORR_SMEM_BESIDE ? CORR_SMEM_BESIDE
-                                                                              : CORR_SMEM;
+  // on its SM, where it can. Alone, more sequences than SMs share them (a state of up to 128, 256, 512
+  // leaves registers for four, three, two) as far as the smallest ring with residual rows allows:
+  // 608 sequences of 32 positions, K = 8: S = 128 97 us with the deepest ring, 74 so; S = 512 228,
+  // 170; K = 32, S = 128 274, 170. (Rows left out of the ring for one more CTA an SM: 134 us there
+  // with 4000 ids, but 407 instead of 358 with S = 512 and 60000 ids.)
+  size_t room = a.beside_sweep && bytes(2, 1, true) <= CORR_SMEM_BESIDE ? CORR_SMEM_BESIDE : CORR_SMEM;
+  if (!a.beside_sweep) {
+    int n = a.S <= 128 ? 4 : (a.S <= 256 ? 3 : (a.S <= 512 ? 2 : 1));
+    if (n > (a.B + CORR_SMS - 1) / CORR_SMS) n = (a.B + CORR_SMS - 1) / CORR_SMS;
+    while (n > 1 && bytes(2, 1, true) > CORR_SMEM / n - 1024) --n;
+    if (n > 1) room = CORR_SMEM / n - 1024;
+  }
   // the ring's depth, the token rows a stage holds, and whether it holds the residual rows: the
   // first of these that fits
   struct Shape { int depth, ranks; bool rows; };
@@ -929,11 +947,9 @@ cudaError_t launch_corrector(const ScanArgs& args, cudaStream_t stream) {
     if (bytes(s.depth, s.ranks, s.rows) <= room) break;
   }
   a.ask_rows = a.ring_depth < 4;
-  if (a.K <= 8)
-    return rows ? launch_corrector_m<8, true>(a, stream) : launch_corrector_m<8, false>(a, stream);
-  if (a.K <= 16)
-    return rows ? launch_corrector_m<16, true>(a, stream) : launch_corrector_m<16, false>(a, stream);
-  return rows ? launch_corrector_m<32, true>(a, stream) : launch_corrector_m<32, false>(a, stream);
+  if (a.K <= 8) return launch_corrector_n<8>(a, rows, stream);
+  if (a.K <= 16) return launch_corrector_n<16>(a, rows, stream);
+  return launch_corrector_n<32>(a, rows, stream);
 }
 
 }  // namespace

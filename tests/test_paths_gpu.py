@@ -127,3 +127,14 @@ def test_split_products_parity(brisk, dtype, B, L, d, r):  # noqa: F811
     assert rep.max_ref_err <= 1e-3
     for k in g:
         np.testing.assert_array_equal(g[k], g2[k], err_msg=k)
+
+
+@pytest.mark.parametrize("B,K,r", [(153, 8, 256), (305, 32, 128), (457, 16, 16), (609, 8, 64)])
+def test_more_sequences_than_sms_parity(brisk, B, K, r):  # noqa: F811
+    """A lone corrector of two, three and four sequences an SM, and of a wave more: the same bits as
+    beside a sweep, and the oracle's results."""
+    wl = synth.Workload("sequences", B=B, L=5, V=900, d=64, K=K, r=r, agree0=0.9, weight_std=0.1)
+    weights = _to(synth.make_weights(wl, "cpu"), "cuda")
+    block = _to(synth.make_block(wl, "cpu"), "cuda")
+    rep, _ = _run_and_check(brisk, wl, weights, block, seqs=[0, B - 1])
+    assert rep.max_ref_err <= 1e-3
