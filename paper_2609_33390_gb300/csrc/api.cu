@@ -215,14 +215,16 @@ brisk_status hidden_products(const brisk_dims* d, const brisk_params* p, const v
   float* Hc = Hm + (size_t)BL * r;
   cudaStream_t cs = ctx_st ? ctx_st : st;   // the context's two products wait for no other
   if (part & HIDDEN_FIRST) {
-    BRISK_CUDA(gemm_simt(BL, r, d->d, hidden, hd, d->d, p->P_h, hd, d->d, false, Hm, r, st));
-    BRISK_CUDA(gemm_simt(d->B, r, d->d, h_ctx, hd, d->d, p->P_h, hd, d->d, false, Hc, r, cs));
+    BRISK_CUDA(gemm_simt(BL, r, d->d, hidden, hd, d->d, p->P_h, hd, d->d, false, Hm, r, st, nullptr, 1,
+                         BL));
+    BRISK_CUDA(gemm_simt(d->B, r, d->d, h_ctx, hd, d->d, p->P_h, hd, d->d, false, Hc, r, cs, nullptr, 1,
+                         BL));
   }
   if (part & HIDDEN_SECOND) {
     BRISK_CUDA(gemm_simt(BL, 2 * S, r, Hm, BRISK_DT_F32, r, at<float>(tables, t.W2), BRISK_DT_F32,
-                         r, false, at<float>(ws, w.G), 2 * S, st, at<float>(tables, t.posG), d->L));
+                         r, false, at<float>(ws, w.G), 2 * S, st, at<float>(tables, t.posG), d->L, BL));
     BRISK_CUDA(gemm_simt(d->B, S, r, Hc, BRISK_DT_F32, r, at<float>(tables, t.W0h), BRISK_DT_F32, r,
-                         false, at<float>(ws, w.G0), S, cs));
+                         false, at<float>(ws, w.G0), S, cs, nullptr, 1, BL));
   }
   return BRISK_OK;
 }

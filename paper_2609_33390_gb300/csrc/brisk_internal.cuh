@@ -373,10 +373,11 @@ cudaError_t launch_sweep(const SweepLaunch& a, cudaStream_t stream);
 
 // ---------------------------------------------------------------- dense products (SIMT, fp32 accumulate)
 // C[m, n] = sum_k A(m, k) B(n, k) (+ bias[m % bias_period][n]), A(m,k) = A[m*lda + k],
-// B(n,k) = transB ? B[k*ldb + n] : B[n*ldb + k].
+// B(n,k) = transB ? B[k*ldb + n] : B[n*ldb + k]. call_rows: the most rows of a product of the call.
 cudaError_t gemm_simt(int M, int N, int K, const void* A, int a_dt, int lda, const void* B,
                       int b_dt, int ldb, bool transB, float* C, int ldc, cudaStream_t stream,
-                      const float* bias = nullptr, int bias_period = 1);
+                      const float* bias = nullptr, int bias_period = 1,
+                      int call_rows = 0x7fffffff);
 // Tensor-core product on sm_103a: C = A B^T with A [M, K] and B [N, K] bf16 (row strides lda, ldb),
 // fp32 accumulation; mode 0 stores fp32 C[m*ldc + n], mode 1 stores three bf16 parts whose sum
 // is c to about 2^-24 relative (hi at [m*ldc + n], mid at [m*ldc + N + n], lo at [m*ldc + 2N + n]).

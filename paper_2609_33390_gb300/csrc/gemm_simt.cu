@@ -1,6 +1,6 @@
-// Tiled fp32 dense products and the folds of the corrector's own weights. They serve the fp32 configurations (the
-// hidden products of a call and the one-off folds of the frozen vocabulary rows, App. C.3) and
-// the token folds' fallback; every product accumulates in fp32.
+// Tiled fp32 dense products, products of few rows, and the folds of the corrector's own weights. They
+// serve the fp32 configurations (the hidden products of a call and the one-off folds of the frozen
+// vocabulary rows, App. C.3) and the token folds' fallback; every product accumulates in fp32.
 #include "brisk_internal.cuh"
 
 namespace brisk {
@@ -189,6 +189,57 @@ gemm_simt_kernel(const __grid_constant__ SimtProblem P) {
   cluster_sync();   // the other CTAs have read this one's part
 }
 
+// Products of few rows: a warp an output column, whose lanes take four k each of every 128 for every
+// row, then a warp sum a row. A tile has nothing to share among so few rows, and its barriers and the
+// cluster's cost more than they are worth: a lone corrector of eight positions (d = 96, r = 112) 47 us
+// with its products on tiles, 34 so. Up to a k of 128; a longer one only where every product of the
+// call has few rows (one sequence of two positions, d = 512, r = 112: 43 us, 26; d = 4096, r = 256: 89,
+// 35): with longer products of other rows beside it, a tail's is no faster for it (8 rows, d = 512: 30.9
+// us with the context's product of k = 512 on tiles, 34.8 without).
+constexpr int FEW_WARPS = 8;
+constexpr int FEW_ROWS = 4;             // rows of a call up to which every k is taken so
+constexpr int FEW_ROWS_SHORT = 8;       // rows of a product up to which a k of FEW_SHORT_K is (16 in a
+constexpr int FEW_SHORT_K = 128;        // tail, k = 128: 38 us, 40)
+
+// UNROLL: four k a lane of the column and of every row that are on their way at once.
+template <typename TA, typename TB, int ROWS, int UNROLL>
+__global__ void __launch_bounds__(FEW_WARPS * 32)
+gemm_few_kernel(const __grid_constant__ SimtProblem P) {
+  const int lane = threadIdx.x & 31;
+  const long long n = (long long)blockIdx.x * FEW_WARPS + (threadIdx.x >> 5);
+  if (n >= P.N) return;
+  const TA* A = static_cast<const TA*>(P.A);
+  const TB* b = static_cast<const TB*>(P.B) + n * P.ldb;
+  float2 acc[ROWS];
+#pragma unroll
+  for (int m = 0; m < ROWS; ++m) acc[m] = make_float2(0.f, 0.f);
+  for (int k0 = 4 * lane; k0 < P.K; k0 += 128 * UNROLL) {
+    float4 y[UNROLL], x[UNROLL][ROWS];
+#pragma unroll
+    for (int u = 0; u < UNROLL; ++u) {
+      y[u] = row4(b, k0 + 128 * u, P.K, P.vecB);
+#pragma unroll
+      for (int m = 0; m < ROWS; ++m)
+        if (m < P.M) x[u][m] = row4(A + (long long)m * P.lda, k0 + 128 * u, P.K, P.vecA);
+    }
+#pragma unroll
+    for (int u = 0; u < UNROLL; ++u)
+#pragma unroll
+      for (int m = 0; m < ROWS; ++m)
+        if (m < P.M) {
+          acc[m] = __ffma2_rn(make_float2(x[u][m].x, x[u][m].y), make_float2(y[u].x, y[u].y), acc[m]);
+          acc[m] = __ffma2_rn(make_float2(x[u][m].z, x[u][m].w), make_float2(y[u].z, y[u].w), acc[m]);
+        }
+  }
+#pragma unroll
+  for (int m = 0; m < ROWS; ++m) {
+    if (m >= P.M) break;
+    const float v = warp_sum(acc[m].x + acc[m].y);
+    if (lane == 0)
+      P.C[(long long)m * P.ldc + n] = v + (P.bias ? P.bias[(long long)(m % P.bias_period) * P.N + n] : 0.f);
+  }
+}
+
 // One thread an item: the weight blocks' element (j, t) in every form the products read, then the
 // position shares, the feature shares and the gate weights (each a sum of 16 products in order).
 // Bound by launches when done block by block: 29 launches took about 100 us.
@@ -251,7 +302,7 @@ __global__ void __launch_bounds__(256) pack_kernel(const __grid_constant__ PackA
 template <typename TA, typename TB>
 cudaError_t gemm_t(int M, int N, int K, const void* A, int lda, const void* B, int ldb,
                    bool transB, float* C, int ldc, cudaStream_t stream, const float* bias,
-                   int bias_period) {
+                   int bias_period, bool few) {
   const int ntiles = (N + TN - 1) / TN, slices = (K + TK - 1) / TK;
   const long long tiles = (long long)((M + TM - 1) / TM) * ntiles;
   int split = 1;
@@ -263,6 +314,13 @@ cudaError_t gemm_t(int M, int N, int K, const void* A, int lda, const void* B, i
   };
   const SimtProblem P{M, N, K, A, lda, B, ldb, transB ? 1 : 0, C, ldc, ntiles, split,
                       vec(A, sizeof(TA), lda), vec(B, sizeof(TB), ldb), bias, bias_period};
+  if (!transB && M <= FEW_ROWS_SHORT && (few || K <= FEW_SHORT_K)) {
+    auto kernel = M <= FEW_ROWS ? gemm_few_kernel<TA, TB, FEW_ROWS, 4>
+                                : gemm_few_kernel<TA, TB, FEW_ROWS_SHORT, 1>;
+    const cudaError_t e = launch_prio(kernel, dim3((unsigned)((N + FEW_WARPS - 1) / FEW_WARPS)),
+                                      dim3(FEW_WARPS * 32), 0, stream, P);
+    return e != cudaSuccess ? e : cudaGetLastError();
+  }
   const cudaError_t e = launch_cluster(gemm_simt_kernel<TA, TB>, dim3((unsigned)(tiles * split)),
                                        dim3(SIMT_THREADS), 0, stream, split, P);
   return e != cudaSuccess ? e : cudaGetLastError();
@@ -272,19 +330,19 @@ cudaError_t gemm_t(int M, int N, int K, const void* A, int lda, const void* B, i
 
 cudaError_t gemm_simt(int M, int N, int K, const void* A, int a_dt, int lda, const void* B,
                       int b_dt, int ldb, bool transB, float* C, int ldc, cudaStream_t stream,
-                      const float* bias, int bias_period) {
+                      const float* bias, int bias_period, int call_rows) {
   if (M <= 0 || N <= 0) return cudaSuccess;
+  const bool few = call_rows <= FEW_ROWS;
   if (a_dt == BRISK_DT_BF16 && b_dt == BRISK_DT_BF16)
     return gemm_t<__nv_bfloat16, __nv_bfloat16>(M, N, K, A, lda, B, ldb, transB, C, ldc, stream,
-                                                bias, bias_period);
+                                                bias, bias_period, few);
   if (a_dt == BRISK_DT_F32 && b_dt == BRISK_DT_BF16)
-    return gemm_t<float, __nv_bfloat16>(M, N, K, A, lda, B, ldb, transB, C, ldc, stream,
-                                                bias, bias_period);
+    return gemm_t<float, __nv_bfloat16>(M, N, K, A, lda, B, ldb, transB, C, ldc, stream, bias,
+                                        bias_period, few);
   if (a_dt == BRISK_DT_BF16 && b_dt == BRISK_DT_F32)
-    return gemm_t<__nv_bfloat16, float>(M, N, K, A, lda, B, ldb, transB, C, ldc, stream,
-                                                bias, bias_period);
-  return gemm_t<float, float>(M, N, K, A, lda, B, ldb, transB, C, ldc, stream,
-                                                bias, bias_period);
+    return gemm_t<__nv_bfloat16, float>(M, N, K, A, lda, B, ldb, transB, C, ldc, stream, bias,
+                                        bias_period, few);
+  return gemm_t<float, float>(M, N, K, A, lda, B, ldb, transB, C, ldc, stream, bias, bias_period, few);
 }
 
 cudaError_t pack_weights(const PackArgs& a, cudaStream_t stream) {

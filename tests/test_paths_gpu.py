@@ -129,6 +129,19 @@ def test_split_products_parity(brisk, dtype, B, L, d, r):  # noqa: F811
         np.testing.assert_array_equal(g[k], g2[k], err_msg=k)
 
 
+@pytest.mark.parametrize("B,L,d,r", [(1, 1, 8, 16), (1, 4, 1000, 512), (4, 1, 2000, 80), (1, 5, 96, 128),
+                                     (8, 1, 128, 16), (1, 8, 136, 144), (9, 1, 40, 32)])
+def test_few_row_products_parity(brisk, B, L, d, r):  # noqa: F811
+    """fp32 products of 1 to 4 rows, of 5 to 8 rows up to a k of 128, and just past either. Against
+    the oracle."""
+    wl = synth.Workload("few", B=B, L=L, V=400, d=d, K=8, r=r, hidden_dtype=F32, agree0=0.9,
+                        weight_std=0.05)
+    weights = _to(synth.make_weights(wl, "cpu"), "cuda")
+    block = _to(synth.make_block(wl, "cpu"), "cuda")
+    rep, _ = _run_and_check(brisk, wl, weights, block)
+    assert rep.max_ref_err <= 1e-3
+
+
 @pytest.mark.parametrize("B,K,r", [(153, 8, 256), (305, 32, 128), (457, 16, 16), (609, 8, 64)])
 def test_more_sequences_than_sms_parity(brisk, B, K, r):  # noqa: F811
     """A lone corrector of two, three and four sequences an SM, and of a wave more: the same bits as
