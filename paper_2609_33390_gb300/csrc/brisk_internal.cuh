@@ -16,7 +16,6 @@ namespace brisk {
 
 constexpr unsigned FULL_MASK = 0xffffffffu;
 constexpr float LOG2E = 1.4426950408889634f;   // log2(e): exp(x) = 2^(x log2 e)
-constexpr float LN2 = 0.6931471805599453f;
 constexpr int INVALID_ID = 0x7fffffff;
 constexpr float RESID_Z_FLOOR = 1e-6f;         // residual mass below which the verifier argmax is used
 
@@ -62,67 +61,6 @@ __device__ __forceinline__ float ex2(float x) {
 // Candidate order of the method: logit descending, then id ascending.
 __device__ __forceinline__ bool better(float v1, int i1, float v2, int i2) {
   return v1 > v2 || (v1 == v2 && i1 < i2);
-}
-
-// Insert (v, id) into a list sorted best-first; the worst entry falls off.
-template <int KP>
-__device__ __forceinline__ void list_insert(float v, int id, float (&vals)[KP], int (&ids)[KP]) {
-#pragma unroll
-  for (int j = 0; j < KP; ++j) {
-    const bool sw = better(v, id, vals[j], ids[j]);
-    const float tv = vals[j];
-    const int ti = ids[j];
-    vals[j] = sw ? v : tv;
-    ids[j] = sw ? id : ti;
-    v = sw ? tv : v;
-    id = sw ? ti : id;
-  }
-}
-
-template <int KP>
-__device__ __forceinline__ void list_clear(float (&vals)[KP], int (&ids)[KP]) {
-#pragma unroll
-  for (int j = 0; j < KP; ++j) {
-    vals[j] = -INFINITY;
-    ids[j] = INVALID_ID;
-  }
-}
-
-// Warp-wide extraction of the best `kout` entries of 32 sorted lists. Lane r < kout ends
-// holding the r-th best in (out_v, out_i).
-template <int KP>
-__device__ __forceinline__ void warp_extract(float (&vals)[KP], int (&ids)[KP], int kout,
-                                             float& out_v, int& out_i) {
-  const int lane = threadIdx.x & 31;
-  out_v = -INFINITY;
-  out_i = INVALID_ID;
-  for (int r = 0; r < kout; ++r) {
-    float bv = vals[0];
-    int bi = ids[0];
-#pragma unroll
-    for (int off = 16; off; off >>= 1) {
-      const float ov = __shfl_xor_sync(FULL_MASK, bv, off);
-      const int oi = __shfl_xor_sync(FULL_MASK, bi, off);
-      if (better(ov, oi, bv, bi)) {
-        bv = ov;
-        bi = oi;
-      }
-    }
-    const bool win = (ids[0] == bi) && (vals[0] == bv);
-#pragma unroll
-    for (int j = 0; j < KP - 1; ++j) {
-      vals[j] = win ? vals[j + 1] : vals[j];
-      ids[j] = win ? ids[j + 1] : ids[j];
-    }
-    if (win) {
-      vals[KP - 1] = -INFINITY;
-      ids[KP - 1] = INVALID_ID;
-    }
-    if (lane == r) {
-      out_v = bv;
-      out_i = bi;
-    }
-  }
 }
 
 __device__ __forceinline__ float warp_sum(float x) {

@@ -165,7 +165,7 @@ struct TcProblem {
   int mode;         // 0: fp32 C[m*ldc + n]; 1: bf16 parts hi, mid, lo at [m*ldc + {0, N, 2N} + n]
   void* C;
   int ldc;
-  int mtiles, ntiles;
+  int ntiles;
   const float* bias;   // optional fp32 [bias_period, N], added to row m as bias[m % bias_period]
   int bias_period;
 };
@@ -200,9 +200,9 @@ constexpr int TC_SMS = 152;
 constexpr int TC_PART_PAD = 4;      // floats between the rows of a part in shared memory
 
 // SMALL_CARVEOUT does not change the code: it makes a separate kernel whose shared-memory
-// carveout preference (a per-kernel attribute) is the sweep's.
+// carveout preference (a per-kernel attribute) is the sweep's. At most 128 registers a thread: a CTA
+// fits beside three sweep CTAs.
 template <int TC_STAGES, bool SMALL_CARVEOUT = false>
-// At most 128 registers a thread: a CTA fits beside three sweep CTAs.
 __global__ void __launch_bounds__(TC_THREADS, 4)
 gemm_tc_kernel(const __grid_constant__ TcMaps maps, const __grid_constant__ TcArgs a) {
   extern __shared__ __align__(1024) uint8_t smem_raw[];
@@ -578,10 +578,10 @@ cudaError_t gemm_tc_grouped(const TcSpec* spec, int nprob, int32_t* status, cuda
     P.M = q.M; P.N = q.N; P.K = q.K; P.mode = q.mode; P.C = q.C; P.ldc = q.ldc;
     P.bias = q.bias;
     P.bias_period = q.bias_period > 0 ? q.bias_period : 1;
-    P.mtiles = (q.M + TC_BM - 1) / TC_BM;
     P.ntiles = (q.N + BN - 1) / BN;
-    if (i == 0) a.tiles0 = P.mtiles * P.ntiles;
-    total += P.mtiles * P.ntiles;
+    const int tiles = (q.M + TC_BM - 1) / TC_BM * P.ntiles;
+    if (i == 0) a.tiles0 = tiles;
+    total += tiles;
   }
   if (total == 0) return cudaSuccess;
   const size_t smem = gemm_tc_smem(BN, stages);

@@ -553,7 +553,8 @@ __device__ __forceinline__ float dot4(const float4& x, const float4& y) {
                               __fmul2_rn(make_float2(x.x, x.y), make_float2(y.x, y.y)));
   return p.x + p.y;
 }
-// Logistic function on the hardware exponential and reciprocal (relative error ~1e-7).
+// Logistic function on the hardware exponential and reciprocal (relative error about 1e-7 for small
+// |x|, 1e-6 at -20: that of the exponential's rounded argument).
 __device__ __forceinline__ float rcp_hw(float x) {
   float y;
   asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
