@@ -235,8 +235,10 @@ inline cudaError_t launch_prio(void (*kernel)(KArgs...), dim3 grid, dim3 block, 
   return launch_cluster(kernel, grid, block, smem, stream, 1, std::forward<Args>(args)...);
 }
 
-// Every thread of every CTA of the cluster arrives; writes before it are visible after it.
+// Every thread of every CTA of the cluster arrives; writes before it are visible after it. (The
+// barrier wants its warps whole, which a loop whose lanes leave it in turn does not promise.)
 __device__ __forceinline__ void cluster_sync() {
+  __syncwarp();
   asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" :::
                "memory");
 }

@@ -214,7 +214,6 @@ __device__ int residual_sample(const Smem& sm, const void* rowp, int dt, int V, 
     }
   }
   if (parts > 1) {
-    __syncwarp();
     cluster_sync();
     if (part) return -1;
   }
@@ -522,8 +521,10 @@ __device__ __forceinline__ void prefetch_l2(const float* p, unsigned bytes, uint
   asm volatile("cp.async.bulk.prefetch.L2.global.L2::cache_hint [%0], %1, %2;" ::"l"(p), "r"(bytes),
                "l"(policy));
 }
-// The block's barrier, for code that only some warps run.
+// The block's barrier, for code that only some warps run. (It wants its warps whole, which a wait
+// that lanes leave one by one does not promise.)
 __device__ __forceinline__ void block_sync(int threads) {
+  __syncwarp();
   asm volatile("bar.sync 0, %0;" ::"r"(threads) : "memory");
 }
 // Bounded wait for the phase of the given parity (more than `limit` SM cycles: false).
