@@ -584,7 +584,9 @@ __device__ __forceinline__ float sigmoid_hw(float x) { return rcp_hw(1.f + ex2(-
 // an SM is asked of the compiler: left to itself it settles on 80 to 103 registers, some spilled on
 // the chain, and one sequence's graph replay takes 61 us, not 51.)
 // LONE does not change the code: it makes a separate kernel whose shared-memory carveout preference
-// leaves a call without a sweep beside it all that an SM has.
+// gives a call without a sweep beside it all that an SM has. Not without ROWS: the residual rows'
+// loads then want L1 (K = 32, one sequence of 61 positions: S = 864 180 us with it, 163 without;
+// S = 1024 187, 169).
 template <int NP, bool ROWS, bool SAMPLE, bool VERIFY, bool LONE>
 __global__ void __launch_bounds__(32 * CORR_PART + CORR_OTHERS, 1)
 corrector_kernel(const __grid_constant__ ScanArgs a) {
@@ -903,9 +905,9 @@ cudaError_t launch_corrector_k(const ScanArgs& a, cudaStream_t stream) {
 
 template <int NP, bool ROWS, bool SAMPLE>
 cudaError_t launch_corrector_m(const ScanArgs& a, cudaStream_t stream) {
-  if (a.do_verify) return launch_corrector_k<NP, ROWS, SAMPLE, true, true>(a, stream);
+  if (a.do_verify) return launch_corrector_k<NP, ROWS, SAMPLE, true, ROWS>(a, stream);
   return a.beside_sweep ? launch_corrector_k<NP, ROWS, SAMPLE, false, false>(a, stream)
-                        : launch_corrector_k<NP, ROWS, SAMPLE, false, true>(a, stream);
+                        : launch_corrector_k<NP, ROWS, SAMPLE, false, ROWS>(a, stream);
 }
 template <int NP>
 cudaError_t launch_corrector_n(const ScanArgs& a, bool rows, cudaStream_t stream) {
