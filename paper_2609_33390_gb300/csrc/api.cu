@@ -35,12 +35,22 @@ enum TailSchedule { SCHEDULE_OVERLAP = 0, SCHEDULE_FUSED = 1 };
 // V = 126464 bf16, greedy (fused / both sweeps overlapping): one sequence (16 MB) 56 / 58 us, four
 // (65 MB) 67 / 70, sixteen (259 MB) 101 / 88.
 constexpr size_t FUSE_MAX_BYTES = size_t(64) << 20;
-constexpr size_t FUSE_MIN_VECTORS = 2048;  // 16-byte vectors a row below which it does not pay
+// 16-byte vectors a row from which the fused schedule is taken. Its verification walks a row with one
+// CTA, the overlapping one's with a cluster, so the better one depends on the verification too (fused /
+// overlapping, S = 256, greedy verification; stochastic): 8000 ids, one sequence 46 / 55; 52 / 57,
+// sixteen 59 / 62; 65 / 65; 32000 ids, one sequence 46 / 55; 60 / 59, sixteen 65 / 65; 85 / 69. The
+// line is not at a crossing: greedy verification gains from fusing at every size measured.
+constexpr size_t FUSE_MIN_VECTORS = 2048;
 // Rows below which fp32 products keep the verifier rows' sweep waiting: they run on the same units as
-// it and slow down beside two sweeps (16 sequences, d = 2048, S = 512: 115 us a tail, up to 126
-// with both from the start; 100 sequences: 355 with both from the start).
+// it and may slow down beside two sweeps. Which wins moves with both sizes (from the start / waiting,
+// 32 positions; d = 1024, S = 256: 32000 ids 32 sequences 83 / 89, 64 113 / 100, 100 146 / 133, 128
+// 165 / 175; 126464 ids 4 to 8 % for the start throughout; d = 2048, S = 512: 32000 ids 32 132 / 123,
+// 64 179 / 178; 126464 ids 16 114 / 108, 32 148 / 162, 48 206 / 203, 64 261 / 275, 100 387 / 392).
 constexpr size_t F32_ROWS = 2432;
-constexpr int BESIDE_STATE = 512;          // state width up to which the products share SMs with them
+// State width up to which the products share SMs with the sweeps (alone / sharing, 126464 ids, d = 2048,
+// 16, 64 and 128 sequences): S = 256 81 / 80, 194 / 184, 355 / 347; S = 512 90 / 84, 215 / 200, 383 /
+// 367; S = 640 95 / 95, 206 / 213, 401 / 389; S = 1024 95 / 109, 247 / 237, 426 / 442.
+constexpr int BESIDE_STATE = 512;
 
 struct WsLayout {
   size_t status, counters, part_val, part_id, part_m, part_s, argmax_p, lse_p;
@@ -134,7 +144,7 @@ TbLayout tb_layout(const brisk_dims* d) {
 
 // Whether the hidden products take the form that shares SMs with a sweep. Not in the fused
 // schedule (the sweep is as short as they are), nor for wide states, whose second product is four
-// times larger (64 sequences, S = 1024: 525 us a tail, 625 so).
+// times larger.
 inline bool products_beside(const WsLayout& w, const brisk_dims* d) {
   return w.schedule == SCHEDULE_OVERLAP && 2 * d->r <= BESIDE_STATE;
 }
